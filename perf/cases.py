@@ -168,7 +168,8 @@ def _make_mask(c, gen):
 
 
 # ------------------------------------------------------------------ one case
-def prepare(case, seed):
+def _inputs(case, seed):
+    """The block mask (one byte per block) and Q, K, V of one seed."""
     gen = torch.Generator(device="cuda")
     gen.manual_seed(seed)
     mask = _make_mask(case, gen)
@@ -179,7 +180,12 @@ def prepare(case, seed):
         shape = (H, n, d) if case["layout"] == "hnd" else (n, H, d)
         return torch.randn(shape, device="cuda", generator=gen, dtype=torch.float32).to(dt)
 
-    q, k, v = tokens(case["N"]), tokens(case["N_kv"]), tokens(case["N_kv"])
+    return mask, tokens(case["N"]), tokens(case["N_kv"]), tokens(case["N_kv"])
+
+
+def prepare(case, seed):
+    mask, q, k, v = _inputs(case, seed)
+    H, d = case["heads"], case["d"]
     kw = {"N_kv": case["N_kv"], "dtype": case["dtype"], "layout": case["layout"]}
     st = {"path": case["path"], "args": (case["B_Q"], case["B_KV"], case["N"], H, d), "kw": kw}
     stride = 0
@@ -242,3 +248,25 @@ def tolerance(case):
     # P and O are rounded to the element type once each, sums are fp32; measured against the same rows in 64-bit
     # arithmetic (2.3e-3 in bf16, 2.9e-4 in fp16 on every case), times four
     return {"rel": 1e-2} if case["dtype"] == "bf16" else {"rel": 1.2e-3}
+
+
+def exact(case, seed):
+    """O and LSE by dense masked softmax in 64 bits, a strip of query rows at a time."""
+    mask, q, k, v = _inputs(case, seed)
+    if case["layout"] == "nhd":
+        q, k, v = (t.transpose(0, 1) for t in (q, k, v))
+    H, N, N_kv, d = case["heads"], case["N"], case["N_kv"], case["d"]
+    O = torch.empty((H, N, d), dtype=torch.float64, device="cuda")
+    LSE = torch.empty((H, N), dtype=torch.float64, device="cuda")
+    key_block = torch.arange(N_kv, device="cuda") // case["B_KV"]
+    strip = max(case["B_Q"], (1 << 28) // N_kv // case["B_Q"] * case["B_Q"])  # 2 GB of scores
+    for h in range(H):
+        kt, vh = k[h].double().t() / math.sqrt(d), v[h].double()
+        for r in range(0, N, strip):
+            e = min(N, r + strip)
+            off = mask[h, r // case["B_Q"]:-(-e // case["B_Q"])] == 0
+            S = q[h, r:e].double() @ kt
+            S.masked_fill_(off[:, key_block].repeat_interleave(case["B_Q"], dim=0)[:e - r], -math.inf)
+            LSE[h, r:e] = torch.logsumexp(S, dim=1)
+            O[h, r:e] = S.sub_(LSE[h, r:e, None]).exp_() @ vh
+    return (O if case["layout"] == "hnd" else O.transpose(0, 1).contiguous()), LSE
