@@ -1327,13 +1327,30 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // item's tiles; the epilogue warpgroup waits for the item's last P V, drains the accumulator,
 // normalises and stores, and releases the accumulator for the next item's first P V, which cannot
 // be issued before that item's first softmax tile is done anyway.
-//   warps 0-3 / 4-7 : softmax warpgroups 0 / 1      warp 8 : K and Q TMA producer   warp 11 : V TMA producer
-//   warp 9 : Q K^T issuer      warp 10 : P V issuer    warps 12-15 : epilogue warpgroup
+//   warps 0-3 / 4-7 : softmax warpgroups 0 / 1      warp 8 : K TMA producer   warp 11 : V TMA producer
+//   warp 9 : Q K^T issuer      warp 10 : P V issuer    warps 12-15 : epilogue warpgroup (and Q tiles)
 // Registers (setmaxnreg): softmax 192, epilogue 80, producers and issuers 48 per thread; the sum over the CTA,
 // 256*192 + 128*80 + 128*48 = 65536, is exactly the launch allocation of 512 threads x 128.
-// TMEM columns: S0 0, S1 128, O 256, P0 384, P1 448.
+//
+// Q K^T takes Q, its A operand, from TMEM: a 128x128x16 MMA with both operands in shared memory reads the full
+// 128 B/clk for as long as it runs, so per 128-key tile (d = 128) 160 KB went through shared memory (Q and K 64, V 32,
+// the two TMA tiles 64); now 128 KB.  The epilogue warpgroup, idle for most of an item, moves the next item's Q tile
+// from the buffer it lands in to TMEM.  With all columns taken at d = 128 the two warpgroups share one P buffer: tile
+// j's P V has long read it when tile j+1 stores its P.  Together with the warp-uniform waits (mbar_wait_warp) measured
+// on one GPU, the two builds in turn: 16384 tokens, 8 heads, d = 128, (128,128) blocks 177.8 -> 173.2 us; 115200
+// tokens, 24 heads 14.56 -> 14.26 ms (global order); 32768 tokens, 16 heads, d = 64, (256,256) 1355 -> 1307 us.  These
+// launches run at the 1 kW power cap (1.3-1.9 GHz of 1.965), so less traffic shows as a higher clock.
+// TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448; d = 64: S0 0, S1 128, O 256, Q 320 and 352, P0 384, P1 448.
 // ==========================================================================================
 constexpr int kPpThreads = 512;
+
+// The whole warp waits for one barrier phase: one test and one vote when the phase has completed, the bounded wait
+// otherwise.  The result is the same in every lane.  (With the wait's loop and its early return in front of the vote the
+// common case crossed a divergent region: about 2 % of the softmax warpgroups' time.)
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
 
 // The k-th work item of CTA b out of G: rounds of G consecutive items, alternately dealt forwards and backwards.
 // Items arrive longest first, so dealing every round in the same direction would hand CTA 0 the longest item of
@@ -1387,9 +1404,20 @@ struct RingPos {
 };
 
 struct __align__(8) PpBarriers {
-    uint64_t q_full[2], q_empty[2], o_free, o_full, e_ready, e_taken;
+    uint64_t q_full, q_drained, qt_full[2], qt_free[2], o_free, o_full, e_ready, e_taken;
     uint64_t k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2];
+};
+
+// Tensor-memory columns of the ping-pong kernel.  Q is the A operand of Q K^T and lives in TMEM (D/2 columns).
+template <int D, int TK>
+struct PpCols {
+    static constexpr bool kTight = (D == 128 && TK == 128);  // all 512 columns in use
+    static constexpr uint32_t kP0 = kColP0, kP1 = kTight ? kColP0 : kColP1;
+    static constexpr bool kOneP = (kP0 == kP1);
+    static constexpr int kQBuffers = kTight ? 1 : 2;
+    static constexpr uint32_t kQ0 = kTight ? 448 : (D == 64 ? 320 : 64);
+    static constexpr uint32_t kQ1 = kTight ? 448 : (D == 64 ? 352 : 192);
 };
 
 template <int D, int TK, bool F16>
@@ -1400,10 +1428,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int Q_SUB = kTQ * 128;
     constexpr int KV_SUB = TK * 128;
     constexpr int KV_TILE = NSUB * KV_SUB;
+    using Cols = PpCols<D, TK>;
+    constexpr int NQT = Cols::kQBuffers;
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* sQ = smem;                      // two Q tiles: the next item's is loaded while this one's is in use
-    uint8_t* sK = sQ + 2 * NSUB * Q_SUB;     // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
+    uint8_t* sQ = smem;                      // landing buffer of the next item's Q tile, which then moves to TMEM
+    uint8_t* sK = sQ + NSUB * Q_SUB;         // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
     uint8_t* sV = sK + p.stages * KV_TILE;   // NSV V tiles (a V tile lives about two tiles longer, until its P V)
     __shared__ PpBarriers bars;
     // [publishing warpgroup][row]: the reference maximum after that warpgroup's latest tile.  One 32-bit word per
@@ -1429,9 +1459,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
     if (tid == 0) {
         abort_flag = 0;
+        mbar_init(smem_u32(&bars.q_full), 1);       // the Q tile has landed in shared memory
+        mbar_init(smem_u32(&bars.q_drained), 128);  // epilogue threads: it has been read from there
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&bars.q_full[b]), 1);
-            mbar_init(smem_u32(&bars.q_empty[b]), 1);
+            mbar_init(smem_u32(&bars.qt_full[b]), 128);  // epilogue threads: the Q tile is in TMEM
+            mbar_init(smem_u32(&bars.qt_free[b]), 1);    // the item's last Q K^T has completed
         }
         mbar_init(smem_u32(&bars.o_free), 128);   // epilogue threads: accumulator drained
         mbar_init(smem_u32(&bars.o_full), 1);     // P V issuer: the item's last P V has completed
@@ -1481,6 +1513,50 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         uint32_t itn = 0;  // non-empty items seen
         bool ok = true;
         BSA_TRACE_DECL(tn);
+        // ---- Q tiles: TMA into shared memory one item ahead, then into TMEM through this warpgroup's registers ----
+        int kq = 0;       // round of the next Q tile to load
+        uint32_t nq = 0;  // Q tiles loaded so far
+        auto load_q = [&]() {  // lane 0 of the warpgroup's first warp issues; every thread follows the item list
+            WorkItem w;
+            do {
+                if (kq >= n_rounds) return;
+                w = load_item(p.items, cta_item_index(kq++, blockIdx.x, gridDim.x), n_items);
+            } while (w.ntiles <= 0);
+            ++nq;
+            if (tw == 0) {
+                mbar_arrive_expect_tx(smem_u32(&bars.q_full), NSUB * Q_SUB);
+                tma_load_4d(smem_u32(sQ), &tmQ, smem_u32(&bars.q_full), 0, w.q_tile * kTQ, 0, w.head);
+            }
+        };
+        uint32_t sq = 0;  // Q tiles moved to TMEM
+        auto stage_q = [&]() -> bool {
+            const uint32_t b = (NQT == 2) ? (sq & 1) : 0, use = (NQT == 2) ? (sq >> 1) : sq;
+            bool good = mbar_wait(smem_u32(&bars.q_full), sq & 1, abortp);
+            good = good && mbar_wait(smem_u32(&bars.qt_free[b]), (use & 1) ^ 1, abortp);
+            if (!__all_sync(0xffffffffu, good)) return false;
+            tc_fence_after();
+            const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (b ? Cols::kQ1 : Cols::kQ0);
+#pragma unroll 1
+            for (int s = 0; s < NSUB; ++s) {  // 64 head-dimension columns: eight swizzled 16-byte chunks of this row
+                uint32_t v[32];
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(sQ + s * Q_SUB + tw * 128 + ((c ^ (tw & 7)) << 4));
+                    v[4 * c] = w.x; v[4 * c + 1] = w.y; v[4 * c + 2] = w.z; v[4 * c + 3] = w.w;
+                }
+                tmem_st32(t_q + s * 32, v);
+            }
+            mbar_arrive(smem_u32(&bars.q_drained));
+            tc_wait_st();
+            tc_fence_before();
+            mbar_arrive(smem_u32(&bars.qt_full[b]));
+            if (tw == 0) good = mbar_wait(smem_u32(&bars.q_drained), sq & 1, abortp);  // then the next Q tile may land
+            if (!__all_sync(0xffffffffu, good)) return false;
+            ++sq;
+            load_q();
+            return true;
+        };
+        load_q();
         WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
         for (int kr = 0; kr < n_rounds && ok; ++kr) {
             const WorkItem it = it_next;
@@ -1497,6 +1573,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 continue;
             }
+            // the next item's Q tile goes to TMEM first (its Q K^T runs ahead of this item's softmax); with one TMEM
+            // buffer that waits for this item's last Q K^T, which comes well before its last P V
+            while (ok && nq > sq && sq <= itn + 1) ok = stage_q();
+            if (!ok) break;
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
             if (!ok) break;
             const float l_tot = lfin[0][tw] + lfin[1][tw];
@@ -1551,70 +1631,31 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             }
             if (lane == 0) BSA_TRACE_POINT(11, tn, 34);
         }
+        if (!ok && tw == 0) {  // a Q tile in flight lands before the CTA's shared memory goes away
+            const uint64_t t0 = globaltimer_ns();
+            while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
+        }
     } else if (warp >= 8) {
         reg_dec<48>();
         if (warp == 8 && lane == 0) {
-            // =========================== K and Q producer ===========================
+            // =========================== K producer ===========================
             // K tiles run up to NSK tiles ahead of the Q K^T issuer and never wait for V slots (the V tiles have a
-            // thread of their own in warp 11).  Q tiles alternate between two buffers: an item's Q tile may be
-            // loaded once the last Q K^T of the item two before it has completed, so it is queued when this thread
-            // enters the item BEFORE it and issued as soon as that condition is implied by a K slot this thread has
-            // already waited for (Q K^T of tile g-NSK done) or is found true: this thread never blocks on a Q buffer
-            // while K slots are free, and a new item's first Q K^T does not wait for its Q tile.
-            uint32_t g = 0, itq = 0;  // itq: Q tiles issued (buffer itq & 1)
-            uint32_t seq = 0;          // non-empty items entered
-            RingPos ring;              // K ring position of tile g
+            // thread of their own in warp 11).
+            uint32_t g = 0;
+            RingPos ring;  // K ring position of tile g
             bool ok = true;
             BSA_TRACE_DECL(tn);
-            int pq_row0 = 0, pq_row1 = 0, pq_row2 = 0, pq_head0 = 0, pq_head1 = 0, pq_head2 = 0;
-            int pq_need0 = 0, pq_need1 = 0, pq_need2 = 0, npend = 0;
-            uint32_t queued = 0;             // Q tiles queued so far (= sequence number of the next item to queue)
-            int buf_last0 = -1000000, buf_last1 = -1000000;  // last global tile of the item that last used each buffer
-            auto issue_q = [&]() -> bool {  // loads the oldest pending Q tile
-                const uint32_t b = itq & 1;
-                if (!mbar_wait(smem_u32(&bars.q_empty[b]), ((itq >> 1) & 1) ^ 1, abortp)) return false;
-                mbar_arrive_expect_tx(smem_u32(&bars.q_full[b]), NSUB * Q_SUB);
-                tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, smem_u32(&bars.q_full[b]), 0, pq_row0, 0, pq_head0);
-                ++itq;
-                pq_row0 = pq_row1; pq_head0 = pq_head1; pq_need0 = pq_need1;
-                pq_row1 = pq_row2; pq_head1 = pq_head2; pq_need1 = pq_need2;
-                --npend;
-                return true;
-            };
-            // queue the Q tile of an item whose tiles are [first, first + n): it needs its buffer's previous user done
-            auto queue_q = [&](const WorkItem& w, int first, int n) -> bool {
-                while (npend >= 3)  // queue full (many short items ahead of the Q K^T issuer): wait for a buffer
-                    if (!issue_q()) return false;
-                const uint32_t b = queued & 1;
-                const int qrow = w.q_tile * kTQ, need = b ? buf_last1 : buf_last0;
-                if (npend == 0) { pq_row0 = qrow; pq_head0 = w.head; pq_need0 = need; }
-                else if (npend == 1) { pq_row1 = qrow; pq_head1 = w.head; pq_need1 = need; }
-                else { pq_row2 = qrow; pq_head2 = w.head; pq_need2 = need; }
-                ++npend;
-                if (b) buf_last1 = first + n - 1; else buf_last0 = first + n - 1;
-                ++queued;
-                return true;
-            };
             WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const WorkItem it = it_next;
                 it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
                 if (it.ntiles <= 0) continue;
-                if (queued == seq) ok = queue_q(it, (int)g, it.ntiles);  // not queued ahead (first item, or after an empty one)
-                if (ok && it_next.ntiles > 0 && queued == seq + 1) ok = queue_q(it_next, (int)g + it.ntiles, it_next.ntiles);
-                if (!ok) break;
-                ++seq;
                 int col_next = p.tile_col[it.tile_begin];
-                for (int j = it.tile_begin; j < it.tile_end && ok; ++j, ++g, ring.advance(NSK)) {
+                for (int j = it.tile_begin; j < it.tile_end; ++j, ++g, ring.advance(NSK)) {
                     const int col_cur = col_next;
                     if (j + 1 < it.tile_end) col_next = p.tile_col[j + 1];
                     const int stage = ring.stage;
                     const uint32_t ph = ring.phase;
-                    while (ok && npend > 0 &&
-                           (pq_need0 <= (int)g - NSK ||
-                            mbar_test_wait(smem_u32(&bars.q_empty[itq & 1]), ((itq >> 1) & 1) ^ 1)))
-                        ok = issue_q();
-                    if (!ok) break;
                     BSA_TRACE_POINT(0, tn, 19);
                     ok = mbar_wait(smem_u32(&bars.k_empty[stage]), ph ^ 1, abortp);
                     if (!ok) break;
@@ -1624,7 +1665,6 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     BSA_TRACE_POINT(0, tn, 21);
                 }
             }
-            while (ok && npend > 0) ok = issue_q();
             if (!ok) {
                 const uint64_t t0 = globaltimer_ns();
                 while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
@@ -1660,7 +1700,6 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         } else if (warp == 9 && lane == 0) {
             // =========================== Q K^T issuer ===========================
             constexpr uint32_t idesc_qk = make_idesc_f32(kTQ, TK, 0, 0, F16);
-            const uint64_t descQ0 = make_smem_desc_sw128(smem_u32(sQ), 16, 1024);
             const uint64_t descK = make_smem_desc_sw128(smem_u32(sK), 16, 1024);
             RingPos ring;  // K ring position of the tile being issued
             uint32_t itq = 0, g = 0;
@@ -1672,10 +1711,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const int n = n_next;
                 n_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles;
                 if (n <= 0) continue;
-                const uint32_t qb = itq & 1;  // this item's Q buffer
-                ok = mbar_wait(smem_u32(&bars.q_full[qb]), (itq >> 1) & 1, abortp);
+                const uint32_t qb = (NQT == 2) ? (itq & 1) : 0;  // this item's Q buffer in TMEM
+                ok = mbar_wait(smem_u32(&bars.qt_full[qb]), ((NQT == 2) ? (itq >> 1) : itq) & 1, abortp);
                 if (!ok) break;
-                const uint64_t descQ = descQ0 + (uint64_t)((qb * NSUB * Q_SUB) >> 4);
+                const uint32_t a_q = tmem + (qb ? Cols::kQ1 : Cols::kQ0);
                 for (int j = 0; j < n; ++j, ring.advance(NSK)) {
                     const uint32_t gs = g + j;
                     const int stage = ring.stage;
@@ -1693,9 +1732,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     const uint32_t d_s = tmem + (sb ? kColS1 : kColS0);
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k) {
-                        const uint64_t a = descQ + (uint64_t)(((k / 4) * Q_SUB + (k % 4) * 32) >> 4);
                         const uint64_t b = descK + (uint64_t)((stage * KV_TILE + (k / 4) * KV_SUB + (k % 4) * 32) >> 4);
-                        mma_ss(d_s, a, b, idesc_qk, k > 0);
+                        mma_ts(d_s, a_q + k * 8, b, idesc_qk, k > 0);
                     }
                     mma_commit(smem_u32(&bars.k_empty[stage]));
                     mma_commit(smem_u32(&bars.s_full[sb]));
@@ -1705,7 +1743,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     ++ph_n;
 #endif
                     BSA_TRACE_POINT(1, tn, 2);
-                    if (j == n - 1) mma_commit(smem_u32(&bars.q_empty[qb]));
+                    if (j == n - 1) mma_commit(smem_u32(&bars.qt_free[qb]));
                 }
                 g += n;
                 ++itq;
@@ -1744,7 +1782,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     BSA_TRACE_POINT(10, tn, 3);
 
                     tc_fence_after();
-                    const uint32_t a_p = tmem + (sb ? kColP1 : kColP0);
+                    const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0);
 #pragma unroll
                     for (int k = 0; k < TK / 16; ++k) {
                         const uint64_t b = descV + (uint64_t)((stage * KV_TILE + k * 2048) >> 4);
@@ -1774,7 +1812,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const int tw = tid & 127;
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t t_s = tmem + lane_base + (x ? kColS1 : kColS0);
-        const uint32_t t_p = tmem + lane_base + (x ? kColP1 : kColP0);
+        const uint32_t t_p = tmem + lane_base + (x ? Cols::kP1 : Cols::kP0);
         const uint32_t t_o = tmem + lane_base + kColO;
         uint32_t g = 0;          // running tile index at the start of the current item (all warpgroups agree)
         uint32_t itn = 0;        // non-empty items finished
@@ -1848,12 +1886,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     col_next = ldg_pinned_s32(p.tile_col + it.tile_begin + j + 2);
                     member_next = ldg_pinned_u64(p.tile_member + it.tile_begin + j + 2);
                 }
-                const bool need_mask = (member != p.full_member) || (kv0 + TK > p.Nkv);
+                const bool need_mask = __any_sync(0xffffffffu, (member != p.full_member) || (kv0 + TK > p.Nkv));
                 const uint32_t row_bits = (uint32_t)((member >> ((tw >> p.lgBQ) * p.sK)) & sub_mask);
                 const int n_valid = p.Nkv - kv0;
                 if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
                 BSA_PH(7);
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp));
+                ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
                 if (!ok) break;
                 BSA_PH(0);
                 if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
@@ -1898,8 +1936,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 float m_prev = -INFINITY;
                 if (gs > 0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
                     float m_taken;
-                    ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
-                    if (!ok) break;
+                    if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) + 1) & 3u))) {
+                        m_taken = __uint_as_float(ref_word & ~3u);
+                    } else {
+                        ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
+                        if (!ok) break;
+                    }
                     if (j > 0) m_prev = m_taken;  // the previous tile belongs to this item
                 }
 #ifdef BSA_PHASES
@@ -1937,7 +1979,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
                 constexpr bool kStoreInLoop = (D == 64);
                 if (kStoreInLoop && gs >= 2) {
-                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp));
+                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
                     if (!ok) break;
                     tc_fence_after();
                 }
@@ -1968,8 +2010,14 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
                 if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
                 if (!kStoreInLoop) {
-                    if (gs >= 2) {
-                        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp));
+                    if (Cols::kOneP) {  // the P tile before this one (other warpgroup's) must have been consumed
+                        if (gs >= 1) {
+                            ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                    } else if (gs >= 2) {
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
                         if (!ok) break;
                     }
                     BSA_PH(5);
@@ -1980,7 +2028,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 // ---- the reference moved at this tile: rescale the running output (after the P V of tile gs-1) ----
                 if (j > 0 && __any_sync(0xffffffffu, rescale)) {
                     const uint32_t gp = gs - 1;
-                    ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.pv_done[x ^ 1]), (gp >> 1) & 1, abortp));
+                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), (gp >> 1) & 1, abortp);
                     if (!ok) break;
                     tc_fence_after();
 #pragma unroll 1  // rare path: kept small
@@ -2016,7 +2064,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 if (m_final != m_know) l *= ex2_approx(m_know - m_final);  // l = 0 whenever m_know = -inf
                 // the previous item's sums must have been read
-                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp));
+                ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
                 if (!ok) break;
                 lfin[x][tw] = l;
                 if (owner) mfin[tw] = m_final;
@@ -2250,7 +2298,7 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
 static int static_smem_bytes(int kernel) { return (kernel == 2 || kernel == 4) ? 3072 : 1024; }
 
 static int kv_buffers_that_fit(int d, int T_KV, int kernel) {
-    const int q = ((kernel == 1 || kernel == 4) ? 2 : 1) * kTQ * d * 2;  // kernel 1: two Q slots; kernel 4: two Q buffers
+    const int q = (kernel == 1 ? 2 : 1) * kTQ * d * 2;  // kernel 1: two Q slots
     const int kv = T_KV * d * 2;
     return (232448 - static_smem_bytes(kernel) - q) / kv;
 }
@@ -2279,7 +2327,7 @@ int attention_max_stages(int d, int T_KV, int kernel) {
 }
 
 int attention_smem_bytes(int d, int T_KV, int stages, int kernel) {
-    const int q = ((kernel == 1 || kernel == 4) ? 2 : 1) * kTQ * d * 2;
+    const int q = (kernel == 1 ? 2 : 1) * kTQ * d * 2;
     const int kv = T_KV * d * 2;
     int need = q + ((kernel == 1 || kernel == 4) ? stages : 2 * stages) * kv;
     // more than half of the SM's shared memory, so exactly one CTA (and one 512-column TMEM allocation) per SM
