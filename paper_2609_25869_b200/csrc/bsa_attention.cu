@@ -86,7 +86,7 @@ struct AttnParams {
     int32_t Nkv;  // key/value tokens per head
     int32_t lgBQ;   // log2(B_Q) when B_Q < 128, else 31 (row >> 31 == 0)
     int32_t lgBKV;  // log2(B_KV) when B_KV < T_KV, else 31
-    int32_t sK;     // logical KV sub-blocks per tile
+    int32_t sK, lgSK;  // logical KV sub-blocks per entry of the tile list, and its logarithm
     int32_t stages;    // K ring depth (and V ring depth for the single-tile kernel)
     int32_t stages_v;  // V ring depth of the paired kernel
     float scale_log2;  // log2(e) / sqrt(d)
@@ -1340,9 +1340,19 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // on one GPU, the two builds in turn: 16384 tokens, 8 heads, d = 128, (128,128) blocks 177.8 -> 173.2 us; 115200
 // tokens, 24 heads 14.56 -> 14.26 ms (global order); 32768 tokens, 16 heads, d = 64, (256,256) 1355 -> 1307 us.  These
 // launches run at the 1 kW power cap (1.3-1.9 GHz of 1.965), so less traffic shows as a higher clock.
+//
+// G: a 128-key tile is made up of G entries of the plan's tile list (T_KV = 128 / G keys each), whichever they are: the
+// producers copy them one by one, and a 128-row, 128-column MMA works on a tile without gaps.  G = 1 where the logical
+// key blocks have 128 keys or more.  Narrower blocks used to be Coarsened onto aligned 128-key tiles, which also compute
+// their inactive neighbours, or walked in tiles of 64 keys, each with the hand-overs of a whole one.  On one GPU
+// (75600 tokens, d = 128, forward, builds in turn): (64,64) blocks, 24 heads, 10 % active 17.0 -> 11.4 ms (covered over
+// active pairs 1.44 both times); (32,32) 22.3 -> 14.9 ms (2.53 -> 1.92); (128,64) fp16, 12 heads, 30 % 11.7 -> 10.4 ms.
+// A K tile takes G*d/64 copies (the MMA wants its rows 128 bytes x 1024 apart across entries), a V tile G (an entry's
+// 64-column halves lie together, the MMA's descriptor moves from entry to entry).
 // TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448; d = 64: S0 0, S1 128, O 256, Q 320 and 352, P0 384, P1 448.
 // ==========================================================================================
 constexpr int kPpThreads = 512;
+constexpr int kPpTK = 128;  // keys of a tile
 
 // The whole warp waits for one barrier phase: one test and one vote when the phase has completed, the bounded wait
 // otherwise.  The result is the same in every lane.  (With the wait's loop and its early return in front of the vote the
@@ -1410,25 +1420,43 @@ struct __align__(8) PpBarriers {
 };
 
 // Tensor-memory columns of the ping-pong kernel.  Q is the A operand of Q K^T and lives in TMEM (D/2 columns).
-template <int D, int TK>
+template <int D>
 struct PpCols {
-    static constexpr bool kTight = (D == 128 && TK == 128);  // all 512 columns in use
+    static constexpr bool kTight = (D == 128);  // all 512 columns in use
     static constexpr uint32_t kP0 = kColP0, kP1 = kTight ? kColP0 : kColP1;
     static constexpr bool kOneP = (kP0 == kP1);
     static constexpr int kQBuffers = kTight ? 1 : 2;
-    static constexpr uint32_t kQ0 = kTight ? 448 : (D == 64 ? 320 : 64);
-    static constexpr uint32_t kQ1 = kTight ? 448 : (D == 64 ? 352 : 192);
+    static constexpr uint32_t kQ0 = kTight ? 448 : 320, kQ1 = kTight ? 448 : 352;
 };
 
-template <int D, int TK, bool F16>
+// Tiles of a list of n entries, G entries to a tile (n <= 0: no tiles, or past the end of the list).
+template <int G>
+__device__ __forceinline__ int tiles_of(int n) {
+    return n > 0 ? (n + G - 1) / G : n;
+}
+// First keys of the entries of one tile; entries beyond the list start at N_kv, where the copy reads zeros.
+template <int G, int GK>
+struct TileKeys {
+    int key0[G];
+    __device__ __forceinline__ void load(const int32_t* cols, int e0, int end, int n_kv) {
+#pragma unroll
+        for (int e = 0; e < G; ++e) key0[e] = (G == 1 || e0 + e < end) ? cols[e0 + e] * GK : n_kv;
+    }
+};
+
+template <int D, bool F16, int G>
 __global__ void __launch_bounds__(kPpThreads, 1)
 bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
+    constexpr int TK = kPpTK;
     constexpr int NSUB = D / 64;
     constexpr int Q_SUB = kTQ * 128;
     constexpr int KV_SUB = TK * 128;
     constexpr int KV_TILE = NSUB * KV_SUB;
-    using Cols = PpCols<D, TK>;
+    constexpr int GK = TK / G;  // keys of one entry of the tile list
+    constexpr int GV_TILE = KV_TILE / G;
+    constexpr int V_SUB = (G == 1) ? KV_SUB : GK * 128;  // a V tile holds its entries one after the other
+    using Cols = PpCols<D>;
     constexpr int NQT = Cols::kQBuffers;
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -1650,10 +1678,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const WorkItem it = it_next;
                 it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
                 if (it.ntiles <= 0) continue;
-                int col_next = p.tile_col[it.tile_begin];
-                for (int j = it.tile_begin; j < it.tile_end; ++j, ++g, ring.advance(NSK)) {
-                    const int col_cur = col_next;
-                    if (j + 1 < it.tile_end) col_next = p.tile_col[j + 1];
+                TileKeys<G, GK> next;
+                next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
+                for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSK)) {
+                    const TileKeys<G, GK> cur = next;
+                    if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
                     const int stage = ring.stage;
                     const uint32_t ph = ring.phase;
                     BSA_TRACE_POINT(0, tn, 19);
@@ -1661,7 +1690,16 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     if (!ok) break;
                     BSA_TRACE_POINT(0, tn, 20);
                     mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), KV_TILE);
-                    tma_load_4d(smem_u32(sK + stage * KV_TILE), &tmK, smem_u32(&bars.k_full[stage]), 0, col_cur * TK, 0, it.head);
+                    if constexpr (G == 1) {
+                        tma_load_4d(smem_u32(sK + stage * KV_TILE), &tmK, smem_u32(&bars.k_full[stage]), 0, cur.key0[0], 0, it.head);
+                    } else {
+#pragma unroll
+                        for (int e = 0; e < G; ++e)
+#pragma unroll
+                            for (int s = 0; s < NSUB; ++s)
+                                tma_load_4d(smem_u32(sK + stage * KV_TILE + s * KV_SUB + e * GK * 128), &tmK,
+                                            smem_u32(&bars.k_full[stage]), 0, cur.key0[e], s, it.head);
+                    }
                     BSA_TRACE_POINT(0, tn, 21);
                 }
             }
@@ -1680,17 +1718,21 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const WorkItem it = it_next;
                 it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
                 if (it.ntiles <= 0) continue;
-                int col_next = p.tile_col[it.tile_begin];
-                for (int j = it.tile_begin; j < it.tile_end; ++j, ++g, ring.advance(NSV)) {
-                    const int col_cur = col_next;
-                    if (j + 1 < it.tile_end) col_next = p.tile_col[j + 1];
+                TileKeys<G, GK> next;
+                next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
+                for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSV)) {
+                    const TileKeys<G, GK> cur = next;
+                    if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
                     const int stage = ring.stage;
                     const uint32_t ph = ring.phase;
                     if (withhold && g == 0) continue;  // this tile never arrives
                     ok = mbar_wait(smem_u32(&bars.v_empty[stage]), ph ^ 1, abortp);
                     if (!ok) break;
                     mbar_arrive_expect_tx(smem_u32(&bars.v_full[stage]), KV_TILE);
-                    tma_load_4d(smem_u32(sV + stage * KV_TILE), &tmV, smem_u32(&bars.v_full[stage]), 0, col_cur * TK, 0, it.head);
+#pragma unroll
+                    for (int e = 0; e < G; ++e)
+                        tma_load_4d(smem_u32(sV + stage * KV_TILE + e * GV_TILE), &tmV, smem_u32(&bars.v_full[stage]), 0,
+                                    cur.key0[e], 0, it.head);
                 }
             }
             if (!ok) {
@@ -1706,10 +1748,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             bool ok = true;
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
-            int n_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles;
+            int n_next = tiles_of<G>(load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const int n = n_next;
-                n_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles;
+                n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
                 if (n <= 0) continue;
                 const uint32_t qb = (NQT == 2) ? (itq & 1) : 0;  // this item's Q buffer in TMEM
                 ok = mbar_wait(smem_u32(&bars.qt_full[qb]), ((NQT == 2) ? (itq >> 1) : itq) & 1, abortp);
@@ -1754,16 +1796,16 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         } else if (warp == 10 && lane == 0) {
             // =========================== P V issuer ===========================
             constexpr uint32_t idesc_pv = make_idesc_f32(kTQ, D, 0, 1, F16);
-            const uint64_t descV = make_smem_desc_sw128(smem_u32(sV), KV_SUB, 1024);
+            const uint64_t descV = make_smem_desc_sw128(smem_u32(sV), V_SUB, 1024);
             RingPos ring;  // V ring position of the tile being issued
             uint32_t itq = 0, g = 0;
             bool ok = true;
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
-            int n_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles;
+            int n_next = tiles_of<G>(load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const int n = n_next;
-                n_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles;
+                n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
                 if (n <= 0) continue;
                 for (int j = 0; j < n; ++j, ring.advance(NSV)) {
                     const uint32_t gp = g + j;
@@ -1785,7 +1827,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0);
 #pragma unroll
                     for (int k = 0; k < TK / 16; ++k) {
-                        const uint64_t b = descV + (uint64_t)((stage * KV_TILE + k * 2048) >> 4);
+                        const uint64_t b = descV + (uint64_t)((stage * KV_TILE + (k / (GK / 16)) * GV_TILE + (k % (GK / 16)) * 2048) >> 4);
                         mma_ts(tmem + kColO, a_p + k * 8, b, idesc_pv, (j > 0 || k > 0) ? 1u : 0u);
                     }
                     mma_commit(smem_u32(&bars.v_empty[stage]));
@@ -1819,7 +1861,21 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         bool ok = true;
         BSA_TRACE_DECL(tn);
         const float c2 = p.scale_log2;
-        const unsigned long long sub_mask = (p.sK >= 64) ? ~0ull : ((1ull << p.sK) - 1ull);
+        // Membership (64-row, 128-key blocks, 75600 tokens, 12 heads: 5.74 -> 5.27 ms against reading the 64-bit word and
+        // the column of every tile in every thread): each half-warp of 16 rows lies inside one logical row block, and a
+        // tile has at most eight key sub-blocks, so lane l of a half-warp fetches the bit of sub-block l for the
+        // half-warp's rows and one ballot hands all of them to every lane.  Plans whose entries have a single membership
+        // bit need no loads at all.
+        const int nb = G * p.sK, l16 = lane & 15;
+        const bool has_bits = p.full_member != 1ull;
+        const int mbit = (((tw & ~15) >> p.lgBQ) * p.sK) + (l16 & (p.sK - 1));
+        const int ment = l16 >> p.lgSK;  // entry of the tile this lane's bit belongs to
+        const uint32_t full_bits = (1u << nb) - 1u, full_ballot = full_bits | (full_bits << 16);
+        const int32_t* mwords = reinterpret_cast<const int32_t*>(p.tile_member) + (mbit >> 5);
+        auto load_bit = [&](int entry, int end) -> uint32_t {  // word that holds this lane's bit (0 beyond the list)
+            if (l16 >= nb || entry + ment >= end) return 0u;
+            return has_bits ? (uint32_t)ldg_pinned_s32(mwords + 2 * (int64_t)(entry + ment)) : 0xffffffffu;
+        };
         BSA_PH_DECL;
         // The reference after global tile t (taken by the other warpgroup), given a word read earlier from its slot:
         // if that word already carries the publish's tag it is used, else the slot is polled (bounded).
@@ -1850,28 +1906,25 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // item nor the metadata that depends on it is waited for at an item boundary
         ItemSpan it_next = load_item_span(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
         ItemSpan it_next2 = load_item_span(p.items, cta_item_index(1, blockIdx.x, gridDim.x), n_items);
-        int first_col = 0;
-        unsigned long long first_member = 0ull;
+        int last_col = 0;
+        uint32_t first_word = 0;
         {
             const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
-            if (j0n < it_next.ntiles) {
-                first_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + j0n);
-                first_member = ldg_pinned_u64(p.tile_member + it_next.tile_begin + j0n);
-            }
+            first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+            if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
         }
         for (int kr = 0; kr < n_rounds && ok; ++kr) {
             const ItemSpan it = it_next;
             it_next = it_next2;
             it_next2 = load_item_span(p.items, cta_item_index(kr + 2, blockIdx.x, gridDim.x), n_items);
-            const int n = it.ntiles;
-            int col_next = first_col;
-            unsigned long long member_next = first_member;
+            const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
+            uint32_t word_next = first_word;
+            // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
+            const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
             {   // the next item's first tile of this warpgroup: its parity follows from g + n
                 const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
-                if (j0n < it_next.ntiles) {
-                    first_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + j0n);
-                    first_member = ldg_pinned_u64(p.tile_member + it_next.tile_begin + j0n);
-                }
+                first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+                if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
             }
             if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
             float m_know = -INFINITY;  // reference maximum this thread's partial sum l is expressed in
@@ -1880,15 +1933,14 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
             for (int j = j0; j < n; j += 2) {
                 const uint32_t gs = g + j;
-                const int kv0 = col_next * TK;
-                const unsigned long long member = member_next;
-                if (j + 2 < n) {
-                    col_next = ldg_pinned_s32(p.tile_col + it.tile_begin + j + 2);
-                    member_next = ldg_pinned_u64(p.tile_member + it.tile_begin + j + 2);
+                uint32_t ballot = full_ballot;
+                if (G > 1 || has_bits) {
+                    ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
+                    if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
                 }
-                const bool need_mask = __any_sync(0xffffffffu, (member != p.full_member) || (kv0 + TK > p.Nkv));
-                const uint32_t row_bits = (uint32_t)((member >> ((tw >> p.lgBQ) * p.sK)) & sub_mask);
-                const int n_valid = p.Nkv - kv0;
+                const bool need_mask = ballot != full_ballot;
+                const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
+                const bool ragged = (j == n - 1) && n_valid < TK;
                 if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
                 BSA_PH(7);
                 ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
@@ -1909,16 +1961,18 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 // word checked after the max phase, so that the shared-memory round trip overlaps that phase.
                 const uint32_t ref_word = *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]);
                 if (need_mask) {
-                    // B_KV >= 16, so a group of 16 key columns lies inside one logical block: one activity bit per
-                    // group, two instructions per element.  (Skipping, per warp, the groups none of its 32 rows needs
-                    // was tried and lost: a warpgroup still waits for its slowest warp, and the branches cost more
-                    // than the exponentials they save.)
+                    // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
+                    // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
 #pragma unroll
                     for (int gq = 0; gq < TK / 16; ++gq) {
                         const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
 #pragma unroll
-                        for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = (grp && i < n_valid) ? r[i] : 0xff800000u;
+                        for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
                     }
+                }
+                if (ragged) {
+#pragma unroll
+                    for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
                 }
                 float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
 #pragma unroll
@@ -2194,7 +2248,9 @@ bool encode_map(CUtensorMap* m, const void* base, int64_t N, int heads, int d, i
 
 // The same tensor as {64 columns, N rows, d/64 column groups, heads}; box = {64, rows, d/64, 1}: one copy lands all
 // 64-column sub-tiles of a row block back to back (the [sub-tile][row][64] layout the MMA descriptors address).
-bool encode_map4(CUtensorMap* m, const void* base, int64_t N, int heads, int d, int box_rows, bool f16, bool nhd) {
+// `col_groups` > 0: that many sub-tiles per copy instead of all d/64.
+bool encode_map4(CUtensorMap* m, const void* base, int64_t N, int heads, int d, int box_rows, bool f16, bool nhd,
+                 int col_groups = 0) {
     EncodeTiledFn enc = get_encode_fn();
     if (!enc) return false;
     cuuint64_t dims[4] = {64, (cuuint64_t)N, (cuuint64_t)(d / 64), (cuuint64_t)heads};
@@ -2203,7 +2259,7 @@ bool encode_map4(CUtensorMap* m, const void* base, int64_t N, int heads, int d, 
         strides[0] = (cuuint64_t)heads * (cuuint64_t)d * 2;
         strides[2] = (cuuint64_t)d * 2;
     }
-    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, (cuuint32_t)(d / 64), 1};
+    cuuint32_t box[4] = {64, (cuuint32_t)box_rows, (cuuint32_t)(col_groups > 0 ? col_groups : d / 64), 1};
     cuuint32_t es[4] = {1, 1, 1, 1};
     return enc(m, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 4, const_cast<void*>(base), dims,
                strides, box, es,
@@ -2211,13 +2267,13 @@ bool encode_map4(CUtensorMap* m, const void* base, int64_t N, int heads, int d, 
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-template <int D, int TK, int KERNEL>
+template <int D, int TK, int KERNEL, int G = 1>
 cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t stream, const char** err) {
     CUtensorMap tq, tk, tv;
     const bool ok_maps = (KERNEL == 4)
                              ? (encode_map4(&tq, a.Q, a.g.N, a.g.H, D, kTQ, a.f16, a.nhd) &&
-                                encode_map4(&tk, a.K, a.g.N_kv, a.g.H, D, TK, a.f16, a.nhd) &&
-                                encode_map4(&tv, a.V, a.g.N_kv, a.g.H, D, TK, a.f16, a.nhd))
+                                encode_map4(&tk, a.K, a.g.N_kv, a.g.H, D, TK / G, a.f16, a.nhd, G > 1 ? 1 : D / 64) &&
+                                encode_map4(&tv, a.V, a.g.N_kv, a.g.H, D, TK / G, a.f16, a.nhd))
                              : (encode_map(&tq, a.Q, a.g.N, a.g.H, D, kTQ, a.f16, a.nhd) &&
                                 encode_map(&tk, a.K, a.g.N_kv, a.g.H, D, TK, a.f16, a.nhd) &&
                                 encode_map(&tv, a.V, a.g.N_kv, a.g.H, D, TK, a.f16, a.nhd));
@@ -2246,9 +2302,9 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         else if constexpr (KERNEL == 2)
             e = cudaFuncSetAttribute(bsa_attention_cs_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         else {
-            e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, TK, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
             if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, TK, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, true, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         }
         if (e != cudaSuccess) {
             *err = "cudaFuncSetAttribute(max dynamic shared memory)";
@@ -2282,8 +2338,8 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t le = a.f16 ? cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, TK, true>, tq, tk, tv, p)
-                               : cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, TK, false>, tq, tk, tv, p);
+        cudaError_t le = a.f16 ? cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, true, G>, tq, tk, tv, p)
+                               : cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, false, G>, tq, tk, tv, p);
         count_launch();
         return le;
     }
@@ -2318,6 +2374,7 @@ static void split_stages(int total, int kernel, int* nk, int* nv) {
 }
 
 int attention_max_stages(int d, int T_KV, int kernel) {
+    if (kernel == 4) T_KV = kPpTK;
     if (kernel == kKernelRowBlock) return (d <= 128 && T_KV <= rb_max_chunk(d)) ? 2 : 0;  // one K and one V buffer per warp
     if (d == 256 && !((kernel == 0 || kernel == 3) && T_KV == 64)) return 0;  // see launch_forward
     const int nb = kv_buffers_that_fit(d, T_KV, kernel);
@@ -2327,6 +2384,7 @@ int attention_max_stages(int d, int T_KV, int kernel) {
 }
 
 int attention_smem_bytes(int d, int T_KV, int stages, int kernel) {
+    if (kernel == 4) T_KV = kPpTK;
     const int q = (kernel == 1 ? 2 : 1) * kTQ * d * 2;
     const int kv = T_KV * d * 2;
     int need = q + ((kernel == 1 || kernel == 4) ? stages : 2 * stages) * kv;
@@ -2371,7 +2429,12 @@ cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t stream, const char
     p.o_row = a.nhd ? (int64_t)a.g.H * a.d : (int64_t)a.d;
     p.lgBQ = (a.g.sQ128 > 1) ? a.g.lgBQ : 31;
     p.lgBKV = (a.g.sK > 1) ? a.g.lgBKV : 31;
+    if (a.kernel == 4) {  // columns of a tile that share a membership bit
+        p.lgBKV = -a.g.lgSK;
+        while ((1 << (p.lgBKV + a.g.lgSK)) < a.g.T_KV) ++p.lgBKV;
+    }
     p.sK = a.g.sK;
+    p.lgSK = a.g.lgSK;
     p.stages = a.stages;
     p.stages_v = a.stages;
     if (a.kernel == 1 || a.kernel == 4) split_stages(a.stages, a.kernel, &p.stages, &p.stages_v);
@@ -2399,10 +2462,13 @@ cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t stream, const char
     // buffers only where P is written in place over S (the single-tile kernels), with 64-key tiles
     else if (key == 256 + 1) e = launch_attn<256, 64, 0>(a, p, stream, err_detail);
     else if (key == 3000 + 256 + 1) e = launch_attn<256, 64, 3>(a, p, stream, err_detail);
-    else if (key == 4000 + 128 + 2) e = launch_attn<128, 128, 4>(a, p, stream, err_detail);
-    else if (key == 4000 + 128 + 1) e = launch_attn<128, 64, 4>(a, p, stream, err_detail);
-    else if (key == 4000 + 64 + 2) e = launch_attn<64, 128, 4>(a, p, stream, err_detail);
-    else if (key == 4000 + 64 + 1) e = launch_attn<64, 64, 4>(a, p, stream, err_detail);
+    else if (key == 4000 + 128 + 2) e = launch_attn<128, kPpTK, 4>(a, p, stream, err_detail);
+    else if (key == 4000 + 64 + 2) e = launch_attn<64, kPpTK, 4>(a, p, stream, err_detail);
+    // narrower entries: two of 64 keys or four of 32 to a tile
+    else if (key == 4000 + 128 + 1) e = launch_attn<128, kPpTK, 4, 2>(a, p, stream, err_detail);
+    else if (key == 4000 + 128 && a.g.T_KV == 32) e = launch_attn<128, kPpTK, 4, 4>(a, p, stream, err_detail);
+    else if (key == 4000 + 64 + 1) e = launch_attn<64, kPpTK, 4, 2>(a, p, stream, err_detail);
+    else if (key == 4000 + 64 && a.g.T_KV == 32) e = launch_attn<64, kPpTK, 4, 4>(a, p, stream, err_detail);
     else {
         *err_detail = "no kernel for this (d, T_KV)";
         return cudaErrorInvalidValue;

@@ -67,6 +67,12 @@ static const bsa_plan_desc_t kCatalog[] = {
     {36, 16, 16, 0, 0, 1, BSA_ORDER_HEAD_MAJOR_LPT, 5, "q16k16_rb"},
     {37, 16, 64, 0, 0, 1, BSA_ORDER_NATURAL, 5, "q16k64_rb_natural"},
     {38, 16, 32, 0, 0, 1, BSA_ORDER_NATURAL, 5, "q16k32_rb_natural"},
+    // 32-key entries, four to a 128-key tile of the ping-pong kernel: for logical key blocks of 16 and 32
+    {39, 128, 32, 0, 0, 1, BSA_ORDER_HEAD_MAJOR_LPT, 4, "q128k32_pp"},
+    {40, 128, 32, 0, 0, 1, BSA_ORDER_GLOBAL_LPT, 4, "q128k32_pp_global"},
+    {41, 128, 32, 0, 0, 1, BSA_ORDER_NATURAL, 4, "q128k32_pp_natural"},
+    {42, 128, 32, 0, 0, 1, BSA_ORDER_GLOBAL_BUCKETS, 4, "q128k32_pp_gb"},
+    {43, 128, 32, 0, 16, 8, BSA_ORDER_HEAD_MAJOR_LPT, 4, "q128k32_pp_split16x8"},
 };
 static const int kCatalogSize = (int)(sizeof(kCatalog) / sizeof(kCatalog[0]));
 static const int64_t kDefaultWorkspace = 2ll << 30;
@@ -129,6 +135,8 @@ bool plan_eligible(int plan_id, int B_Q, int B_KV, int64_t N, int heads, int d, 
         // no larger than a warp's staging buffer, no Split-K
         if (B_Q > 64 || B_KV < P->T_KV || P->T_KV > rb_max_chunk(d) || P->split_pmax > 1) return false;
     }
+    // 32-key entries cost a copy instruction each: only where the logical blocks are that narrow
+    if (P->kernel == 4 && P->T_KV == 32 && B_KV > 32) return false;
     if (!(d == 64 || d == 128 || d == 256)) return false;
     if (!pow2_in(B_Q, 16, 256) || !pow2_in(B_KV, 16, 256)) return false;
     if (N <= 0 || heads <= 0 || N > (1ll << 30)) return false;

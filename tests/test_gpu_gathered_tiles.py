@@ -1,0 +1,36 @@
+"""GPU parity of the ping-pong kernel on tiles gathered from several narrow entries of the tile list (two of 64 keys,
+four of 32): list lengths around multiples of the entries per tile, ragged last blocks, every row-block size, both
+head dimensions and element types, Split-K partitions that start anywhere in the list."""
+import numpy as np
+import pytest
+
+from paper_2609_25869_b200 import inputs as I
+from tests import helpers as Hh
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("B_Q,B_KV,N,N_kv,d,dtype,plan_id", [
+    (16, 16, 1000, 0, 64, "bf16", 39), (16, 32, 777, 1300, 128, "bf16", 39), (32, 16, 900, 0, 128, "fp16", 40),
+    (32, 32, 3000, 0, 128, "bf16", 42), (64, 32, 1300, 1111, 64, "fp16", 41), (128, 32, 1000, 0, 128, "bf16", 39),
+    (256, 16, 900, 0, 64, "bf16", 43), (32, 32, 2000, 3001, 128, "bf16", 43),
+    (16, 16, 1000, 0, 128, "bf16", 23), (32, 32, 1500, 0, 64, "fp16", 26), (64, 64, 1301, 0, 128, "bf16", 33),
+    (128, 64, 2000, 999, 128, "fp16", 32), (16, 64, 1000, 0, 64, "bf16", 28), (256, 256, 1100, 0, 128, "bf16", 23),
+    (64, 128, 1000, 0, 128, "bf16", 27)])
+def test_gathered_tiles_match_the_oracle(B_Q, B_KV, N, N_kv, d, dtype, plan_id):
+    H = 3
+    M = I.random_mask(B_Q + 7 * B_KV + N, H, I.cdiv(N, B_Q), I.cdiv(N_kv or N, B_KV), 0.3, empty_rows=0.15)
+    Hh.run_request(I.Request("gather", H, N, d, B_Q, B_KV, M, qkv_seed=N, N_kv=N_kv, dtype=dtype), plan_id=plan_id)
+
+
+@pytest.mark.parametrize("B,plan_id", [(32, 39), (64, 23)])
+def test_list_lengths_around_whole_tiles(B, plan_id):
+    """Query block i has i + 1 active key blocks: lists of 1, 2, ... entries, each with the ragged last block or not."""
+    n = 13
+    M = np.zeros((2, n, n), np.uint8)
+    for i in range(n):
+        M[0, i, n - 1 - i:] = 1
+        M[1, i, :i + 1] = 1
+    Hh.run_request(I.Request("lengths", 2, n * B - 5, 128, B, B, M, qkv_seed=B), plan_id=plan_id)
+    # 128-row query blocks: every list length belongs to one work item
+    Hh.run_request(I.Request("lengths", 2, n * 128, 128, 128, B, M, qkv_seed=B + 1, N_kv=n * B - 5), plan_id=plan_id)
