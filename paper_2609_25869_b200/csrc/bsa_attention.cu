@@ -1354,14 +1354,6 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 constexpr int kPpThreads = 512;
 constexpr int kPpTK = 128;  // keys of a tile
 
-// The whole warp waits for one barrier phase: one test and one vote when the phase has completed, the bounded wait
-// otherwise.  The result is the same in every lane.  (With the wait's loop and its early return in front of the vote the
-// common case crossed a divergent region: about 2 % of the softmax warpgroups' time.)
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
-    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
-}
-
 // The k-th work item of CTA b out of G: rounds of G consecutive items, alternately dealt forwards and backwards.
 // Items arrive longest first, so dealing every round in the same direction would hand CTA 0 the longest item of
 // every round and the last CTA the shortest; reversing every other round evens the per-CTA sums out.
@@ -2348,6 +2340,10 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
 }
 
 }  // namespace
+
+bool encode_kv_map(CUtensorMap* m, const void* base, int64_t N, int heads, int d, int box_rows, bool f16, bool nhd) {
+    return encode_map4(m, base, N, heads, d, box_rows, f16, nhd);
+}
 
 // Shared-memory budget: 227 KB per CTA minus each kernel's static shared memory (barriers, exchange
 // buffer), which the compiler rounds up to the 1024-byte alignment of the dynamic part.

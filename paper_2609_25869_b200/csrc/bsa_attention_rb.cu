@@ -7,54 +7,51 @@
 // their own granularity instead: one WARP owns a 16-row fragment of a logical row block (a 16-row physical tile,
 // Refined along Q for B_Q > 16) and walks that block's own KV tile list with the register-level tensor instruction
 // mma.sync.m16n8k16 (bf16 or fp16 in, fp32 accumulate), FlashAttention-2 style:
-//   * K and V chunks of T_KV keys (8 KB each at most) are gathered with cp.async into a 16 KB staging area private to
-//     the warp (128-byte-row XOR swizzle), K read back with ldmatrix, V with ldmatrix.trans; the next K chunk is in
-//     flight during the softmax and P V of the current one, the next V chunk during the next Q K^T;
+//   * K and V are copied in steps of at most 32 keys into two 8 KB rings private to the warp, by TMA tiles (128-byte
+//     swizzle) that one lane issues: K read back with ldmatrix, V with ldmatrix.trans; a ring slot is refilled as soon
+//     as the warp has read it, so the next steps' copies are in flight during the arithmetic of the current one;
 //   * S = Q K^T, online softmax with the running row maximum in the exp2 domain, P rounded to bf16 in registers
 //     (the accumulator layout of two 8-key tiles is the A-operand layout of one 16-key step), O += P V;
 //   * no block-level synchronisation at all: warps are independent, twelve per SM.
+// A block of 16 rows and 64 keys (d = 64) is 262 kflop on 16 KB of K and V, each byte used once: shared memory sees it
+// twice (copy in, ldmatrix), 256 clk per SM at 128 B/clk against 133 clk of MMA, which makes 2.2 ms of the workload
+// below.  With per-thread cp.async copies of whole entries the load path stopped at about 41 B/clk per SM (bulk copies
+// reach 80); now, on one GPU, 32768 tokens, 16 heads, d = 64, (16,64) blocks, 15 % active in runs: 3.58 -> 2.77 ms; the
+// same with 32-key entries 4.01 -> 2.94 ms, (32,32) blocks at d = 128 52 -> 40 ms.  (Fragments loaded straight from
+// global memory, no shared memory at all: 5.4 ms, the L1 miss path moves about 32 B/clk.  Fourteen warps: spills, 3.95.)
 // The register-level instruction peaks at about a third of the tcgen05 rate on this GPU, so the kernel pays off only
 // where Coarsening wastes more than that; the plan table decides per regime.
+#include <cuda.h>
 #include <cuda_bf16.h>
 #include <math.h>
 
 #include <atomic>
 
 #include "bsa_common.h"
+#include "sm100_ptx.cuh"
 
 namespace bsa {
+
+using namespace ptx;
+
 namespace {
 
 constexpr int kRbWarps = 12;        // warps per CTA (one CTA per SM)
-constexpr int kRbStageBytes = 8192; // one K or V chunk
+constexpr int kRbStageBytes = 8192; // one warp's K or V ring
 constexpr unsigned kFullMask = 0xffffffffu;
 
 struct RbParams {
     const __nv_bfloat16* Q;
-    const __nv_bfloat16* K;
-    const __nv_bfloat16* V;
     __nv_bfloat16* O;
     float* LSE;
     const WorkItem* items;
     const int32_t* tile_col;
-    const PlanCountersDev* counters;
+    PlanCountersDev* counters;
     long long q_head, q_row;    // element strides of Q and O between heads / token rows
-    long long kv_head, kv_row;  // the same for K and V
     int32_t N, Nkv;
     float scale_log2;           // log2(e) / sqrt(d)
 };
 
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return static_cast<uint32_t>(__cvta_generic_to_shared(p)); }
-
-// 16-byte asynchronous copy global -> shared; src_bytes = 0 writes zeros (rows beyond the last key).
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes) {
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() {
-    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
-}
 __device__ __forceinline__ void ldmatrix_x4(uint32_t addr, uint32_t& r0, uint32_t& r1, uint32_t& r2, uint32_t& r3) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
                  : "=r"(r0), "=r"(r1), "=r"(r2), "=r"(r3)
@@ -94,52 +91,59 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {  // two fp32
     return r;
 }
 
-// Byte offset of 16-byte chunk `chunk` of row `row` in a staged tile whose rows are ROWB bytes: the chunk index is
-// XORed with the row's low three bits, so the eight row addresses of an ldmatrix fall into eight different bank groups.
-template <int ROWB>
+// Byte offset of 16-byte chunk `chunk` of row `row` in a ring slot of ROWS rows as the copy lays it out: 64-column
+// halves one after the other, 128-byte rows, the chunk index XORed with the row's low three bits, so that the eight row
+// addresses of an ldmatrix fall into eight different bank groups.
+template <int ROWS>
 __device__ __forceinline__ uint32_t swz(int row, int chunk) {
-    return (uint32_t)(row * ROWB + ((chunk ^ (row & 7)) << 4));
+    return (uint32_t)((chunk >> 3) * (ROWS * 128) + row * 128 + (((chunk & 7) ^ (row & 7)) << 4));
 }
 
-// Gathers keys [key0, key0 + CK) of one head (rows of D bf16) into a staging buffer; rows at or beyond n_rows are
-// written as zeros.  512 bytes per warp instruction, consecutive lanes on consecutive 16-byte chunks of a row.
+// Keys per step: small enough that a ring holds two of them.
 template <int D, int CK>
-__device__ __forceinline__ void stage_chunk(uint32_t dst, const __nv_bfloat16* __restrict__ base, long long row_stride,
-                                            int key0, int n_rows, int lane) {
-    constexpr int CPR = D / 8;                 // 16-byte chunks per row
-    constexpr int ITERS = CK * CPR / 32;
-#pragma unroll
-    for (int i = 0; i < ITERS; ++i) {
-        const int idx = i * 32 + lane;
-        const int row = idx / CPR, chunk = idx % CPR;
-        const int key = key0 + row;
-        const bool ok = key < n_rows;
-        const __nv_bfloat16* src = base + (long long)(ok ? key : n_rows - 1) * row_stride + chunk * 8;
-        cp_async16(dst + swz<D * 2>(row, chunk), src, ok ? 16 : 0);
-    }
-}
+constexpr int kRbStep = (CK * D * 4 <= kRbStageBytes) ? CK : kRbStageBytes / (D * 4);
 
 template <int D, int CK, bool F16>
-__global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(const RbParams p) {
-    static_assert(CK * D * 2 <= kRbStageBytes, "a chunk must fit its staging buffer");
-    static_assert(CK % 16 == 0 && D % 16 == 0, "whole MMA steps");
-    constexpr int NT_S = CK / 8;   // 8-key accumulator tiles of S
+__global__ void __launch_bounds__(kRbWarps * 32, 1)
+bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_constant__ CUtensorMap tmV, const RbParams p) {
+    constexpr int KS = kRbStep<D, CK>;      // keys per step
+    constexpr int SPE = CK / KS;            // steps per entry of the tile list
+    constexpr int SLOT = KS * D * 2;        // bytes of a ring slot
+    constexpr int NST = kRbStageBytes / SLOT;
+    static_assert(KS % 16 == 0 && CK % KS == 0 && D % 64 == 0 && NST >= 2, "whole MMA steps");
+    constexpr int NT_S = KS / 8;   // 8-key accumulator tiles of S
     constexpr int KS_QK = D / 16;  // 16-wide steps over the head dimension
-    constexpr int KS_PV = CK / 16; // 16-key steps of P V
+    constexpr int KS_PV = KS / 16; // 16-key steps of P V
     constexpr int NT_O = D / 8;    // 8-column accumulator tiles of O
-    extern __shared__ __align__(128) uint8_t smem[];
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ __align__(8) uint64_t bars[kRbWarps][2 * NST];  // K slots, then V slots: the copy has landed
+    __shared__ uint32_t abort_flag;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
-    uint8_t* stage = smem + warp * 2 * kRbStageBytes;
-    const uint32_t sK = smem_addr(stage), sV = sK + kRbStageBytes;
+    const uint32_t sK = smem_u32(smem + warp * 2 * kRbStageBytes), sV = sK + kRbStageBytes;
+    const uint32_t bK = smem_u32(&bars[warp][0]), bV = bK + NST * 8;
+    if (smem_u32(smem) & 1023u) {  // never expected; fail with a status instead of corrupting tiles
+        if (threadIdx.x == 0) atomicExch(&p.counters->status, (int)BSA_ERR_CUDA);
+        return;
+    }
+    if (threadIdx.x == 0) abort_flag = 0;
+    if (lane == 0) {
+        for (int i = 0; i < 2 * NST; ++i) mbar_init(bK + i * 8, 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    volatile uint32_t* abortp = &abort_flag;
 
     const int n_items = p.counters->nitems;
     const int total_warps = (int)gridDim.x * kRbWarps;
     const int gw = (int)blockIdx.x * kRbWarps + warp;
     const int n_rounds = (n_items + total_warps - 1) / total_warps;
     const float c2 = p.scale_log2;
+    int slot = 0;          // ring slot of the current step (the same for K and V)
+    uint32_t phase = 0;    // its barriers' phase
+    bool ok = true;
 
-    for (int k = 0; k < n_rounds; ++k) {
+    for (int k = 0; k < n_rounds && ok; ++k) {
         // items arrive longest first: rounds are dealt alternately forwards and backwards to even out the warps' sums
         const int idx = k * total_warps + ((k & 1) ? (total_warps - 1 - gw) : gw);
         if (idx >= n_items) continue;
@@ -161,14 +165,24 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
             }
             continue;
         }
-        const __nv_bfloat16* Kh = p.K + (long long)head * p.kv_head;
-        const __nv_bfloat16* Vh = p.V + (long long)head * p.kv_head;
-        // first K and V chunks on their way while the Q fragment is loaded
-        int col = __ldg(p.tile_col + tile_begin);
-        stage_chunk<D, CK>(sK, Kh, p.kv_row, col * CK, p.Nkv, lane);
-        cp_async_commit();
-        stage_chunk<D, CK>(sV, Vh, p.kv_row, col * CK, p.Nkv, lane);
-        cp_async_commit();
+        const int n_steps = (tile_end - tile_begin) * SPE;
+        auto first_key = [&](int st) { return __ldg(p.tile_col + tile_begin + st / SPE) * CK + (st % SPE) * KS; };
+        auto copy_in = [&](uint32_t dst, const CUtensorMap* map, uint32_t bar, int key0) {
+            mbar_arrive_expect_tx(bar, SLOT);
+            tma_load_4d(dst, map, bar, 0, key0, 0, head);
+        };
+        // the first steps' copies are on their way while the Q fragment is loaded
+        if (lane == 0) {
+            int sl = slot;
+            for (int st = 0; st < NST && st < n_steps; ++st) {
+                const int key0 = first_key(st);
+                copy_in(sK + sl * SLOT, &tmK, bK + sl * 8, key0);
+                copy_in(sV + sl * SLOT, &tmV, bV + sl * 8, key0);
+                if (++sl == NST) sl = 0;
+            }
+        }
+        const int last_key = __ldg(p.tile_col + tile_end - 1) * CK;  // columns ascend: only the last entry can be ragged
+        int key_next = (NST < n_steps) ? first_key(NST) : 0;         // of the step to copy next
         // Q fragment (A operand, row-major 16 x 16 per step): rows g and g+8, columns 2t, 2t+1 and 8 further
         uint32_t qa[KS_QK][4];
         {
@@ -189,13 +203,14 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
         float m_lo = -INFINITY, m_hi = -INFINITY;  // running row maxima, exp2 domain (score * c2)
         float l_lo = 0.f, l_hi = 0.f;              // this thread's share of the row sums
 
-        for (int j = tile_begin; j < tile_end; ++j) {
-            const int key0 = col * CK;
-            const bool more = j + 1 < tile_end;
-            const int col_next = more ? __ldg(p.tile_col + j + 1) : 0;
+        for (int st = 0; st < n_steps; ++st) {
+            const bool more = st + NST < n_steps;
+            const int key_in = key_next;
+            if (st + NST + 1 < n_steps) key_next = first_key(st + NST + 1);
+            const uint32_t cK = sK + slot * SLOT, cV = sV + slot * SLOT;
             // ---- S = Q K^T ----
-            cp_async_wait<1>();  // K chunk j has landed (V chunk j may still be in flight)
-            __syncwarp();
+            ok = mbar_wait_warp(bK + slot * 8, phase, abortp);
+            if (!ok) break;
             float s[NT_S][4];
 #pragma unroll
             for (int n = 0; n < NT_S; ++n) s[n][0] = s[n][1] = s[n][2] = s[n][3] = 0.f;
@@ -207,19 +222,18 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
                     const int key = np * 16 + ((lane >> 4) << 3) + (lane & 7);
                     const int chunk = ks * 2 + ((lane >> 3) & 1);
                     uint32_t b0, b1, b2, b3;
-                    ldmatrix_x4(sK + swz<D * 2>(key, chunk), b0, b1, b2, b3);
+                    ldmatrix_x4(cK + swz<KS>(key, chunk), b0, b1, b2, b3);
                     mma_16816<F16>(s[2 * np], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b0, b1);
                     mma_16816<F16>(s[2 * np + 1], qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], b2, b3);
                 }
             }
-            __syncwarp();  // every lane has read the K buffer
-            if (more) stage_chunk<D, CK>(sK, Kh, p.kv_row, col_next * CK, p.Nkv, lane);
-            cp_async_commit();
+            __syncwarp();  // every lane has read the K slot
+            if (more && lane == 0) copy_in(cK, &tmK, bK + slot * 8, key_in);
             // ---- online softmax ----
-            if (key0 + CK > p.Nkv) {  // ragged last chunk: keys at or beyond N_kv do not exist
+            if (st >= n_steps - SPE && last_key + CK > p.Nkv) {  // ragged last entry: keys at or beyond N_kv do not exist
 #pragma unroll
                 for (int n = 0; n < NT_S; ++n) {
-                    const int kc = key0 + n * 8 + 2 * t;
+                    const int kc = last_key + (st % SPE) * KS + n * 8 + 2 * t;
                     if (kc >= p.Nkv) s[n][0] = s[n][2] = -INFINITY;
                     if (kc + 1 >= p.Nkv) s[n][1] = s[n][3] = -INFINITY;
                 }
@@ -263,8 +277,8 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
                 }
             }
             // ---- O += P V ----
-            cp_async_wait<1>();  // V chunk j has landed (K chunk j+1 may still be in flight)
-            __syncwarp();
+            ok = mbar_wait_warp(bV + slot * 8, phase, abortp);
+            if (!ok) break;
 #pragma unroll
             for (int ks = 0; ks < KS_PV; ++ks) {
 #pragma unroll
@@ -273,17 +287,19 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
                     const int key = ks * 16 + (((lane >> 3) & 1) << 3) + (lane & 7);
                     const int chunk = nd * 2 + (lane >> 4);
                     uint32_t b0, b1, b2, b3;
-                    ldmatrix_x4_trans(sV + swz<D * 2>(key, chunk), b0, b1, b2, b3);
+                    ldmatrix_x4_trans(cV + swz<KS>(key, chunk), b0, b1, b2, b3);
                     mma_16816<F16>(o[2 * nd], pa[ks][0], pa[ks][1], pa[ks][2], pa[ks][3], b0, b1);
                     mma_16816<F16>(o[2 * nd + 1], pa[ks][0], pa[ks][1], pa[ks][2], pa[ks][3], b2, b3);
                 }
             }
-            __syncwarp();  // every lane has read the V buffer
-            if (more) stage_chunk<D, CK>(sV, Vh, p.kv_row, col_next * CK, p.Nkv, lane);
-            cp_async_commit();
-            col = col_next;
+            __syncwarp();  // every lane has read the V slot
+            if (more && lane == 0) copy_in(cV, &tmV, bV + slot * 8, key_in);
+            if (++slot == NST) {
+                slot = 0;
+                phase ^= 1u;
+            }
         }
-        cp_async_wait<0>();
+        if (!ok) break;
         // ---- epilogue: row sums over the four lanes of a row, normalise, store ----
         l_lo += __shfl_xor_sync(kFullMask, l_lo, 1);
         l_hi += __shfl_xor_sync(kFullMask, l_hi, 1);
@@ -301,6 +317,11 @@ __global__ void __launch_bounds__(kRbWarps * 32, 1) bsa_attention_rb_kernel(cons
             if (r_hi < p.N)
                 p.LSE[(long long)head * p.N + r_hi] = (l_hi > 0.f) ? fmaf(m_hi, 0.6931471805599453f, logf(l_hi)) : -INFINITY;
         }
+    }
+    if (!ok) {  // a wait ran out: copies in flight land before the CTA's shared memory goes away
+        if (lane == 0) atomicExch(&p.counters->status, (int)BSA_ERR_DEVICE_TIMEOUT);
+        const uint64_t t0 = globaltimer_ns();
+        while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
     }
 }
 
@@ -320,7 +341,13 @@ cudaError_t launch_rb_t(const ForwardArgs& a, const RbParams& p, cudaStream_t st
     long long want = ((long long)a.max_items + kRbWarps - 1) / kRbWarps;
     int grid = want < a.num_sms ? (int)want : a.num_sms;
     if (grid < 1) grid = 1;
-    bsa_attention_rb_kernel<D, CK, F16><<<grid, kRbWarps * 32, smem, stream>>>(p);
+    CUtensorMap tk, tv;
+    if (!encode_kv_map(&tk, a.K, a.g.N_kv, a.g.H, D, kRbStep<D, CK>, F16, a.nhd) ||
+        !encode_kv_map(&tv, a.V, a.g.N_kv, a.g.H, D, kRbStep<D, CK>, F16, a.nhd)) {
+        *err = "cuTensorMapEncodeTiled failed";
+        return cudaErrorInvalidValue;
+    }
+    bsa_attention_rb_kernel<D, CK, F16><<<grid, kRbWarps * 32, smem, stream>>>(tk, tv, p);
     count_launch();
     return cudaGetLastError();
 }
@@ -331,14 +358,12 @@ cudaError_t launch_rb(const ForwardArgs& a, const RbParams& p, cudaStream_t stre
 
 }  // namespace
 
-// Largest KV chunk (keys) the row-block kernel can stage for head dimension d.
+// Largest KV entry (keys) the row-block kernel takes for head dimension d.
 int rb_max_chunk(int d) { return kRbStageBytes / (d * 2); }
 
 cudaError_t launch_forward_rb(const ForwardArgs& a, cudaStream_t stream, const char** err_detail) {
     RbParams p;
     p.Q = reinterpret_cast<const __nv_bfloat16*>(a.Q);
-    p.K = reinterpret_cast<const __nv_bfloat16*>(a.K);
-    p.V = reinterpret_cast<const __nv_bfloat16*>(a.V);
     p.O = reinterpret_cast<__nv_bfloat16*>(a.O);
     p.LSE = a.LSE;
     p.items = a.items;
@@ -346,8 +371,6 @@ cudaError_t launch_forward_rb(const ForwardArgs& a, cudaStream_t stream, const c
     p.counters = a.counters;
     p.q_head = a.nhd ? (long long)a.d : (long long)a.g.N * a.d;
     p.q_row = a.nhd ? (long long)a.g.H * a.d : (long long)a.d;
-    p.kv_head = a.nhd ? (long long)a.d : (long long)a.g.N_kv * a.d;
-    p.kv_row = a.nhd ? (long long)a.g.H * a.d : (long long)a.d;
     p.N = (int32_t)a.g.N;
     p.Nkv = (int32_t)a.g.N_kv;
     p.scale_log2 = (float)(1.4426950408889634 / sqrt((double)a.d));

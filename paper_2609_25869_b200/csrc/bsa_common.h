@@ -1,5 +1,6 @@
 // Internal declarations shared by the planner, the attention kernels and the C ABI.
 #pragma once
+#include <cuda.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -126,6 +127,9 @@ cudaError_t launch_merge(const ForwardArgs& a, cudaStream_t stream);  // the Spl
 // Row-block kernel (bsa_attention_rb.cu): 16-row physical Q tiles on the register-level tensor instruction.
 constexpr int kKernelRowBlock = 5;
 cudaError_t launch_forward_rb(const ForwardArgs& a, cudaStream_t stream, const char** err_detail);
+// Tensor map of K or V as {64 columns, N rows, d/64 column groups, heads}: a copy brings box_rows whole rows, 128-byte
+// swizzle, 64-column halves one after the other (defined with the other tensor maps).
+bool encode_kv_map(CUtensorMap* m, const void* base, int64_t N, int heads, int d, int box_rows, bool f16, bool nhd);
 int rb_max_chunk(int d);  // largest T_KV (keys per staged chunk) for head dimension d
 // `stages` counts K buffers plus V buffers for the paired kernel (kernel 1), K = V ring depth for kernel 0
 int attention_max_stages(int d, int T_KV, int kernel);

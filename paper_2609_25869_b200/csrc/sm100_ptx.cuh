@@ -95,6 +95,14 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// The whole warp waits for one barrier phase: one test and one vote when the phase has completed, the bounded wait
+// otherwise.  The result is the same in every lane.  (With the wait's loop and its early return in front of the vote the
+// common case crossed a divergent region: about 2 % of the softmax warpgroups' time.)
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile uint32_t* abort_flag) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag));
+}
+
 // Bounded wait for two barriers.  Both are tested first, back to back, so that when both phases have completed the
 // thread pays one shared-memory round trip instead of two dependent ones.
 __device__ __forceinline__ bool mbar_wait2(uint32_t bar_a, uint32_t parity_a, uint32_t bar_b, uint32_t parity_b,
