@@ -344,10 +344,16 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
         BSA_CUDA(cudaMallocAsync(&p->arena2, arena2_have, stream), "arena2 (predicted)");
     }
     {
-        volatile unsigned* flag = &posted->seq;
+        volatile unsigned long long* words = posted->word;
+        auto all_here = [&]() {
+            for (int i = 0; i < 10; ++i)
+                if ((unsigned)(words[i] >> 32) != seq) return false;
+            return true;
+        };
+        auto value = [&](int i) { return (words[2 * i] & 0xffffffffull) | (words[2 * i + 1] << 32); };
         const double t_poll = now_us();
         bool arrived = true;
-        while (*flag != seq) {
+        while (!all_here()) {
             if (now_us() - t_poll > 1000.0) {
                 arrived = false;
                 break;
@@ -355,19 +361,19 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
         }
         if (!arrived) {  // a long queue in front of the kernel: wait for the stream instead of spinning on
             BSA_CUDA(cudaStreamSynchronize(stream), "stats sync");
-            if (*flag != seq) {
+            if (!all_here()) {
                 set_cuda_err(cudaErrorUnknown, "statistics were not posted");
                 free_plan(p);
                 return BSA_ERR_CUDA;
             }
         }
         std::atomic_thread_fence(std::memory_order_acquire);
-        p->hstats.nnz = posted->nnz;
-        p->hstats.in_runs = posted->in_runs;
-        p->hstats.max_row_nnz = posted->max_row_nnz;
+        p->hstats.nnz = value(0);
+        p->hstats.in_runs = value(1);
+        p->hstats.max_row_nnz = (unsigned)value(2);
         p->hstats.blocks_done = 0;
-        p->hstats.hash[0] = posted->hash[0];
-        p->hstats.hash[1] = posted->hash[1];
+        p->hstats.hash[0] = value(3);
+        p->hstats.hash[1] = value(4);
         acc_clean[p->device] = true;  // the kernel's last CTA left the accumulators at zero
     }
     const double t2 = now_us();

@@ -40,14 +40,13 @@ struct MaskStatsDev {
     unsigned int blocks_done;  // CTAs of the statistics kernel that have added their share (starts at zero)
     unsigned long long hash[2];  // 128-bit fingerprint of the activity pattern (only when asked for, else 0)
 };
-// The statistics as the kernel's last CTA posts them into pinned host memory; `seq` is written last.
+// The statistics as the kernel's last CTA posts them into pinned host memory: the 32-bit halves of MaskStatsDev, each in
+// a 64-bit word with the request's sequence number in its upper half.  A word is written in one piece, so the host can
+// tell for each by itself whether it has arrived and the kernel needs no fence between the values and a flag.
 struct MaskStatsHost {
-    unsigned long long nnz;
-    unsigned long long in_runs;
-    unsigned long long hash[2];
-    unsigned int max_row_nnz;
-    unsigned int seq;
+    unsigned long long word[10];
 };
+static_assert(sizeof(MaskStatsDev) == 40, "five 64-bit accumulators");
 struct PlanCountersDev {
     unsigned long long ntiles;       // physical tiles (a 256-row tile counts once)
     unsigned long long nslot_tiles;  // 128-row MMA tiles actually computed
