@@ -1349,7 +1349,13 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // active pairs 1.44 both times); (32,32) 22.3 -> 14.9 ms (2.53 -> 1.92); (128,64) fp16, 12 heads, 30 % 11.7 -> 10.4 ms.
 // A K tile takes G*d/64 copies (the MMA wants its rows 128 bytes x 1024 apart across entries), a V tile G (an entry's
 // 64-column halves lie together, the MMA's descriptor moves from entry to entry).
-// TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448; d = 64: S0 0, S1 128, O 256, Q 320 and 352, P0 384, P1 448.
+//
+// d = 64: two accumulators fit, so each softmax warpgroup has its own (and its own reference maximum): nothing is handed
+// from tile to tile, no shared-memory round trip and vote per tile, and the epilogue adds the two up with their weights.
+// Q then stays in shared memory, double-buffered (every TMEM column is taken; at d = 64 shared memory is half idle).
+// Builds in turn: 3600 x 1111 tokens, 16 heads, (64,32) fp16 29.5 -> 26.4 us; 32768 tokens, 16 heads, (16,64) as 64-key
+// entries 4.94 -> 4.73 ms; (256,256) 1.27 -> 1.25 ms; 2048 tokens, 2 heads 23.0 -> 22.5 us.
+// TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448; d = 64: S0 0, S1 128, O0 256, O1 320, P0 384, P1 448.
 // ==========================================================================================
 constexpr int kPpThreads = 512;
 constexpr int kPpTK = 128;  // keys of a tile
@@ -1414,11 +1420,11 @@ struct __align__(8) PpBarriers {
 // Tensor-memory columns of the ping-pong kernel.  Q is the A operand of Q K^T and lives in TMEM (D/2 columns).
 template <int D>
 struct PpCols {
-    static constexpr bool kTight = (D == 128);  // all 512 columns in use
-    static constexpr uint32_t kP0 = kColP0, kP1 = kTight ? kColP0 : kColP1;
-    static constexpr bool kOneP = (kP0 == kP1);
-    static constexpr int kQBuffers = kTight ? 1 : 2;
-    static constexpr uint32_t kQ0 = kTight ? 448 : 320, kQ1 = kTight ? 448 : 352;
+    static constexpr bool kOwnO = (D == 64);  // an accumulator per softmax warpgroup (then Q stays in shared memory)
+    static constexpr uint32_t kO0 = kColO, kO1 = kOwnO ? 320 : kColO;
+    static constexpr uint32_t kP0 = kColP0, kP1 = kOwnO ? kColP1 : kColP0;
+    static constexpr uint32_t kQ = 448;
+    static constexpr int kQBuffers = kOwnO ? 2 : 1;
 };
 
 // Tiles of a list of n entries, G entries to a tile (n <= 0: no tiles, or past the end of the list).
@@ -1449,11 +1455,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int GV_TILE = KV_TILE / G;
     constexpr int V_SUB = (G == 1) ? KV_SUB : GK * 128;  // a V tile holds its entries one after the other
     using Cols = PpCols<D>;
-    constexpr int NQT = Cols::kQBuffers;
+    constexpr int NQB = Cols::kQBuffers;
+    constexpr bool kOwnO = Cols::kOwnO;
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
     uint8_t* sQ = smem;                      // landing buffer of the next item's Q tile, which then moves to TMEM
-    uint8_t* sK = sQ + NSUB * Q_SUB;         // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
+    uint8_t* sK = sQ + NQB * NSUB * Q_SUB;   // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
     uint8_t* sV = sK + p.stages * KV_TILE;   // NSV V tiles (a V tile lives about two tiles longer, until its P V)
     __shared__ PpBarriers bars;
     // [publishing warpgroup][row]: the reference maximum after that warpgroup's latest tile.  One 32-bit word per
@@ -1482,7 +1489,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         mbar_init(smem_u32(&bars.q_full), 1);       // the Q tile has landed in shared memory
         mbar_init(smem_u32(&bars.q_drained), 128);  // epilogue threads: it has been read from there
         for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&bars.qt_full[b]), 128);  // epilogue threads: the Q tile is in TMEM
+            mbar_init(smem_u32(&bars.qt_full[b]), kOwnO ? 1 : 128);  // the Q tile is in place (TMEM: epilogue threads)
             mbar_init(smem_u32(&bars.qt_free[b]), 1);    // the item's last Q K^T has completed
         }
         mbar_init(smem_u32(&bars.o_free), 128);   // epilogue threads: accumulator drained
@@ -1529,11 +1536,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // =========================== epilogue warpgroup ===========================
         reg_dec<80>();
         const int tw = tid & 127;
-        const uint32_t t_o = tmem + ((uint32_t)((warp & 3) * 32) << 16) + kColO;
+        const uint32_t t_lane = tmem + ((uint32_t)((warp & 3) * 32) << 16);
         uint32_t itn = 0;  // non-empty items seen
+        uint32_t g_start = 0;  // running tile index at the start of the item
         bool ok = true;
         BSA_TRACE_DECL(tn);
-        // ---- Q tiles: TMA into shared memory one item ahead, then into TMEM through this warpgroup's registers ----
+        // ---- Q tiles: TMA into shared memory one item ahead, then (d = 128) into TMEM through this warpgroup's registers ----
         int kq = 0;       // round of the next Q tile to load
         uint32_t nq = 0;  // Q tiles loaded so far
         auto load_q = [&]() {  // lane 0 of the warpgroup's first warp issues; every thread follows the item list
@@ -1542,20 +1550,25 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (kq >= n_rounds) return;
                 w = load_item(p.items, cta_item_index(kq++, blockIdx.x, gridDim.x), n_items);
             } while (w.ntiles <= 0);
-            ++nq;
+            const uint32_t b = nq % NQB;
+            const uint32_t full = smem_u32(kOwnO ? &bars.qt_full[b] : &bars.q_full);
             if (tw == 0) {
-                mbar_arrive_expect_tx(smem_u32(&bars.q_full), NSUB * Q_SUB);
-                tma_load_4d(smem_u32(sQ), &tmQ, smem_u32(&bars.q_full), 0, w.q_tile * kTQ, 0, w.head);
+                // two buffers: the item before last has read this one long ago
+                if (kOwnO && !mbar_wait(smem_u32(&bars.qt_free[b]), ((nq >> 1) & 1) ^ 1, abortp)) ok = false;
+                if (ok) {
+                    mbar_arrive_expect_tx(full, NSUB * Q_SUB);
+                    tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, full, 0, w.q_tile * kTQ, 0, w.head);
+                }
             }
+            ++nq;
         };
         uint32_t sq = 0;  // Q tiles moved to TMEM
         auto stage_q = [&]() -> bool {
-            const uint32_t b = (NQT == 2) ? (sq & 1) : 0, use = (NQT == 2) ? (sq >> 1) : sq;
             bool good = mbar_wait(smem_u32(&bars.q_full), sq & 1, abortp);
-            good = good && mbar_wait(smem_u32(&bars.qt_free[b]), (use & 1) ^ 1, abortp);
+            good = good && mbar_wait(smem_u32(&bars.qt_free[0]), (sq & 1) ^ 1, abortp);
             if (!__all_sync(0xffffffffu, good)) return false;
             tc_fence_after();
-            const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (b ? Cols::kQ1 : Cols::kQ0);
+            const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + Cols::kQ;
 #pragma unroll 1
             for (int s = 0; s < NSUB; ++s) {  // 64 head-dimension columns: eight swizzled 16-byte chunks of this row
                 uint32_t v[32];
@@ -1569,7 +1582,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             mbar_arrive(smem_u32(&bars.q_drained));
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(smem_u32(&bars.qt_full[b]));
+            mbar_arrive(smem_u32(&bars.qt_full[0]));
             if (tw == 0) good = mbar_wait(smem_u32(&bars.q_drained), sq & 1, abortp);  // then the next Q tile may land
             if (!__all_sync(0xffffffffu, good)) return false;
             ++sq;
@@ -1593,14 +1606,28 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 continue;
             }
-            // the next item's Q tile goes to TMEM first (its Q K^T runs ahead of this item's softmax); with one TMEM
-            // buffer that waits for this item's last Q K^T, which comes well before its last P V
-            while (ok && nq > sq && sq <= itn + 1) ok = stage_q();
+            // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); d = 128: the one TMEM buffer is
+            // free after this item's last Q K^T, which comes well before its last P V
+            if constexpr (kOwnO) {
+                load_q();
+                ok = __all_sync(0xffffffffu, ok);
+            } else {
+                while (ok && nq > sq && sq <= itn + 1) ok = stage_q();
+            }
             if (!ok) break;
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
             if (!ok) break;
-            const float l_tot = lfin[0][tw] + lfin[1][tw];
-            const float m_final = mfin[tw];
+            float l_tot, m_final, w0 = 1.f, w1 = 1.f;  // weights of the two accumulators
+            if constexpr (kOwnO) {
+                const float m0 = __uint_as_float(mref[0][tw]), m1 = __uint_as_float(mref[1][tw]);
+                m_final = fmaxf(m0, m1);
+                w0 = (m0 == -INFINITY) ? 0.f : ex2_approx(m0 - m_final);
+                w1 = (m1 == -INFINITY) ? 0.f : ex2_approx(m1 - m_final);
+                l_tot = lfin[0][tw] * w0 + lfin[1][tw] * w1;
+            } else {
+                l_tot = lfin[0][tw] + lfin[1][tw];
+                m_final = mfin[tw];
+            }
             mbar_arrive(smem_u32(&bars.e_taken));
             const float inv_l = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
             const float lse = (l_tot > 0.f) ? fmaf(m_final, 0.6931471805599453f, logf(l_tot)) : -INFINITY;
@@ -1612,12 +1639,31 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             ++itn;
             __nv_bfloat16* orow = p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row);
             float* wrow = p.ws_O + ((size_t)it.ws_slot * kTQ + tw) * D;
+            constexpr int CW = kOwnO ? 16 : 32;  // columns at a time
+            const int n_tiles = tiles_of<G>(it.ntiles);
+            const uint32_t first = g_start & 1u;  // accumulator of the item's first tile; the other one is stale if n_tiles == 1
+            g_start += (uint32_t)n_tiles;
+            const float sa = inv_l * (first ? w1 : w0), sb = inv_l * (first ? w0 : w1);
 #pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
-            for (int c = 0; c < D / 32; ++c) {
-                uint32_t o[32];
-                tmem_ld32(t_o + c * 32, o);
-                tc_wait_ld();
-                if (c == D / 32 - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
+            for (int c = 0; c < D / CW; ++c) {
+                uint32_t o[CW];
+                if constexpr (kOwnO) {
+                    uint32_t ob[CW];
+                    tmem_ld16(t_lane + (first ? Cols::kO1 : Cols::kO0) + c * CW, o);
+                    tmem_ld16(t_lane + (first ? Cols::kO0 : Cols::kO1) + c * CW, ob);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < CW; ++e) {
+                        const float a = __uint_as_float(o[e]) * sa;
+                        o[e] = __float_as_uint(n_tiles > 1 ? fmaf(__uint_as_float(ob[e]), sb, a) : a);
+                    }
+                } else {
+                    tmem_ld32(t_lane + kColO + c * CW, o);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int e = 0; e < CW; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * sa);
+                }
+                if (c == D / CW - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
                     tc_fence_before();
                     mbar_arrive(smem_u32(&bars.o_free));
                     if (lane == 0) BSA_TRACE_POINT(11, tn, 33);
@@ -1625,23 +1671,17 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (it.nparts == 1) {
                     if (row_ok) {  // 32-byte stores: every thread fills whole 32-byte sectors of its own row
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) {
+                        for (int q = 0; q < CW / 16; ++q) {
                             uint32_t v[8];
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
-                                v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]) * inv_l,
-                                                   __uint_as_float(o[q * 16 + 2 * e + 1]) * inv_l);
-                            st_global_v8(orow + c * 32 + q * 16, v);
+                                v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]), __uint_as_float(o[q * 16 + 2 * e + 1]));
+                            st_global_v8(orow + c * CW + q * 16, v);
                         }
                     }
                 } else {  // Split-K partial: normalised fp32 rows in the workspace
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        uint32_t v[8];
-#pragma unroll
-                        for (int e = 0; e < 8; ++e) v[e] = __float_as_uint(__uint_as_float(o[q * 8 + e]) * inv_l);
-                        st_global_v8(wrow + c * 32 + q * 8, v);
-                    }
+                    for (int q = 0; q < CW / 8; ++q) st_global_v8(wrow + c * CW + q * 8, o + q * 8);
                 }
             }
             if (it.nparts == 1) {
@@ -1734,6 +1774,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         } else if (warp == 9 && lane == 0) {
             // =========================== Q K^T issuer ===========================
             constexpr uint32_t idesc_qk = make_idesc_f32(kTQ, TK, 0, 0, F16);
+            const uint64_t descQ0 = make_smem_desc_sw128(smem_u32(sQ), 16, 1024);
             const uint64_t descK = make_smem_desc_sw128(smem_u32(sK), 16, 1024);
             RingPos ring;  // K ring position of the tile being issued
             uint32_t itq = 0, g = 0;
@@ -1745,10 +1786,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const int n = n_next;
                 n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
                 if (n <= 0) continue;
-                const uint32_t qb = (NQT == 2) ? (itq & 1) : 0;  // this item's Q buffer in TMEM
-                ok = mbar_wait(smem_u32(&bars.qt_full[qb]), ((NQT == 2) ? (itq >> 1) : itq) & 1, abortp);
+                const uint32_t qb = itq % NQB;  // this item's Q buffer
+                ok = mbar_wait(smem_u32(&bars.qt_full[qb]), (itq / NQB) & 1, abortp);
                 if (!ok) break;
-                const uint32_t a_q = tmem + (qb ? Cols::kQ1 : Cols::kQ0);
+                const uint64_t descQ = descQ0 + (uint64_t)((qb * NSUB * Q_SUB) >> 4);
                 for (int j = 0; j < n; ++j, ring.advance(NSK)) {
                     const uint32_t gs = g + j;
                     const int stage = ring.stage;
@@ -1767,7 +1808,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                     for (int k = 0; k < D / 16; ++k) {
                         const uint64_t b = descK + (uint64_t)((stage * KV_TILE + (k / 4) * KV_SUB + (k % 4) * 32) >> 4);
-                        mma_ts(d_s, a_q + k * 8, b, idesc_qk, k > 0);
+                        if constexpr (kOwnO)
+                            mma_ss(d_s, descQ + (uint64_t)(((k / 4) * Q_SUB + (k % 4) * 32) >> 4), b, idesc_qk, k > 0);
+                        else
+                            mma_ts(d_s, tmem + Cols::kQ + k * 8, b, idesc_qk, k > 0);
                     }
                     mma_commit(smem_u32(&bars.k_empty[stage]));
                     mma_commit(smem_u32(&bars.s_full[sb]));
@@ -1816,11 +1860,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     BSA_TRACE_POINT(10, tn, 3);
 
                     tc_fence_after();
-                    const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0);
+                    const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0), d_o = tmem + (sb ? Cols::kO1 : Cols::kO0);
 #pragma unroll
                     for (int k = 0; k < TK / 16; ++k) {
                         const uint64_t b = descV + (uint64_t)((stage * KV_TILE + (k / (GK / 16)) * GV_TILE + (k % (GK / 16)) * 2048) >> 4);
-                        mma_ts(tmem + kColO, a_p + k * 8, b, idesc_pv, (j > 0 || k > 0) ? 1u : 0u);
+                        mma_ts(d_o, a_p + k * 8, b, idesc_pv, (j > (kOwnO ? 1 : 0) || k > 0) ? 1u : 0u);
                     }
                     mma_commit(smem_u32(&bars.v_empty[stage]));
                     mma_commit(smem_u32(&bars.pv_done[sb]));
@@ -1847,7 +1891,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const uint32_t lane_base = (uint32_t)((warp & 3) * 32) << 16;
         const uint32_t t_s = tmem + lane_base + (x ? kColS1 : kColS0);
         const uint32_t t_p = tmem + lane_base + (x ? Cols::kP1 : Cols::kP0);
-        const uint32_t t_o = tmem + lane_base + kColO;
+        const uint32_t t_o = tmem + lane_base + (x ? Cols::kO1 : Cols::kO0);
         uint32_t g = 0;          // running tile index at the start of the current item (all warpgroups agree)
         uint32_t itn = 0;        // non-empty items finished
         bool ok = true;
@@ -1951,7 +1995,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
                 // The previous tile's reference has normally been published by now: its slot is read here and the
                 // word checked after the max phase, so that the shared-memory round trip overlaps that phase.
-                const uint32_t ref_word = *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]);
+                uint32_t ref_word = 0;
+                if constexpr (!kOwnO) ref_word = *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]);
                 if (need_mask) {
                     // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
                     // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
@@ -1978,44 +2023,48 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #ifdef BSA_TRACE
                 if (lane == 0 && mx2 != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 17);
 #endif
-                // ---- reference maximum handed over from the previous tile (other warpgroup) ----
-                float m_prev = -INFINITY;
-                if (gs > 0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
-                    float m_taken;
-                    if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) + 1) & 3u))) {
-                        m_taken = __uint_as_float(ref_word & ~3u);
-                    } else {
-                        ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
-                        if (!ok) break;
+                if constexpr (!kOwnO) {
+                    // ---- reference maximum handed over from the previous tile (other warpgroup) ----
+                    float m_prev = -INFINITY;
+                    if (gs > 0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
+                        float m_taken;
+                        if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) + 1) & 3u))) {
+                            m_taken = __uint_as_float(ref_word & ~3u);
+                        } else {
+                            ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
+                            if (!ok) break;
+                        }
+                        if (j > 0) m_prev = m_taken;  // the previous tile belongs to this item
                     }
-                    if (j > 0) m_prev = m_taken;  // the previous tile belongs to this item
-                }
 #ifdef BSA_PHASES
-                {
-                    float f0_ = mx2, f1_ = m_prev;  // real instructions that read the values: the clock is read after them
-                    asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+f"(f1_));
-                }
+                    {
+                        float f0_ = mx2, f1_ = m_prev;  // real instructions that read the values: the clock is read after them
+                        asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+f"(f1_));
+                    }
 #endif
-                BSA_PH(2);
+                    BSA_PH(2);
 #ifdef BSA_TRACE
-                if (lane == 0 && m_prev != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 18);
+                    if (lane == 0 && m_prev != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 18);
 #endif
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 12);
-                if (m_prev != m_know) {  // the other warpgroup moved the reference since this thread last looked
-                    l *= ex2_approx(m_know - m_prev);  // m_know = -inf only while l = 0
-                    m_know = m_prev;
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 12);
+                    if (m_prev != m_know) {  // the other warpgroup moved the reference since this thread last looked
+                        l *= ex2_approx(m_know - m_prev);  // m_know = -inf only while l = 0
+                        m_know = m_prev;
+                    }
                 }
                 float alpha = 1.f;
                 bool rescale = false;
                 if (mx2 > m_know + kRescaleThreshold) {
-                    const float m_new = __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
+                    const float m_new = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
                     alpha = ex2_approx(m_know - m_new);
-                    rescale = (j > 0) && (m_know != -INFINITY);
+                    rescale = (j > (kOwnO ? 1 : 0)) && (m_know != -INFINITY);
                     l *= alpha;
                     m_know = m_new;
                 }
-                // publish: the next tile's warpgroup may take its decision
-                *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) + 1) & 3u);
+                if constexpr (!kOwnO) {
+                    // publish: the next tile's warpgroup may take its decision
+                    *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) + 1) & 3u);
+                }
                 BSA_PH(3);
                 const float neg_m = (m_know == -INFINITY) ? 0.f : -m_know;
                 const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
@@ -2056,15 +2105,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
                 if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
                 if (!kStoreInLoop) {
-                    if (Cols::kOneP) {  // the P tile before this one (other warpgroup's) must have been consumed
-                        if (gs >= 1) {
-                            ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
-                            if (!ok) break;
-                            tc_fence_after();
-                        }
-                    } else if (gs >= 2) {
-                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
+                    if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
                         if (!ok) break;
+                        tc_fence_after();
                     }
                     BSA_PH(5);
                     if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
@@ -2073,10 +2117,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 // ---- the reference moved at this tile: rescale the running output (after the P V of tile gs-1) ----
                 if (j > 0 && __any_sync(0xffffffffu, rescale)) {
-                    const uint32_t gp = gs - 1;
-                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), (gp >> 1) & 1, abortp);
-                    if (!ok) break;
-                    tc_fence_after();
+                    if constexpr (!kOwnO) {  // (an accumulator of its own: tile gs-2 has been waited for above)
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
 #pragma unroll 1  // rare path: kept small
                     for (int c = 0; c < D / 32; ++c) {
                         uint32_t o[32];
@@ -2103,7 +2148,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const uint32_t gl = g + n - 1;  // last tile of the item
                 const bool owner = (gl & 1) == (uint32_t)x;
                 float m_final = m_know;
-                if (!owner) {  // the other warpgroup took the last tile: its publish holds the final reference
+                if (!kOwnO && !owner) {  // the other warpgroup took the last tile: its publish holds the final reference
                     ok = __all_sync(0xffffffffu,
                                     take_reference(gl, *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]), m_final));
                     if (!ok) break;
@@ -2113,7 +2158,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
                 if (!ok) break;
                 lfin[x][tw] = l;
-                if (owner) mfin[tw] = m_final;
+                if (kOwnO) mref[x][tw] = __float_as_uint(m_know);
+                else if (owner) mfin[tw] = m_final;
                 mbar_arrive(smem_u32(&bars.e_ready));
                 ++itn;
                 if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
@@ -2350,7 +2396,7 @@ bool encode_kv_map(CUtensorMap* m, const void* base, int64_t N, int heads, int d
 static int static_smem_bytes(int kernel) { return (kernel == 2 || kernel == 4) ? 3072 : 1024; }
 
 static int kv_buffers_that_fit(int d, int T_KV, int kernel) {
-    const int q = (kernel == 1 ? 2 : 1) * kTQ * d * 2;  // kernel 1: two Q slots
+    const int q = (kernel == 1 || (kernel == 4 && d == 64) ? 2 : 1) * kTQ * d * 2;  // two Q slots (kernel 1) or buffers
     const int kv = T_KV * d * 2;
     return (232448 - static_smem_bytes(kernel) - q) / kv;
 }
@@ -2381,7 +2427,7 @@ int attention_max_stages(int d, int T_KV, int kernel) {
 
 int attention_smem_bytes(int d, int T_KV, int stages, int kernel) {
     if (kernel == 4) T_KV = kPpTK;
-    const int q = (kernel == 1 ? 2 : 1) * kTQ * d * 2;
+    const int q = (kernel == 1 || (kernel == 4 && d == 64) ? 2 : 1) * kTQ * d * 2;
     const int kv = T_KV * d * 2;
     int need = q + ((kernel == 1 || kernel == 4) ? stages : 2 * stages) * kv;
     // more than half of the SM's shared memory, so exactly one CTA (and one 512-column TMEM allocation) per SM

@@ -23,14 +23,28 @@ def test_gathered_tiles_match_the_oracle(B_Q, B_KV, N, N_kv, d, dtype, plan_id):
     Hh.run_request(I.Request("gather", H, N, d, B_Q, B_KV, M, qkv_seed=N, N_kv=N_kv, dtype=dtype), plan_id=plan_id)
 
 
-@pytest.mark.parametrize("B,plan_id", [(32, 39), (64, 23)])
-def test_list_lengths_around_whole_tiles(B, plan_id):
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("B,plan_id", [(32, 39), (64, 23), (128, 22)])
+def test_list_lengths_around_whole_tiles(B, plan_id, d):
     """Query block i has i + 1 active key blocks: lists of 1, 2, ... entries, each with the ragged last block or not."""
     n = 13
     M = np.zeros((2, n, n), np.uint8)
     for i in range(n):
         M[0, i, n - 1 - i:] = 1
         M[1, i, :i + 1] = 1
-    Hh.run_request(I.Request("lengths", 2, n * B - 5, 128, B, B, M, qkv_seed=B), plan_id=plan_id)
+    Hh.run_request(I.Request("lengths", 2, n * B - 5, d, B, B, M, qkv_seed=B), plan_id=plan_id)
     # 128-row query blocks: every list length belongs to one work item
-    Hh.run_request(I.Request("lengths", 2, n * 128, 128, 128, B, M, qkv_seed=B + 1, N_kv=n * B - 5), plan_id=plan_id)
+    Hh.run_request(I.Request("lengths", 2, n * 128, d, 128, B, M, qkv_seed=B + 1, N_kv=n * B - 5), plan_id=plan_id)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_rows_that_only_every_other_tile_reaches(d):
+    """Two row blocks of one work item whose tiles alternate: each of the two softmax warpgroups sees only masked tiles
+    for half of its rows, in lists of two tiles and more."""
+    M = np.zeros((2, 6, 9), np.uint8)
+    M[0, 0::2, 0::2] = 1
+    M[0, 1::2, 1::2] = 1
+    M[1, 0, 0] = M[1, 1, 1] = M[1, 2, 3] = M[1, 3, 8] = M[1, 5, 8] = 1
+    req = I.Request("alternating", 2, 6 * 64, d, 64, 128, M, qkv_seed=3, N_kv=9 * 128 - 40)
+    for plan_id in (22, 24):
+        Hh.run_request(req, plan_id=plan_id)
