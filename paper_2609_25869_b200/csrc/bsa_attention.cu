@@ -82,6 +82,7 @@ struct AttnParams {
     float* ws_LSE;
     unsigned long long full_member;
     int64_t o_head, o_row;  // element strides of O (and of Q) between heads and between token rows
+    int32_t o_wide;         // O lies on a 32-byte boundary (16 bytes are all that the caller promises)
     int32_t N;    // query tokens per head
     int32_t Nkv;  // key/value tokens per head
     int32_t lgBQ;   // log2(B_Q) when B_Q < 128, else 31 (row >> 31 == 0)
@@ -1676,7 +1677,13 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
                                 v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]), __uint_as_float(o[q * 16 + 2 * e + 1]));
-                            st_global_v8(orow + c * CW + q * 16, v);
+                            if (p.o_wide) {
+                                st_global_v8(orow + c * CW + q * 16, v);
+                            } else {
+                                uint4* dst = reinterpret_cast<uint4*>(orow + c * CW + q * 16);
+                                dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                                dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                            }
                         }
                     }
                 } else {  // Split-K partial: normalised fp32 rows in the workspace
@@ -2468,6 +2475,7 @@ cudaError_t launch_forward(const ForwardArgs& a, cudaStream_t stream, const char
     p.N = (int32_t)a.g.N;
     p.Nkv = (int32_t)a.g.N_kv;
     p.o_head = a.nhd ? (int64_t)a.d : (int64_t)a.g.N * a.d;
+    p.o_wide = (reinterpret_cast<uintptr_t>(a.O) & 31) == 0;
     p.o_row = a.nhd ? (int64_t)a.g.H * a.d : (int64_t)a.d;
     p.lgBQ = (a.g.sQ128 > 1) ? a.g.lgBQ : 31;
     p.lgBKV = (a.g.sK > 1) ? a.g.lgBKV : 31;
