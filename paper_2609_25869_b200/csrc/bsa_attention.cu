@@ -1618,13 +1618,17 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if (!ok) break;
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
             if (!ok) break;
-            float l_tot, m_final, w0 = 1.f, w1 = 1.f;  // weights of the two accumulators
+            // d = 64: weights of the accumulator of the item's first tile (a) and of the other one (b).  Which warpgroup took
+            // the first tile follows from the tiles this CTA had before, so everything below goes by a and b and not by
+            // warpgroup: an item's bits are the same wherever it stands in a CTA's list.
+            const uint32_t first = g_start & 1u;
+            float l_tot, m_final, wa = 1.f, wb = 1.f;
             if constexpr (kOwnO) {
-                const float m0 = __uint_as_float(mref[0][tw]), m1 = __uint_as_float(mref[1][tw]);
-                m_final = fmaxf(m0, m1);
-                w0 = (m0 == -INFINITY) ? 0.f : ex2_approx(m0 - m_final);
-                w1 = (m1 == -INFINITY) ? 0.f : ex2_approx(m1 - m_final);
-                l_tot = lfin[0][tw] * w0 + lfin[1][tw] * w1;
+                const float ma = __uint_as_float(mref[first][tw]), mb = __uint_as_float(mref[first ^ 1u][tw]);
+                m_final = fmaxf(ma, mb);
+                wa = (ma == -INFINITY) ? 0.f : ex2_approx(ma - m_final);
+                wb = (mb == -INFINITY) ? 0.f : ex2_approx(mb - m_final);
+                l_tot = fmaf(lfin[first ^ 1u][tw], wb, lfin[first][tw] * wa);
             } else {
                 l_tot = lfin[0][tw] + lfin[1][tw];
                 m_final = mfin[tw];
@@ -1641,10 +1645,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             __nv_bfloat16* orow = p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row);
             float* wrow = p.ws_O + ((size_t)it.ws_slot * kTQ + tw) * D;
             constexpr int CW = kOwnO ? 16 : 32;  // columns at a time
-            const int n_tiles = tiles_of<G>(it.ntiles);
-            const uint32_t first = g_start & 1u;  // accumulator of the item's first tile; the other one is stale if n_tiles == 1
+            const int n_tiles = tiles_of<G>(it.ntiles);  // 1: the other accumulator is stale
             g_start += (uint32_t)n_tiles;
-            const float sa = inv_l * (first ? w1 : w0), sb = inv_l * (first ? w0 : w1);
+            const float sa = inv_l * wa, sb = inv_l * wb;
 #pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
             for (int c = 0; c < D / CW; ++c) {
                 uint32_t o[CW];
