@@ -83,6 +83,10 @@ struct bsa_plan {
     SplitRow* split_rows;
     int64_t tile_cap;
     int64_t max_items;
+    // Fewer than eight 128-key tiles per work item on average: where the ping-pong kernel keeps Q follows from it (d = 128,
+    // measured there).  Exact where no dimension is Coarsened; a Coarsened list is taken to be that of independent blocks, at
+    // most the true length's multiple by the blocks per tile, on a line where the two forms are within 2 % of each other.
+    int32_t short_lists;
     // Split-K workspace
     float* ws_O;
     float* ws_LSE;
@@ -449,6 +453,11 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
     const int pmax = p->desc.split_pmax < 1 ? 1 : p->desc.split_pmax;
     const int64_t trows = (int64_t)heads * g.nQt;
     p->max_items = trows * pmax;
+    {
+        const double entries = (double)g.nKt * (1.0 - pow(1.0 - density, (double)(g.sQ * g.sK)));
+        const double parts = pmax > 1 ? fmin((double)pmax, fmax(1.0, entries / p->desc.split_tau)) : 1.0;
+        p->short_lists = entries * p->desc.T_KV < 8.0 * 128.0 * parts;
+    }
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
     const size_t o_col = early_fill ? 0 : take(sizeof(int32_t) * (size_t)(nnz_i + 1));
@@ -640,6 +649,7 @@ static void fill_forward_args(const bsa_plan_t* p, const void* Q, const void* K,
     a.stages = p->stages;
     a.kernel = p->desc.kernel;
     a.has_split = p->desc.split_pmax > 1;
+    a.short_lists = p->short_lists;
     a.max_items = (int32_t)(p->max_items < (1 << 30) ? p->max_items : (1 << 30));
     a.max_split_rows = p->g.H * p->g.nQt * p->g.slots;
     a.num_sms = p->num_sms;

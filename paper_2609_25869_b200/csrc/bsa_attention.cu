@@ -1316,15 +1316,15 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // ==========================================================================================
 // Ping-pong kernel: one 128-row Q tile per CTA, TWO softmax warpgroups that take alternate KV
 // tiles (warpgroup x owns the tiles whose running index has parity x, and with them S buffer x
-// and P buffer x).  While one warpgroup is in its exponential phase the other loads its scores,
-// finds its row maxima and waits for nothing but the previous tile's reference maximum, so the
-// XU pipe and the tensor pipe both stay fed.  One O accumulator is shared: both warpgroups
-// follow the SAME reference maximum per row, handed from tile to tile through shared memory
-// (`mref`, one float per row, published right after a tile's max phase).  Each warpgroup keeps a
-// partial row sum, converted whenever the reference it last saw has moved.  P has its own TMEM
-// columns, so S[x] is free again as soon as warpgroup x has read it into registers (`s_free`).
+// at d = 64 P buffer x).  While one warpgroup is in its exponential phase the other loads its scores
+// and finds its row maxima, so the XU pipe and the tensor pipe both stay fed.  At d = 128 one O
+// accumulator is shared: both warpgroups follow the SAME reference maximum per row, handed from tile
+// to tile through shared memory (`mref`, one word per row, published right after a tile's max phase),
+// and each keeps a partial row sum, converted whenever the reference it last saw has moved.  At d = 64
+// each has an accumulator and a reference of its own (below).  P has its own TMEM columns, so S[x] is
+// free again as soon as warpgroup x has read it into registers (`s_free`).
 // A third warpgroup owns the epilogue: at the end of a work item the softmax warpgroups only hand
-// over their row sums (expressed in the item's final reference) and move straight on to the next
+// over their row sums and move straight on to the next
 // item's tiles; the epilogue warpgroup waits for the item's last P V, drains the accumulator,
 // normalises and stores, and releases the accumulator for the next item's first P V, which cannot
 // be issued before that item's first softmax tile is done anyway.
@@ -1333,14 +1333,18 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // Registers (setmaxnreg): softmax 192, epilogue 80, producers and issuers 48 per thread; the sum over the CTA,
 // 256*192 + 128*80 + 128*48 = 65536, is exactly the launch allocation of 512 threads x 128.
 //
-// Q K^T takes Q, its A operand, from TMEM: a 128x128x16 MMA with both operands in shared memory reads the full
-// 128 B/clk for as long as it runs, so per 128-key tile (d = 128) 160 KB went through shared memory (Q and K 64, V 32,
-// the two TMA tiles 64); now 128 KB.  The epilogue warpgroup, idle for most of an item, moves the next item's Q tile
-// from the buffer it lands in to TMEM.  With all columns taken at d = 128 the two warpgroups share one P buffer: tile
-// j's P V has long read it when tile j+1 stores its P.  Together with the warp-uniform waits (mbar_wait_warp) measured
-// on one GPU, the two builds in turn: 16384 tokens, 8 heads, d = 128, (128,128) blocks 177.8 -> 173.2 us; 115200
-// tokens, 24 heads 14.56 -> 14.26 ms (global order); 32768 tokens, 16 heads, d = 64, (256,256) 1355 -> 1307 us.  These
-// launches run at the 1 kW power cap (1.3-1.9 GHz of 1.965), so less traffic shows as a higher clock.
+// Where Q K^T reads Q, its A operand, at d = 128.  From TMEM on long lists: a 128x128x16 MMA with both operands in shared
+// memory reads the full 128 B/clk for as long as it runs, so per 128-key tile 160 KB would go through shared memory (Q and
+// K 64, V 32, the two TMA tiles 64) instead of 128.  The epilogue warpgroup, idle for most of a long item, moves the next
+// item's Q tile from the buffer it lands in to TMEM.  With all columns taken the two warpgroups share one P buffer: tile
+// j's P V has long read it when tile j+1 stores its P.  Together with the warp-uniform waits (mbar_wait_warp), builds in
+// turn: 16384 tokens, 8 heads, (128,128) blocks, 19 tiles per item 177.8 -> 173.2 us.
+// From shared memory on short lists, where the way through the epilogue warpgroup lies on every item's path: two Q tiles
+// (the V ring gives up one of its four), loaded by the K producer.  Forward at 32768 tokens, 8 heads, n tiles per item,
+// TMEM / shared memory in us: n = 1 46.8 / 41.4, 2 55.4 / 52.1, 3 68.3 / 66.0, 4 81.3 / 79.7, 6 107.6 / 106.1; at 16384
+// tokens 8 67.5 / 67.5, 12 93.4 / 93.9.  Hence shared memory below eight tiles per item on average (bsa_plan::short_lists).
+// Two kernels and not a flag in one: what an item pays at its boundary is mostly instruction fetch, and the softmax code
+// has no register to spare (one kernel with both bodies was 1-2 % slower on long lists).
 //
 // G: a 128-key tile is made up of G entries of the plan's tile list (T_KV = 128 / G keys each), whichever they are: the
 // producers copy them one by one, and a 128-row, 128-column MMA works on a tile without gaps.  G = 1 where the logical
@@ -1353,10 +1357,10 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 //
 // d = 64: two accumulators fit, so each softmax warpgroup has its own (and its own reference maximum): nothing is handed
 // from tile to tile, no shared-memory round trip and vote per tile, and the epilogue adds the two up with their weights.
-// Q then stays in shared memory, double-buffered (every TMEM column is taken; at d = 64 shared memory is half idle).
+// Q always stays in shared memory, double-buffered (every TMEM column is taken; at d = 64 shared memory is half idle).
 // Builds in turn: 3600 x 1111 tokens, 16 heads, (64,32) fp16 29.5 -> 26.4 us; 32768 tokens, 16 heads, (16,64) as 64-key
 // entries 4.94 -> 4.73 ms; (256,256) 1.27 -> 1.25 ms; 2048 tokens, 2 heads 23.0 -> 22.5 us.
-// TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448; d = 64: S0 0, S1 128, O0 256, O1 320, P0 384, P1 448.
+// TMEM columns, d = 128: S0 0, S1 128, O 256, P 384, Q 448 (or unused); d = 64: S0 0, S1 128, O0 256, O1 320, P0 384, P1 448.
 // ==========================================================================================
 constexpr int kPpThreads = 512;
 constexpr int kPpTK = 128;  // keys of a tile
@@ -1413,19 +1417,18 @@ struct RingPos {
 };
 
 struct __align__(8) PpBarriers {
-    uint64_t q_full, q_drained, qt_full[2], qt_free[2], o_free, o_full, e_ready, e_taken;
+    uint64_t q_full[2], qt_full, q_free, q_drained, o_free, o_full, e_ready, e_taken;
     uint64_t k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2];
 };
 
-// Tensor-memory columns of the ping-pong kernel.  Q is the A operand of Q K^T and lives in TMEM (D/2 columns).
+// Tensor-memory columns of the ping-pong kernel (Q's are in use only where Q K^T reads it from there).
 template <int D>
 struct PpCols {
-    static constexpr bool kOwnO = (D == 64);  // an accumulator per softmax warpgroup (then Q stays in shared memory)
+    static constexpr bool kOwnO = (D == 64);  // an accumulator per softmax warpgroup
     static constexpr uint32_t kO0 = kColO, kO1 = kOwnO ? 320 : kColO;
     static constexpr uint32_t kP0 = kColP0, kP1 = kOwnO ? kColP1 : kColP0;
     static constexpr uint32_t kQ = 448;
-    static constexpr int kQBuffers = kOwnO ? 2 : 1;
 };
 
 // Tiles of a list of n entries, G entries to a tile (n <= 0: no tiles, or past the end of the list).
@@ -1443,7 +1446,7 @@ struct TileKeys {
     }
 };
 
-template <int D, bool F16, int G>
+template <int D, bool F16, int G, bool kSmemQ>
 __global__ void __launch_bounds__(kPpThreads, 1)
 bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -1456,24 +1459,28 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int GV_TILE = KV_TILE / G;
     constexpr int V_SUB = (G == 1) ? KV_SUB : GK * 128;  // a V tile holds its entries one after the other
     using Cols = PpCols<D>;
-    constexpr int NQB = Cols::kQBuffers;
     constexpr bool kOwnO = Cols::kOwnO;
+    static_assert(!kOwnO || kSmemQ, "d = 64 has no tensor-memory columns left for Q");
+    static_assert(kOwnO || NSUB * Q_SUB == KV_TILE, "at d = 128 the second Q tile takes the place of a V tile");
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
-    uint8_t* sQ = smem;                      // landing buffer of the next item's Q tile, which then moves to TMEM
-    uint8_t* sK = sQ + NQB * NSUB * Q_SUB;   // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
-    uint8_t* sV = sK + p.stages * KV_TILE;   // NSV V tiles (a V tile lives about two tiles longer, until its P V)
+    const int NSK = p.stages, NSV = p.stages_v - (!kOwnO && kSmemQ ? 1 : 0);
+    uint8_t* sQ = smem;                                      // two Q tiles, or the landing buffer of the next one
+    uint8_t* sK = sQ + (kSmemQ ? 2 : 1) * (NSUB * Q_SUB);    // NSK K tiles (a K tile lives from its load to the end of its Q K^T)
+    uint8_t* sV = sK + NSK * KV_TILE;                        // NSV V tiles (a V tile lives about two tiles longer, until its P V)
     __shared__ PpBarriers bars;
     // [publishing warpgroup][row]: the reference maximum after that warpgroup's latest tile.  One 32-bit word per
     // row carries value and sequence together: reference values keep their two lowest mantissa bits clear, and
     // the word's two low bits hold (publish index + 1) mod 4, so the reader of the next tile (always the same
     // row's thread of the other warpgroup, which consumes every publish in order) needs one shared-memory
     // read, with no barrier in front of it, to know whether the value it got is the one it waits for.
+    // (d = 64: each warpgroup's own reference at the end of an item, plain.)
     __shared__ uint32_t mref[2][kTQ];
-    __shared__ float lfin[2][kTQ];   // [warpgroup][row]: an item's partial row sums in its final reference
-    __shared__ float mfin[kTQ];      // the item's final reference maximum (log2 domain) per row
+    __shared__ float lfin[2][kTQ];   // [warpgroup][row]: an item's partial row sums (d = 128: in its final reference)
+    __shared__ float mfin[kTQ];      // d = 128: the item's final reference maximum (log2 domain) per row
     __shared__ uint32_t tmem_base_s;
     __shared__ uint32_t abort_flag;
+
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 #ifdef BSA_TRACE
@@ -1483,16 +1490,13 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         if (tid == 0) atomicExch(&p.counters->status, (int)BSA_ERR_CUDA);
         return;
     }
-    const int NSK = p.stages, NSV = p.stages_v;
 
     if (tid == 0) {
         abort_flag = 0;
-        mbar_init(smem_u32(&bars.q_full), 1);       // the Q tile has landed in shared memory
-        mbar_init(smem_u32(&bars.q_drained), 128);  // epilogue threads: it has been read from there
-        for (int b = 0; b < 2; ++b) {
-            mbar_init(smem_u32(&bars.qt_full[b]), kOwnO ? 1 : 128);  // the Q tile is in place (TMEM: epilogue threads)
-            mbar_init(smem_u32(&bars.qt_free[b]), 1);    // the item's last Q K^T has completed
-        }
+        for (int b = 0; b < 2; ++b) mbar_init(smem_u32(&bars.q_full[b]), 1);  // the Q tile has landed in shared memory
+        mbar_init(smem_u32(&bars.qt_full), 128);    // epilogue threads: the Q tile is in TMEM
+        mbar_init(smem_u32(&bars.q_free), 1);       // the item's last Q K^T from TMEM has completed
+        mbar_init(smem_u32(&bars.q_drained), 128);  // epilogue threads: the Q tile has been read from shared memory
         mbar_init(smem_u32(&bars.o_free), 128);   // epilogue threads: accumulator drained
         mbar_init(smem_u32(&bars.o_full), 1);     // P V issuer: the item's last P V has completed
         mbar_init(smem_u32(&bars.e_ready), 256);  // softmax threads: row sums of the item are in shared memory
@@ -1542,7 +1546,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         uint32_t g_start = 0;  // running tile index at the start of the item
         bool ok = true;
         BSA_TRACE_DECL(tn);
-        // ---- Q tiles: TMA into shared memory one item ahead, then (d = 128) into TMEM through this warpgroup's registers ----
+        // ---- Q tiles.  d = 64: TMA into two buffers, two items ahead.  d = 128 from shared memory: the K producer loads
+        // them.  From TMEM: TMA into one buffer one item ahead, then to TMEM through this warpgroup's registers. ----
         int kq = 0;       // round of the next Q tile to load
         uint32_t nq = 0;  // Q tiles loaded so far
         auto load_q = [&]() {  // lane 0 of the warpgroup's first warp issues; every thread follows the item list
@@ -1551,22 +1556,17 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if (kq >= n_rounds) return;
                 w = load_item(p.items, cta_item_index(kq++, blockIdx.x, gridDim.x), n_items);
             } while (w.ntiles <= 0);
-            const uint32_t b = nq % NQB;
-            const uint32_t full = smem_u32(kOwnO ? &bars.qt_full[b] : &bars.q_full);
+            const uint32_t b = kOwnO ? (nq & 1u) : 0u;
             if (tw == 0) {
-                // two buffers: the item before last has read this one long ago
-                if (kOwnO && !mbar_wait(smem_u32(&bars.qt_free[b]), ((nq >> 1) & 1) ^ 1, abortp)) ok = false;
-                if (ok) {
-                    mbar_arrive_expect_tx(full, NSUB * Q_SUB);
-                    tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, full, 0, w.q_tile * kTQ, 0, w.head);
-                }
+                mbar_arrive_expect_tx(smem_u32(&bars.q_full[b]), NSUB * Q_SUB);
+                tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, smem_u32(&bars.q_full[b]), 0, w.q_tile * kTQ, 0, w.head);
             }
             ++nq;
         };
         uint32_t sq = 0;  // Q tiles moved to TMEM
         auto stage_q = [&]() -> bool {
-            bool good = mbar_wait(smem_u32(&bars.q_full), sq & 1, abortp);
-            good = good && mbar_wait(smem_u32(&bars.qt_free[0]), (sq & 1) ^ 1, abortp);
+            bool good = mbar_wait(smem_u32(&bars.q_full[0]), sq & 1, abortp);
+            good = good && mbar_wait(smem_u32(&bars.q_free), (sq & 1) ^ 1, abortp);
             if (!__all_sync(0xffffffffu, good)) return false;
             tc_fence_after();
             const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + Cols::kQ;
@@ -1583,14 +1583,15 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             mbar_arrive(smem_u32(&bars.q_drained));
             tc_wait_st();
             tc_fence_before();
-            mbar_arrive(smem_u32(&bars.qt_full[0]));
+            mbar_arrive(smem_u32(&bars.qt_full));
             if (tw == 0) good = mbar_wait(smem_u32(&bars.q_drained), sq & 1, abortp);  // then the next Q tile may land
             if (!__all_sync(0xffffffffu, good)) return false;
             ++sq;
             load_q();
             return true;
         };
-        load_q();
+        if constexpr (kOwnO || !kSmemQ) load_q();
+        if constexpr (kOwnO) load_q();
         WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
         for (int kr = 0; kr < n_rounds && ok; ++kr) {
             const WorkItem it = it_next;
@@ -1607,17 +1608,15 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 continue;
             }
-            // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); d = 128: the one TMEM buffer is
+            // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); the one TMEM buffer is
             // free after this item's last Q K^T, which comes well before its last P V
-            if constexpr (kOwnO) {
-                load_q();
-                ok = __all_sync(0xffffffffu, ok);
-            } else {
+            if constexpr (!kSmemQ) {
                 while (ok && nq > sq && sq <= itn + 1) ok = stage_q();
+                if (!ok) break;
             }
-            if (!ok) break;
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
             if (!ok) break;
+            if constexpr (kOwnO) load_q();  // this item's scores have all been read: its buffer is free for the item after next
             // d = 64: weights of the accumulator of the item's first tile (a) and of the other one (b).  Which warpgroup took
             // the first tile follows from the tiles this CTA had before, so everything below goes by a and b and not by
             // warpgroup: an item's bits are the same wherever it stands in a CTA's list.
@@ -1680,7 +1679,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                             for (int e = 0; e < 8; ++e)
                                 v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]), __uint_as_float(o[q * 16 + 2 * e + 1]));
-                            if (p.o_wide) {
+                            if constexpr (kSmemQ) {  // (long lists: the branch is the cheaper form)
+                                st_global_v8_or_2v4(orow + c * CW + q * 16, v, p.o_wide);
+                            } else if (p.o_wide) {
                                 st_global_v8(orow + c * CW + q * 16, v);
                             } else {
                                 uint4* dst = reinterpret_cast<uint4*>(orow + c * CW + q * 16);
@@ -1711,7 +1712,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // =========================== K producer ===========================
             // K tiles run up to NSK tiles ahead of the Q K^T issuer and never wait for V slots (the V tiles have a
             // thread of their own in warp 11).
-            uint32_t g = 0;
+            // Where Q stays in shared memory at d = 128 this thread also loads it, an item's tile in front of its first K tile:
+            // with two K tiles in the ring the wait for that K slot says that the last Q K^T of the item before last is done.
+            uint32_t g = 0, itq = 0;
             RingPos ring;  // K ring position of tile g
             bool ok = true;
             BSA_TRACE_DECL(tn);
@@ -1731,6 +1734,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     ok = mbar_wait(smem_u32(&bars.k_empty[stage]), ph ^ 1, abortp);
                     if (!ok) break;
                     BSA_TRACE_POINT(0, tn, 20);
+                    if (!kOwnO && kSmemQ && j == it.tile_begin) {
+                        const uint32_t b = itq++ & 1u;
+                        mbar_arrive_expect_tx(smem_u32(&bars.q_full[b]), NSUB * Q_SUB);
+                        tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, smem_u32(&bars.q_full[b]), 0, it.q_tile * kTQ, 0, it.head);
+                    }
                     mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), KV_TILE);
                     if constexpr (G == 1) {
                         tma_load_4d(smem_u32(sK + stage * KV_TILE), &tmK, smem_u32(&bars.k_full[stage]), 0, cur.key0[0], 0, it.head);
@@ -1796,8 +1804,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const int n = n_next;
                 n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
                 if (n <= 0) continue;
-                const uint32_t qb = itq % NQB;  // this item's Q buffer
-                ok = mbar_wait(smem_u32(&bars.qt_full[qb]), (itq / NQB) & 1, abortp);
+                const uint32_t qb = kSmemQ ? (itq & 1u) : 0u;  // this item's Q buffer
+                ok = kSmemQ ? mbar_wait(smem_u32(&bars.q_full[qb]), (itq >> 1) & 1, abortp)
+                            : mbar_wait(smem_u32(&bars.qt_full), itq & 1, abortp);
                 if (!ok) break;
                 const uint64_t descQ = descQ0 + (uint64_t)((qb * NSUB * Q_SUB) >> 4);
                 for (int j = 0; j < n; ++j, ring.advance(NSK)) {
@@ -1815,10 +1824,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     BSA_TRACE_POINT(1, tn, 6);
                     tc_fence_after();
                     const uint32_t d_s = tmem + (sb ? kColS1 : kColS0);
-#pragma unroll
+#pragma unroll(kSmemQ ? 4 : 8)  // (all eight with both operands' descriptors do not fit this thread's registers)
                     for (int k = 0; k < D / 16; ++k) {
                         const uint64_t b = descK + (uint64_t)((stage * KV_TILE + (k / 4) * KV_SUB + (k % 4) * 32) >> 4);
-                        if constexpr (kOwnO)
+                        if constexpr (kSmemQ)
                             mma_ss(d_s, descQ + (uint64_t)(((k / 4) * Q_SUB + (k % 4) * 32) >> 4), b, idesc_qk, k > 0);
                         else
                             mma_ts(d_s, tmem + Cols::kQ + k * 8, b, idesc_qk, k > 0);
@@ -1831,7 +1840,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     ++ph_n;
 #endif
                     BSA_TRACE_POINT(1, tn, 2);
-                    if (j == n - 1) mma_commit(smem_u32(&bars.qt_free[qb]));
+                    if (!kSmemQ && j == n - 1) mma_commit(smem_u32(&bars.q_free));
                 }
                 g += n;
                 ++itq;
@@ -2125,9 +2134,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                     for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
                 }
-                // ---- the reference moved at this tile: rescale the running output (after the P V of tile gs-1) ----
+                // ---- the reference moved at this tile: rescale the running output (its last P V has been waited for above) ----
                 if (j > 0 && __any_sync(0xffffffffu, rescale)) {
-                    if constexpr (!kOwnO) {  // (an accumulator of its own: tile gs-2 has been waited for above)
+                    if constexpr (!kOwnO && !kSmemQ) {  // (returns at once; without it ptxas spills in the gathered kernels)
                         ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
                         if (!ok) break;
                         tc_fence_after();
@@ -2350,9 +2359,13 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         else if constexpr (KERNEL == 2)
             e = cudaFuncSetAttribute(bsa_attention_cs_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         else {
-            e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, false, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(bsa_attention_pp_kernel<D, true, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            const auto allow = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
+            e = allow(bsa_attention_pp_kernel<D, false, G, true>);
+            if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, true>);
+            if constexpr (D != 64) {
+                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, false, G, false>);
+                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, false>);
+            }
         }
         if (e != cudaSuccess) {
             *err = "cudaFuncSetAttribute(max dynamic shared memory)";
@@ -2386,8 +2399,13 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         attr[0].val.programmaticStreamSerializationAllowed = 1;
         cfg.attrs = attr;
         cfg.numAttrs = 1;
-        cudaError_t le = a.f16 ? cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, true, G>, tq, tk, tv, p)
-                               : cudaLaunchKernelEx(&cfg, bsa_attention_pp_kernel<D, false, G>, tq, tk, tv, p);
+        const auto launch = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, tq, tk, tv, p); };
+        cudaError_t le;
+        if (D == 64 || (a.short_lists && p.stages == 2 && p.stages_v > 2)) {  // (the K producer relies on the two K tiles)
+            le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, true>) : launch(bsa_attention_pp_kernel<D, false, G, true>);
+        } else if constexpr (D != 64) {
+            le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, false>) : launch(bsa_attention_pp_kernel<D, false, G, false>);
+        }
         count_launch();
         return le;
     }

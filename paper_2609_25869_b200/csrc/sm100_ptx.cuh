@@ -263,6 +263,18 @@ __device__ __forceinline__ void st_global_v8(void* p, const uint32_t* v) {
                  "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
 }
+// The same 32 bytes to an address on a 16-byte boundary: one store where it also lies on a 32-byte one (`wide`), else two
+// (predicated: a branch around the second form costs about 100 clk per work item).
+__device__ __forceinline__ void st_global_v8_or_2v4(void* p, const uint32_t (&v)[8], int wide) {
+    asm volatile(
+        "{\n\t.reg .pred w;\n\t"
+        "setp.ne.s32 w, %9, 0;\n\t"
+        "@w st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};\n\t"
+        "@!w st.global.v4.b32 [%0], {%1, %2, %3, %4};\n\t"
+        "@!w st.global.v4.b32 [%0+16], {%5, %6, %7, %8};\n\t}"
+        ::"l"(p), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]), "r"(wide)
+        : "memory");
+}
 
 // Read-only global loads the compiler may neither delay nor duplicate: a prefetch into registers stays where it is
 // written (a plain load that is first used an iteration later tends to be moved next to that use, which puts its
