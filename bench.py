@@ -334,6 +334,33 @@ def sweep_block(gen, n_requests: int, heads: int, peaks):
             "lut_hits": sum(x["lut_hit"] for x in rows), "requests": rows}
 
 
+def headline(line):
+    """The line on stdout: every key of the full record with the long blocks cut down to their figures and numbers to six
+    digits, so that the whole line stays below 4000 characters (the full record goes to stderr)."""
+    def short(x):
+        if isinstance(x, float):
+            return float("%.6g" % x)
+        if isinstance(x, dict):
+            return {k: short(v) for k, v in x.items()}
+        return [short(v) for v in x] if isinstance(x, (list, tuple)) else x
+
+    out = dict(line)
+    keep = {"roofline": ("bound", "kernel", "plan", "achieved", "peak", "unit", "frac", "frac_of_sustained", "traffic", "launch_ms",
+                         "covered_over_active"),
+            "request": ("us_per_request_gpu", "us_per_request_host_median", "us_forward", "us_per_warm_request_gpu",
+                        "us_plan_create_host", "us_lookup", "us_planning_gpu", "planning_fraction", "plan", "lut_hit", "ntiles",
+                        "nitems", "density")}
+    for block, keys in keep.items():
+        if block in out:
+            out[block] = {k: out[block][k] for k in keys if k in out[block]}
+    if "others" in out:
+        out["others"] = {n: {k: o[k] for k in ("kernel_tflops", "kernel_ms", "request_ms", "plan")} for n, o in out["others"].items()}
+    if "sweep" in out:
+        out["sweep"] = {k: out["sweep"][k] for k in ("workload", "cold_request_us", "warm_forward_us", "planning_fraction",
+                                                     "tflops_warm_gm_by_geometry", "lut_hits")}
+    return short(out)
+
+
 def run_sweep(args):
     """--workload sweep: the sweep block alone, as one JSON line."""
     pool, gen = start_sweep_generation(args.sweep_requests, args.sweep_heads)
@@ -686,7 +713,8 @@ def main():
         line["sweep"] = sweep_block(gen, args.sweep_requests, args.sweep_heads, peaks)
         pool.terminate()
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps({"bench_details": line}), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 

@@ -89,3 +89,33 @@ def test_two_rank_aggregation_with_gloo():
     for rank, ms, tflops, w, distinct in res:
         assert w == 2 and ms == 5.0 and distinct          # max over ranks; each rank has its own inputs
         assert abs(tflops - (1e12 + 2e12) / 5e-3 / 1e12) < 1e-9
+
+
+def test_the_line_on_stdout_stays_readable_in_one_piece():
+    """The full record of a default run (50 sweep requests, four other workloads) is far longer than the 4000 characters the
+    line may have; every contract key is in the line, the sweep's single requests are not."""
+    sys.path.insert(0, ROOT)
+    import bench
+    f = 1234.567890123456
+    other = {"workload": "w" * 120, "kernel_tflops": f, "kernel_ms": f, "request_ms": f, "plan": "q128k128_pp_split4x8",
+             "back_to_back": {"launch_ms": f, "launches": 200}, "us_lookup": f}
+    line = {"metric": bench.METRIC, "value": f, "unit": "TFLOP/s", "n_gpus": 1, "steps": 20, "warmup": 5, "ms_per_step": f,
+            "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "bf16", "data": "synthetic",
+            "config": {"workload": "w" * 120, "l2": "256 MiB buffer written between timed iterations (L2 flush)"},
+            "step": "s" * 120, "clocks": {"sm_mhz": f, "sm_max_mhz": f, "reasons": ["sw_power_cap"]},
+            "e2e": {"value": f, "unit": "TFLOP/s", "h2d_bytes_per_step": 10 ** 9, "d2h_bytes_per_step": 10 ** 9, "ms_per_request": f},
+            "gpu_launches": 1000, "roofline": {"kernel": "k" * 40, "achieved": f, "peak": f, "frac": f, "traffic_source": "t" * 150},
+            "request": {"us_per_request_gpu": f, "us_planning_gpu_samples": [f] * 100, "plan": "p" * 20},
+            "cpu_baseline": {"value": f, "unit": "TFLOP/s", "cores": 16, "kind": "oracle", "seconds": f, "sample": "s" * 60},
+            "others": {n: other for n in ("tiny", "mid", "stress_a", "stress_b")},
+            "sweep": {"workload": "w" * 90, "protocol": "p" * 300,
+                      "cold_request_us": dict.fromkeys(("mean", "gm", "p50", "p95", "max"), f),
+                      "warm_forward_us": dict.fromkeys(("gm", "p50", "p95"), f), "planning_fraction": {"mean": f, "max": f},
+                      "tflops_warm_gm_by_geometry": {"%dx%d" % (16 << i, 128): f for i in range(5)}, "lut_hits": 50,
+                      "requests": [{"r": i, "plan": "q128k128_pp_natural", "cold_request_us": f} for i in range(50)]}}
+    text = json.dumps(bench.headline(line))
+    assert len(json.dumps(line)) > 4000 > len(text)
+    out = json.loads(text)
+    assert set(out) == set(line) and "requests" not in out["sweep"] and "us_planning_gpu_samples" not in out["request"]
+    assert all(out[k] == line[k] for k in ("metric", "unit", "n_gpus", "steps", "warmup", "config", "gpu_launches", "dtype", "data"))
+    assert abs(out["value"] / line["value"] - 1.0) < 1e-5 and out["e2e"]["h2d_bytes_per_step"] == 10 ** 9
