@@ -936,11 +936,6 @@ __global__ void __launch_bounds__(1024) organize_kernel(MapGeom g, int order, in
     __syncthreads();
 
     // ---- A: unsorted items ----
-    // One pass and one item per row (the common case of a short list under a plan that never splits): the item stays in
-    // this thread's registers until it is written to its final place, instead of going through `items_tmp`.
-    const bool resident = no_split && (row1 - row0) <= (int)blockDim.x;
-    WorkItem mine;
-    mine.head = mine.q_tile = mine.tile_begin = mine.tile_end = mine.part = mine.nparts = mine.ws_slot = mine.ntiles = 0;
     int32_t run_items = 0, run_split = 0, run_slots = 0;
     for (int r0 = row0; r0 < row1; r0 += blockDim.x) {
         const int r = r0 + tid;
@@ -970,10 +965,7 @@ __global__ void __launch_bounds__(1024) organize_kernel(MapGeom g, int order, in
                 it.ws_slot = (P > 1) ? (slot + p) * g.slots : -1;  // 128-row workspace slots
                 it.ntiles = it.tile_end - it.tile_begin;
                 const int32_t li = run_items + off_i + p;
-                if (resident)
-                    mine = it;  // li == tid
-                else
-                    items_tmp[item_base + li] = it;
+                items_tmp[item_base + li] = it;
                 key[li] = bucketed ? length_bucket(it.ntiles) : it.ntiles;
             }
             if (P > 1) {
@@ -993,19 +985,6 @@ __global__ void __launch_bounds__(1024) organize_kernel(MapGeom g, int order, in
     }
     __syncthreads();
     const int32_t n_items = run_items;
-    if (order == BSA_ORDER_NATURAL) {  // unsorted: the items stay in (head, q_tile, part) order
-        if (resident) {
-            if (tid < n_items) items[item_base + tid] = mine;
-        } else {
-            for (int i = tid; i < n_items; i += blockDim.x) items[item_base + i] = items_tmp[item_base + i];
-        }
-        if (tid == 0 && grp == gridDim.x - 1) {
-            counters->nitems = item_base + n_items;
-            counters->nsplit_rows = (split_base + run_split) * g.slots;
-            counters->nslots = slot_base + run_slots;
-        }
-        return;
-    }
     // ---- B + C1: stable counting sort by length (longest first; ties keep (head, q_tile, part) order) ----
     // The items are cut into contiguous chunks, one per ranking warp.  Every warp histograms its chunk into a private
     // row; the column sums give the bucket sizes, their suffix sums the bucket starts (longest first), and within a
@@ -1078,11 +1057,7 @@ __global__ void __launch_bounds__(1024) organize_kernel(MapGeom g, int order, in
     __syncthreads();
 
     // ---- C2: scatter ----
-    if (resident) {
-        if (tid < n_items) items[item_base + key[tid]] = mine;
-    } else {
-        for (int i = tid; i < n_items; i += blockDim.x) items[item_base + key[i]] = items_tmp[item_base + i];
-    }
+    for (int i = tid; i < n_items; i += blockDim.x) items[item_base + key[i]] = items_tmp[item_base + i];
 
     if (tid == 0) {
         if (global_group) {
@@ -1226,7 +1201,7 @@ static bool organize_by_rank(const MapGeom& g, int order, int split_pmax) {
 size_t organize_scratch_bytes(const MapGeom& g, int order, int split_pmax) {
     const bool global_group = (order == BSA_ORDER_GLOBAL_LPT || order == BSA_ORDER_GLOBAL_BUCKETS);
     const long long rows = (long long)g.H * g.nQt;
-    if (!global_group || split_pmax > 1 || rows < 4096 || organize_by_rank(g, order, split_pmax)) return 0;
+    if (!global_group || split_pmax > 1 || organize_by_rank(g, order, split_pmax)) return 0;
     const size_t chunks = (size_t)((rows + kOrgChunk - 1) / kOrgChunk);
     return (chunks + 1) * (size_t)organize_bins(g) * sizeof(int32_t);
 }
@@ -1346,6 +1321,7 @@ cudaError_t launch_organize(const MapGeom& g, int order, int split_pmax, const i
         count_launch();
         return e;
     }
+    if (order == BSA_ORDER_NATURAL) return cudaErrorInvalidValue;  // row order under Split-K: no plan of the catalog
     if (scratch && organize_scratch_bytes(g, order, split_pmax) > 0) {
         const int nrows = g.H * g.nQt, nbins = organize_bins(g);
         const int nchunks = (nrows + kOrgChunk - 1) / kOrgChunk;

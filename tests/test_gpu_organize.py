@@ -1,5 +1,6 @@
-"""Order of the work items against a stable sort on the host: lists around the ranking kernel's rows, tiles and the
-length from which the multi-pass sort takes over; every order; exported items, no forward."""
+"""Order of the work items against a stable sort on the host: lists around the ranking kernel's rows and tiles, and on
+both sides of the length from which the sorts take over (2^28 comparisons: several CTAs for the global orders, one per
+head for the head-major ones); every order; exported items, no forward."""
 import numpy as np
 import pytest
 import torch
@@ -16,7 +17,7 @@ def _bucket(n):  # half-octaves: 0, 1, 2, 3, 4-5, 6-7, 8-11, 12-15, ...
 
 
 @pytest.mark.parametrize("plan_id", [22, 25, 29, 30, 31])
-@pytest.mark.parametrize("H,rows", [(1, 1), (3, 31), (2, 33), (5, 64), (1, 2047), (2, 2049), (4, 4100), (7, 2900)])
+@pytest.mark.parametrize("H,rows", [(1, 1), (3, 31), (2, 33), (5, 64), (1, 2047), (2, 2049), (4, 4100), (7, 2900), (2, 12000)])
 def test_items_are_in_stable_order(H, rows, plan_id):
     nk = 37
     r = np.random.RandomState(H * 10000 + rows)
