@@ -2445,7 +2445,7 @@ static void split_stages(int total, int kernel, int* nk, int* nv) {
 
 int attention_max_stages(int d, int T_KV, int kernel) {
     if (kernel == 4) T_KV = kPpTK;
-    if (kernel == kKernelRowBlock) return (d <= 128 && T_KV <= rb_max_chunk(d)) ? 2 : 0;  // one K and one V buffer per warp
+    if (kernel == kKernelRowBlock) return (d <= 128 && T_KV <= rb_max_chunk(d)) ? 2 : 0;  // rings of two slots and more per warp, see there
     if (d == 256 && !((kernel == 0 || kernel == 3) && T_KV == 64)) return 0;  // see launch_forward
     const int nb = kv_buffers_that_fit(d, T_KV, kernel);
     if (kernel == 1 || kernel == 4) return nb > 2 * kMaxStages ? 2 * kMaxStages : nb;  // total K + V buffers

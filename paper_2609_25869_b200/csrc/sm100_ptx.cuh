@@ -284,11 +284,6 @@ __device__ __forceinline__ int ldg_pinned_s32(const int* p) {
     asm volatile("ld.global.nc.b32 %0, [%1];" : "=r"(v) : "l"(p));
     return v;
 }
-__device__ __forceinline__ unsigned long long ldg_pinned_u64(const uint64_t* p) {
-    unsigned long long v;
-    asm volatile("ld.global.nc.b64 %0, [%1];" : "=l"(v) : "l"(p));
-    return v;
-}
 
 // Three-input maximum and packed two-lane fp32 arithmetic (sm_100): they halve the number of
 // instructions the softmax loop issues around its exponentials.
