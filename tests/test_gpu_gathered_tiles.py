@@ -3,7 +3,9 @@ four of 32): list lengths around multiples of the entries per tile, ragged last 
 head dimensions and element types, Split-K partitions that start anywhere in the list."""
 import numpy as np
 import pytest
+import torch
 
+from paper_2609_25869_b200 import bsa
 from paper_2609_25869_b200 import inputs as I
 from tests import helpers as Hh
 
@@ -48,3 +50,20 @@ def test_rows_that_only_every_other_tile_reaches(d):
     req = I.Request("alternating", 2, 6 * 64, d, 64, 128, M, qkv_seed=3, N_kv=9 * 128 - 40)
     for plan_id in (22, 24):
         Hh.run_request(req, plan_id=plan_id)
+
+
+@pytest.mark.parametrize("B,d,dtype,plan_id", [(32, 64, "fp16", 39), (32, 128, "bf16", 43), (64, 64, "bf16", 23), (64, 128, "fp16", 28)])
+def test_token_major_gathered_tiles(B, d, dtype, plan_id):
+    """The copies of narrow entries out of token-major tensors: the same bits as head-major, which the oracle checks."""
+    H, N, N_kv = 3, 1000, 1301
+    M = I.random_mask(B + d, H, I.cdiv(N, B), I.cdiv(N_kv, B), 0.35, empty_rows=0.1)
+    req = I.Request("nhd", H, N, d, B, B, M, qkv_seed=B, N_kv=N_kv, dtype=dtype)
+    Hh.run_request(req, plan_id=plan_id)
+    mask, q, k, v, _ = Hh.to_dev(req)
+    kw = {"N_kv": N_kv, "dtype": dtype, "plan_id": plan_id}
+    with bsa.plan_create(mask, B, B, N, H, d, **kw) as plan:
+        O, L = plan.forward(q, k, v)
+    with bsa.plan_create(mask, B, B, N, H, d, layout="nhd", **kw) as plan:
+        Ot, Lt = plan.forward(*(t.permute(1, 0, 2).contiguous() for t in (q, k, v)))
+    torch.cuda.synchronize()
+    assert torch.equal(Ot.permute(1, 0, 2), O) and torch.equal(Lt, L)
