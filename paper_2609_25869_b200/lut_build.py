@@ -14,9 +14,10 @@ schema (``bsa_lut_buckets``), and each bucket gets the plans that are valid on a
 ranked by geometric-mean latency, ties by plan id, followed by the key's base plan.  The result
 is the text file ``bsa_lut_load`` reads.
 
-The profiling corpus uses seeds >= 1000, disjoint from every evaluation seed.
+The profiling corpus uses seeds >= 1000, disjoint from every evaluation seed.  The shipped table is what the defaults write
+(about 15 minutes on one B200):
 
-    python -m paper_2609_25869_b200.lut_build --out paper_2609_25869_b200/plan_table_b200.lut
+    python -m paper_2609_25869_b200.lut_build
 """
 from __future__ import annotations
 
@@ -32,6 +33,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 DEFAULT_OUT = os.path.join(HERE, "plan_table_b200.lut")
 
 O_TOL, O_MEAN_TOL, LSE_TOL = 2e-2, 2e-3, 1e-3  # validation gate (the contract tolerances)
+SUSTAIN_MIN_MS = 0.1  # shortest forward that is timed back to back (a forward's host share is about 15 us)
 
 
 # --------------------------------------------------------------------------------------------
@@ -53,9 +55,10 @@ def _by_case(lat: Dict[Tuple[Hashable, int], float]) -> Dict[Hashable, Dict[int,
 
 
 def compile_table(cases: Sequence[Tuple[Hashable, Hashable]], latencies: Dict[Tuple[Hashable, int], float],
-                  base_plan: Dict[Hashable, int], bucket_of: Callable[[Hashable], Hashable]) -> Dict:
+                  base_plan: Dict[Hashable, int], bucket_of: Callable[[Hashable], Hashable], min_cases: int = 1) -> Dict:
     """``cases``: (case id, request key); ``latencies[(case id, plan id)]``: validated median latency
-    (missing = failed validation or not eligible).  Returns {(key, bucket): [ranked ids..., base]}."""
+    (missing = failed validation or not eligible).  Returns {(key, bucket): [ranked ids..., base]}.  A bucket with fewer
+    than ``min_cases`` cases gets no line: its key's tree decides there."""
     table: Dict = {}
     by_key: Dict[Hashable, List[Hashable]] = {}
     for cid, key in cases:
@@ -65,6 +68,8 @@ def compile_table(cases: Sequence[Tuple[Hashable, Hashable]], latencies: Dict[Tu
         for cid in members:
             buckets.setdefault(bucket_of(cid), []).append(cid)
         for b, cids in buckets.items():
+            if len(cids) < min_cases:
+                continue
             candidates = None
             per_case = _by_case(latencies)
             for cid in cids:
@@ -186,18 +191,28 @@ def choose_depth(cids, feats, groups, lat, base: int, min_leaf: int = 8, depths=
     return best, score
 
 
+# Keys whose tree is learned from some of their sources only, by prefix.  (16,64), d = 64: whether 16-row or 128-row tiles
+# are faster depends on how many key blocks neighbouring rows share, which no feature measures.  The masks whose rows each
+# have runs of their own ("sa") lose more by the wrong plan (15 % of 32768 tokens, 16 heads: 2.9 ms on 16-row tiles, 4.7 on
+# 128-row ones) than most of the others do; the others' grid points keep their regimes.
+TREE_SOURCES = {(16, 64, 64): "sa"}
+
+
 def compile_trees(cases, feats, groups, lat, base_plan, min_leaf: int = 8, max_depth: int = 4, folds: int = 4, log=None):
     """One tree per request key that has at least ``min_leaf`` cases (a single leaf, i.e. one ranking for the key, unless
     it has the ``2 * min_leaf`` a split needs); the other keys keep the fixed-edge regimes alone."""
     by_key: Dict[Hashable, List[Hashable]] = {}
     for cid, key in cases:
-        by_key.setdefault(key, []).append(cid)
+        if groups[cid].startswith(TREE_SOURCES.get(key, "")):
+            by_key.setdefault(key, []).append(cid)
     trees = {}
     for key, members in sorted(by_key.items()):
         if len(members) < min_leaf:
             continue
-        depth, score = choose_depth(members, feats, groups, lat, base_plan[key], min_leaf, tuple(range(max_depth + 1)), folds)
-        trees[key] = learn_tree(members, feats, lat, base_plan[key], min_leaf, depth)
+        names = set(members)
+        own = {cp: t for cp, t in lat.items() if cp[0] in names}  # (indexed by case once per dictionary: keep it small)
+        depth, score = choose_depth(members, feats, groups, own, base_plan[key], min_leaf, tuple(range(max_depth + 1)), folds)
+        trees[key] = learn_tree(members, feats, own, base_plan[key], min_leaf, depth)
         if log:
             log(f"tree {key}: {len(members)} cases, depth {depth} chosen from held-out regret "
                 + ", ".join(f"{D}: {math.exp(v):.4f}" for D, v in sorted(score.items()))
@@ -245,7 +260,6 @@ def corpus_specs(scale: str = "full"):
         add("mid", "mid0", seed=1010)
         add("stress_b", "sb0", seed=1030, H=4, N=8192)
         return specs
-    # Every request key gets at least 64 cases, so that a tree with the paper's 32 cases per leaf can split it.
     # (64,64) d=64: Tiny's key
     n = 0
     for N in (1024, 2048, 4096, 8192):
@@ -290,6 +304,27 @@ def corpus_specs(scale: str = "full"):
                     for rho in (0.05, 0.15, 0.35):
                         add("sweep", f"gen{N}@{rho}", r=2000 + n, H=H, N=N, d=d, B=B, rho=rho)
                         n += 1
+    # and at long ones, where the K and V of all heads no longer fit L2 together and the item order decides (fewer and
+    # lighter cases where the mask alone has hundreds of millions of blocks)
+    n = 0
+    for d in (64, 128):
+        for B in ((16, 16), (16, 64), (32, 16), (32, 32), (64, 32), (64, 64), (64, 128), (128, 64), (128, 128), (256, 256)):
+            fine = B[0] * B[1] < 2048
+            for N in ((60000,) if fine else (60000, 108000)):
+                for H in ((3,) if fine else (2, 10)):
+                    for rho in ((0.05, 0.15) if fine else (0.04, 0.12, 0.3)):
+                        add("sweep", f"long{N}@{rho}", r=3000 + n, H=H, N=N, d=d, B=B, rho=rho)
+                        n += 1
+    # the same sizes with independent blocks and heads of one weight: nothing to balance, so the order that keeps one head's
+    # K and V in L2 can win
+    n = 0
+    for d in (64, 128):
+        for B in ((64, 64), (64, 128), (128, 64), (128, 128), (256, 256)):
+            for N in (16384, 60000, 108000):
+                for H in (2, 10):
+                    for p in (0.04, 0.15):
+                        add("random", f"even{N}@{p}", seed=4000 + n, H=H, N=N, d=d, B=B, p=p)
+                        n += 1
     return specs
 
 
@@ -297,6 +332,9 @@ def make_case(spec):
     """One corpus case from its spec (host only; runs in the generation pool)."""
     from . import inputs as I
     gen, kw, group = spec
+    if gen == "random":
+        M = I.random_mask(kw["seed"], kw["H"], I.cdiv(kw["N"], kw["B"][0]), I.cdiv(kw["N"], kw["B"][1]), kw["p"], diag=True)
+        return I.Request(f"random{kw['seed']}", kw["H"], kw["N"], kw["d"], kw["B"][0], kw["B"][1], M, qkv_seed=kw["seed"]), group
     fn = I.config_sweep if gen == "sweep" else I.CONFIGS[gen]
     req = fn(**kw)
     return req, group
@@ -384,10 +422,12 @@ def profile(reqs, plans=None, reps: int = 5, warmup: int = 3, log=print, validat
     every case (``case_features``), which the tree compiler partitions on.  ``reqs`` may be any iterable (a generator
     that produces the cases while earlier ones are profiled).  If it rejects the key's base plan, the
     case has no trusted full-size output to compare the other plans with and every plan is judged by it alone.
-    ``sustain_ms`` > 0: the plans within 15 % of the case's fastest are timed again back to back for that long, because a
-    layer's forwards follow each other and most of them run at the power cap, where the plan that moves less data keeps a
-    higher clock; their latencies are the sustained ones, the other plans' are scaled by the fastest plan's ratio.  Plans
-    that take more than twice the fastest one's time keep their first timing."""
+    ``sustain_ms`` > 0: a plan whose first forward takes more than twice the fastest plan's time so far is not timed
+    again, and where the fastest forward takes at least ``SUSTAIN_MIN_MS`` the plans within 15 % of it are timed back to
+    back for that long, in two rounds of opposite order: a layer's forwards follow each other and the long ones run at the
+    power cap, where the plan that moves less data keeps a higher clock.  Their latencies are then the sustained ones and
+    all others of the case are scaled by the fastest plan's ratio, so that a case's latencies stay comparable.  Shorter
+    forwards never reach the cap, and back to back they would rank the host's launches instead of the kernels."""
     import torch
     from . import bsa
     if validator is None:
@@ -400,6 +440,15 @@ def profile(reqs, plans=None, reps: int = 5, warmup: int = 3, log=print, validat
 
     def passes(req, pid, O, L, qkv):
         return bool(validator(req, pid, O, L, qkv))
+
+    def timed(plan, fill, *tensors):
+        flush.fill_(fill)  # flushes L2, and hides the host's share of the forward queued behind it
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        plan.forward(*tensors)
+        b.record()
+        b.synchronize()
+        return a.elapsed_time(b)
 
     for req in reqs:
         key = (req.B_Q, req.B_KV, req.d)
@@ -442,12 +491,7 @@ def profile(reqs, plans=None, reps: int = 5, warmup: int = 3, log=print, validat
                     continue
                 n_warm, n_reps = warmup, reps
                 if sustain_ms > 0:
-                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    a.record()
-                    plan.forward(q, k, v, O, L)
-                    b.record()
-                    b.synchronize()
-                    once = a.elapsed_time(b)
+                    once = timed(plan, 0, q, k, v, O, L)
                     if row and once > 2.0 * min(row)[0]:
                         lat[(req.name, pid)] = once
                         continue
@@ -455,33 +499,28 @@ def profile(reqs, plans=None, reps: int = 5, warmup: int = 3, log=print, validat
                         n_warm, n_reps = 0, 2
                 for _ in range(n_warm):
                     plan.forward(q, k, v, O, L)
-                ts = []
-                for i in range(n_reps):
-                    flush.fill_(i)
-                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    a.record()
-                    plan.forward(q, k, v, O, L)
-                    b.record()
-                    b.synchronize()
-                    ts.append(a.elapsed_time(b))
-                lat[(req.name, pid)] = statistics.median(ts)
+                lat[(req.name, pid)] = statistics.median(timed(plan, i, q, k, v, O, L) for i in range(n_reps))
                 row.append((lat[(req.name, pid)], pid))
         row.sort()
-        if sustain_ms > 0 and row:
+        if sustain_ms > 0 and row and row[0][0] >= SUSTAIN_MIN_MS:
             quick = dict((p, t) for t, p in row)
             near = [p for t, p in row if t <= 1.15 * row[0][0]]
+            total = dict.fromkeys(near, 0.0)
+            for order in (near, near[::-1]):
+                for pid in order:
+                    with bsa.plan_create(mask, req.B_Q, req.B_KV, req.N, req.H, req.d, plan_id=pid) as plan:
+                        n = max(1, int(0.5 * sustain_ms / quick[pid]))
+                        for _ in range(max(1, n // 3)):
+                            plan.forward(q, k, v, O, L)
+                        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                        a.record()
+                        for _ in range(n):
+                            plan.forward(q, k, v, O, L)
+                        b.record()
+                        b.synchronize()
+                        total[pid] += a.elapsed_time(b) / n
             for pid in near:
-                with bsa.plan_create(mask, req.B_Q, req.B_KV, req.N, req.H, req.d, plan_id=pid) as plan:
-                    n = max(2, int(sustain_ms / quick[pid]))
-                    for _ in range(max(1, n // 3)):
-                        plan.forward(q, k, v, O, L)
-                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    a.record()
-                    for _ in range(n):
-                        plan.forward(q, k, v, O, L)
-                    b.record()
-                    b.synchronize()
-                    lat[(req.name, pid)] = a.elapsed_time(b) / n
+                lat[(req.name, pid)] = 0.5 * total[pid]
             ratio = lat[(req.name, near[0])] / quick[near[0]]
             for pid in plan_ids:
                 if pid not in near and (req.name, pid) in lat:
@@ -492,12 +531,9 @@ def profile(reqs, plans=None, reps: int = 5, warmup: int = 3, log=print, validat
     return cases, lat, bucket, base
 
 
-def leave_source_out(path: str, min_leaf: int = 32, max_depth: int = 4, log=print) -> Dict[str, dict]:
-    """Offline check of how the table generalises, from a latencies file written by ``--latencies``: every mask source
-    in turn is left out of the corpus, regimes and trees are compiled from the rest, and each left-out case is looked
-    up in them in three ways (regimes then trees then base plan, as the runtime does; trees alone; regimes alone).
-    Returns per way the geometric-mean regret, the share within 3 % and the share of cases that found a regime or leaf.
-    Needs the library only for the fixed-edge bucket function and the base plans (no GPU)."""
+def read_latencies(path: str):
+    """(cases, latencies, features, source groups, buckets, base plans) of a file written by ``--latencies``.  Needs the
+    library only for the fixed-edge bucket function and the base plans (no GPU)."""
     import ctypes
     import json
     from . import bsa
@@ -506,7 +542,6 @@ def leave_source_out(path: str, min_leaf: int = 32, max_depth: int = 4, log=prin
     cases = [(c, tuple(k)) for c, k in d["cases"]]
     lat = {(c, int(pid)): t for c, pid, t in d["lat"]}
     feats = {c: tuple(v) for c, v in d["features"].items()}
-    groups = d["groups"]
     lib = bsa.lib()
     lib.bsa_lut_buckets.argtypes = [ctypes.c_int64, ctypes.c_double, ctypes.c_double, ctypes.c_double,
                                     ctypes.POINTER(ctypes.c_int32)]
@@ -518,13 +553,23 @@ def leave_source_out(path: str, min_leaf: int = 32, max_depth: int = 4, log=prin
         lib.bsa_lut_buckets(int(round(2.0 ** lg)), dens, skew, rc, out)
         bucket[c] = (out[0], head_bucket(int(heads)), out[1], out[2], out[3])
         base[key] = int(lib.bsa_base_plan(key[0], key[1], key[2]))
+    return cases, lat, feats, d["groups"], bucket, base
+
+
+def leave_source_out(path: str, min_leaf: int = 32, max_depth: int = 4, log=print, min_regime: int = 1) -> Dict[str, dict]:
+    """Offline check of how the table generalises, from a latencies file written by ``--latencies``: every mask source
+    in turn is left out of the corpus, regimes and trees are compiled from the rest, and each left-out case is looked
+    up in them in three ways (regimes then trees then base plan, as the runtime does; trees alone; regimes alone).
+    Returns per way the geometric-mean regret, the share within 3 % and the share of cases that found a regime or leaf.
+    Needs the library only for the fixed-edge bucket function and the base plans (no GPU)."""
+    cases, lat, feats, groups, bucket, base = read_latencies(path)
     sources = sorted(set(groups.values()))
     acc = {w: {"log": 0.0, "n": 0, "within": 0, "found": 0} for w in ("regime_tree_base", "tree_base", "regime_base")}
     for src in sources:
         held = [(c, k) for c, k in cases if groups[c] == src]
         keys = {k for _, k in held}  # only the tables of the left-out cases' own request keys matter
         train = [(c, k) for c, k in cases if groups[c] != src and k in keys]
-        table = compile_table(train, lat, base, lambda cid: bucket[cid])
+        table = compile_table(train, lat, base, lambda cid: bucket[cid], min_regime)
         trees = compile_trees(train, feats, groups, lat, base, min_leaf=min_leaf, max_depth=max_depth)
         for c, key in held:
             reg = table.get((key, bucket[c]))
@@ -545,6 +590,20 @@ def leave_source_out(path: str, min_leaf: int = 32, max_depth: int = 4, log=prin
     return res
 
 
+def write_compiled(args, cases, lat, feats, groups, bucket, base, gpu_name):
+    from . import bsa
+    table = compile_table(cases, lat, base, lambda cid: bucket[cid], args.min_regime)
+    trees = {} if args.no_trees else compile_trees(cases, feats, groups, lat, base, min_leaf=args.min_leaf,
+                                                   max_depth=args.max_depth, log=print)
+    write_table(args.out, table, int(bsa.lib().bsa_catalog_hash()), gpu_name,
+                notes=[f"{len(cases)} profiling cases, seeds >= 1000: median of 5 forwards after 3 warm-ups, L2 flushed; the plans near the "
+                       f"fastest back to back where a forward takes {SUSTAIN_MIN_MS:g} ms and more",
+                       "regime B_Q B_KV d floor(log2 N) head-bucket density-bucket skew-bucket runcov-bucket : ranked plans, base last",
+                       f"tree features: {' '.join(TREE_FEATURES)}; a request outside the regimes is looked up in its key's tree"],
+                trees=trees)
+    print(f"wrote {args.out}: {len(table)} regimes, {len(trees)} trees")
+
+
 def main(argv=None):
     ap = argparse.ArgumentParser(description=__doc__, formatter_class=argparse.RawDescriptionHelpFormatter)
     ap.add_argument("--leave-source-out", default="", metavar="LATENCIES.json",
@@ -552,15 +611,22 @@ def main(argv=None):
                     "of the left-out cases (host only)")
     ap.add_argument("--out", default=DEFAULT_OUT)
     ap.add_argument("--scale", default="full", choices=["full", "quick"])
-    ap.add_argument("--min-leaf", type=int, default=32, help="fewest cases a tree leaf may hold (Section 5.1: 32)")
+    ap.add_argument("--min-leaf", type=int, default=12, help="fewest cases a tree leaf may hold (Section 5.1: 32, of a corpus "
+                    "thirty times this one)")
+    ap.add_argument("--min-regime", type=int, default=1, help="fewest cases of a fixed-edge regime (below: the key's tree decides)")
     ap.add_argument("--max-depth", type=int, default=4)
     ap.add_argument("--no-trees", action="store_true", help="fixed-edge regimes only")
     ap.add_argument("--sustain-ms", type=float, default=40.0, help="back-to-back time per plan near the fastest (0: single forwards)")
-    ap.add_argument("--kernels", default="", help="profile the plans of these kernel families only (comma-separated), and the base plans")
+    ap.add_argument("--kernels", default="4,5", help="profile the plans of these kernel families only (comma-separated; the "
+                    "default ones are the fastest everywhere), or 'all'")
     ap.add_argument("--latencies", default="", help="also write the measured latencies as JSON (for the regret report)")
+    ap.add_argument("--from-latencies", default="", metavar="LATENCIES.json", help="no profiling: compile the table from a recorded corpus")
     args = ap.parse_args(argv)
     if args.leave_source_out:
-        leave_source_out(args.leave_source_out, args.min_leaf, args.max_depth)
+        leave_source_out(args.leave_source_out, args.min_leaf, args.max_depth, min_regime=args.min_regime)
+        return 0
+    if args.from_latencies:
+        write_compiled(args, *read_latencies(args.from_latencies), "NVIDIA B200")
         return 0
     specs = corpus_specs(args.scale)
     # masks are generated by worker processes (forked before CUDA is touched) while earlier cases are profiled
@@ -583,26 +649,19 @@ def main(argv=None):
     print(f"corpus: {len(specs)} cases")
     feats = {}
     plans = None
-    if args.kernels:
+    if args.kernels != "all":
         kernels = {int(x) for x in args.kernels.split(",")}
         plans = [c["plan_id"] for c in bsa.catalog() if c["kernel"] in kernels]
     cases, lat, bucket, base = profile(cases_in_order(), plans=plans, features_out=feats, sustain_ms=args.sustain_ms)
     pool.terminate()
-    table = compile_table(cases, lat, base, lambda cid: bucket[cid])
-    trees = {} if args.no_trees else compile_trees(cases, feats, groups, lat, base, min_leaf=args.min_leaf,
-                                                   max_depth=args.max_depth, log=print)
-    write_table(args.out, table, int(bsa.lib().bsa_catalog_hash()), torch.cuda.get_device_name(0),
-                notes=[f"{len(cases)} profiling cases, seeds >= 1000, median of 5 forwards after 3 warm-ups, L2 flushed",
-                       "regime B_Q B_KV d floor(log2 N) head-bucket density-bucket skew-bucket runcov-bucket : ranked plans, base last",
-                       f"tree features: {' '.join(TREE_FEATURES)}; a key with a tree is looked up there, the others in the regimes"],
-                trees=trees)
     if args.latencies:
         import json
         with open(args.latencies, "w") as f:
             json.dump({"cases": [[c, list(k)] for c, k in cases], "lat": [[c, p, t] for (c, p), t in lat.items()],
                        "features": feats, "groups": groups}, f)
+    write_compiled(args, cases, lat, feats, groups, bucket, base, torch.cuda.get_device_name(0))
     bsa.lut_load(args.out)
-    print(f"wrote {args.out}: {len(table)} regimes, {len(trees)} trees in {time.time() - t0:.0f} s")
+    print(f"{time.time() - t0:.0f} s")
     return 0
 
 

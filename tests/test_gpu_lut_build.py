@@ -120,3 +120,29 @@ def test_default_reference_of_the_validation_gate_accepts_a_plan_and_rejects_dam
     assert len(empty)
     L3 = L.clone(); L3[1, int(empty[0]) * 64] = 0.0
     assert not val(req, 1, O, L3, (q, k, v))
+
+
+def test_profile_times_long_forwards_back_to_back_and_filters_slow_plans(monkeypatch):
+    """The sustained stage, reached by lowering its limit: only plans near the fastest are timed again, every validated plan
+    keeps one positive latency, and with the limit out of reach nothing is scaled."""
+    req = I.config_mid(seed=1010, H=2)
+    req.name = "mid#0"
+    plans = [0, 22, 25, 29]
+    forwards = []
+    real = bsa.Plan.forward
+
+    def counting(self, *a, **kw):
+        forwards.append(self.info()["plan"]["plan_id"])
+        return real(self, *a, **kw)
+
+    monkeypatch.setattr(bsa.Plan, "forward", counting)
+    quick = lut_build.profile([req], plans=plans, reps=3, warmup=2, log=lambda s: None, sustain_ms=2.0)[1]
+    n_quick = len(forwards)
+    monkeypatch.setattr(lut_build, "SUSTAIN_MIN_MS", 0.0)
+    forwards.clear()
+    long = lut_build.profile([req], plans=plans, reps=3, warmup=2, log=lambda s: None, sustain_ms=2.0)[1]
+    assert set(quick) == set(long) == {(req.name, p) for p in plans} and all(t > 0 for t in list(quick.values()) + list(long.values()))
+    best = min(long, key=long.get)[1]
+    assert len(forwards) > n_quick and forwards.count(best) > 10   # 2 ms of a forward well below 0.2 ms
+    # the single-tile kernel is slower than the ping-pong kernel by more than 15 %: timed once, then scaled
+    assert forwards.count(0) <= 1 + 1 + 2 + 3 and long[(req.name, 0)] > long[(req.name, best)]
