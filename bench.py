@@ -30,9 +30,10 @@ sys.path.insert(0, ROOT)
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 METRIC = "effective TFLOP/s on active blocks (4*d flops per active token pair)"
 # dram__bytes_read.sum + dram__bytes_write.sum of ONE attention-kernel launch, from the ncu captures summarised under
-# profiles/: {workload: (bytes, how the figure was obtained)}.  All three are of kernels before Q moved to tensor memory and
-# before the row-block kernel's copy rings.  The Hunyuan-shaped launch is too large to capture whole; its figure is a 4-head capture of the same shape scaled by heads (the plan keeps
-# heads apart in the queue, so traffic grows in proportion to them).
+# profiles/: {workload: (bytes, how the figure was obtained)}.  All three are of kernels before Q moved to tensor memory
+# and before the row-block kernel's copy rings.  The Hunyuan-shaped launch is too large to capture whole; its figure is a
+# 4-head capture of the same shape scaled by heads (the plan keeps heads apart in the queue, so traffic grows in
+# proportion to them).
 NCU_TRAFFIC_BYTES = {
     "hunyuan": (6 * 798.2e6, "ncu capture of one launch of the same shape at 4 heads (682.3 MB read + 116.0 MB written), x 24/4"),
     "mid": (206.5e6, "one ncu capture of one launch of this workload"),
