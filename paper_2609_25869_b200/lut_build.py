@@ -14,8 +14,8 @@ schema (``bsa_lut_buckets``), and each bucket gets the plans that are valid on a
 ranked by geometric-mean latency, ties by plan id, followed by the key's base plan.  The result
 is the text file ``bsa_lut_load`` reads.
 
-The profiling corpus uses seeds >= 1000, disjoint from every evaluation seed.  The shipped table is what the defaults write
-(about 15 minutes on one B200):
+The profiling corpus uses seeds >= 1000, disjoint from every evaluation seed.  The defaults are meant for the shipped
+table (about 15 minutes on one B200); the present file was compiled from a smaller corpus and says so in its head:
 
     python -m paper_2609_25869_b200.lut_build
 """
