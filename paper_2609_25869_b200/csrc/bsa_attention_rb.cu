@@ -238,36 +238,30 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
                     if (kc + 1 >= p.Nkv) s[n][1] = s[n][3] = -INFINITY;
                 }
             }
-            float mx_lo = -INFINITY, mx_hi = -INFINITY;
+            float mx_lo = max3(s[0][0], s[0][1], s[1][0]), mx_hi = max3(s[0][2], s[0][3], s[1][2]);
+            mx_lo = fmaxf(mx_lo, s[1][1]);
+            mx_hi = fmaxf(mx_hi, s[1][3]);
 #pragma unroll
-            for (int n = 0; n < NT_S; ++n) {
-                mx_lo = fmaxf(mx_lo, fmaxf(s[n][0], s[n][1]));
-                mx_hi = fmaxf(mx_hi, fmaxf(s[n][2], s[n][3]));
+            for (int n = 2; n < NT_S; ++n) {
+                mx_lo = max3(mx_lo, s[n][0], s[n][1]);
+                mx_hi = max3(mx_hi, s[n][2], s[n][3]);
             }
-            mx_lo = fmaxf(mx_lo, __shfl_xor_sync(kFullMask, mx_lo, 1));
-            mx_hi = fmaxf(mx_hi, __shfl_xor_sync(kFullMask, mx_hi, 1));
-            mx_lo = fmaxf(mx_lo, __shfl_xor_sync(kFullMask, mx_lo, 2));
-            mx_hi = fmaxf(mx_hi, __shfl_xor_sync(kFullMask, mx_hi, 2));
-            const float mn_lo = fmaxf(m_lo, mx_lo * c2), mn_hi = fmaxf(m_hi, mx_hi * c2);
-            const float a_lo = (m_lo == -INFINITY) ? 0.f : ex2(m_lo - mn_lo);
-            const float a_hi = (m_hi == -INFINITY) ? 0.f : ex2(m_hi - mn_hi);
-            m_lo = mn_lo;
-            m_hi = mn_hi;
-            const float nm_lo = (mn_lo == -INFINITY) ? 0.f : -mn_lo, nm_hi = (mn_hi == -INFINITY) ? 0.f : -mn_hi;
-            float sum_lo = 0.f, sum_hi = 0.f;
-            uint32_t pa[KS_PV][4];  // P as the A operand of P V
-#pragma unroll
-            for (int n = 0; n < NT_S; ++n) {
-                const float p0 = ex2(fmaf(s[n][0], c2, nm_lo)), p1 = ex2(fmaf(s[n][1], c2, nm_lo));
-                const float p2 = ex2(fmaf(s[n][2], c2, nm_hi)), p3 = ex2(fmaf(s[n][3], c2, nm_hi));
-                sum_lo += p0 + p1;
-                sum_hi += p2 + p3;
-                pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16<F16>(p0, p1);
-                pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16<F16>(p2, p3);
-            }
-            l_lo = fmaf(l_lo, a_lo, sum_lo);
-            l_hi = fmaf(l_hi, a_hi, sum_hi);
-            if (__any_sync(kFullMask, a_lo != 1.f || a_hi != 1.f)) {  // a maximum moved: rescale the running output
+            mx_lo *= c2;
+            mx_hi *= c2;
+            // The running maxima have moved for some row of the fragment in about a third of the steps of a long list: only
+            // then do the four lanes of a row have to agree, and the sums and the output to be rescaled.
+            if (__any_sync(kFullMask, mx_lo > m_lo || mx_hi > m_hi)) {
+                mx_lo = fmaxf(mx_lo, __shfl_xor_sync(kFullMask, mx_lo, 1));
+                mx_hi = fmaxf(mx_hi, __shfl_xor_sync(kFullMask, mx_hi, 1));
+                mx_lo = fmaxf(mx_lo, __shfl_xor_sync(kFullMask, mx_lo, 2));
+                mx_hi = fmaxf(mx_hi, __shfl_xor_sync(kFullMask, mx_hi, 2));
+                const float mn_lo = fmaxf(m_lo, mx_lo), mn_hi = fmaxf(m_hi, mx_hi);
+                const float a_lo = (m_lo == -INFINITY) ? 0.f : ex2(m_lo - mn_lo);
+                const float a_hi = (m_hi == -INFINITY) ? 0.f : ex2(m_hi - mn_hi);
+                m_lo = mn_lo;
+                m_hi = mn_hi;
+                l_lo *= a_lo;
+                l_hi *= a_hi;
 #pragma unroll
                 for (int n = 0; n < NT_O; ++n) {
                     o[n][0] *= a_lo;
@@ -275,6 +269,28 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
                     o[n][2] *= a_hi;
                     o[n][3] *= a_hi;
                 }
+            }
+            const float nm_lo = (m_lo == -INFINITY) ? 0.f : -m_lo, nm_hi = (m_hi == -INFINITY) ? 0.f : -m_hi;
+            const uint64_t c22 = pack_f32x2(c2, c2), nm_lo2 = pack_f32x2(nm_lo, nm_lo), nm_hi2 = pack_f32x2(nm_hi, nm_hi);
+            uint64_t sum_lo2 = pack_f32x2(0.f, 0.f), sum_hi2 = sum_lo2;
+            uint32_t pa[KS_PV][4];  // P as the A operand of P V
+#pragma unroll
+            for (int n = 0; n < NT_S; ++n) {
+                float x0, x1, x2, x3;
+                unpack_f32x2(fma_f32x2(pack_f32x2(s[n][0], s[n][1]), c22, nm_lo2), x0, x1);
+                unpack_f32x2(fma_f32x2(pack_f32x2(s[n][2], s[n][3]), c22, nm_hi2), x2, x3);
+                const float p0 = ex2(x0), p1 = ex2(x1), p2 = ex2(x2), p3 = ex2(x3);
+                sum_lo2 = add_f32x2(sum_lo2, pack_f32x2(p0, p1));
+                sum_hi2 = add_f32x2(sum_hi2, pack_f32x2(p2, p3));
+                pa[n >> 1][(n & 1) * 2 + 0] = pack_bf16<F16>(p0, p1);
+                pa[n >> 1][(n & 1) * 2 + 1] = pack_bf16<F16>(p2, p3);
+            }
+            {
+                float a0, a1, b0, b1;
+                unpack_f32x2(sum_lo2, a0, a1);
+                unpack_f32x2(sum_hi2, b0, b1);
+                l_lo += a0 + a1;
+                l_hi += b0 + b1;
             }
             // ---- O += P V ----
             ok = mbar_wait_warp(bV + slot * 8, phase, abortp);

@@ -34,3 +34,17 @@ def test_token_major_tensors():
         Ot, Lt = b.forward(*(t.permute(1, 0, 2).contiguous() for t in (q, k, v)))
     torch.cuda.synchronize()
     assert torch.equal(Ot.permute(1, 0, 2), O) and torch.equal(Lt, L)
+
+
+@pytest.mark.parametrize("d,B_KV,plan_id,dtype", [(64, 64, 34, "bf16"), (64, 16, 36, "fp16"), (128, 32, 35, "bf16")])
+@pytest.mark.parametrize("growing", [True, False])
+def test_scores_that_move_the_running_maximum(d, B_KV, plan_id, dtype, growing):
+    """Keys whose length grows or falls along the list: the running maximum moves at nearly every step, or after the first
+    ones hardly at all, in some rows of a fragment and not in the rest."""
+    n = 12
+    M = np.ones((1, 3, n), np.uint8)
+    req = I.Request("reference", 1, 40, d, 16, B_KV, M, qkv_seed=3, N_kv=n * B_KV, dtype=dtype)
+    q, k, v = req.qkv()
+    steps = torch.linspace(0.1, 4.0, n)
+    scale = (steps if growing else steps.flip(0)).repeat_interleave(B_KV)[None, :, None]
+    Hh.run_request(req, plan_id=plan_id, qkv=(q, (k.float() * scale).to(k.dtype), v), guards=False)
