@@ -12,12 +12,14 @@
 //     as the warp has read it, so the next steps' copies are in flight during the arithmetic of the current one;
 //   * S = Q K^T, online softmax with the running row maximum in the exp2 domain, P rounded to bf16 in registers
 //     (the accumulator layout of two 8-key tiles is the A-operand layout of one 16-key step), O += P V;
-//   * no block-level synchronisation at all: warps are independent, twelve per SM.
+//   * no block-level synchronisation: twelve independent warps per SM, each takes the next of the CTA's items when it is free.
 // A block of 16 rows and 64 keys (d = 64) is 262 kflop on 16 KB of K and V, each byte used once: shared memory sees it
 // twice (copy in, ldmatrix), 256 clk per SM at 128 B/clk against 133 clk of MMA, which makes 2.2 ms of the workload
 // below.  With per-thread cp.async copies of whole entries the load path stopped at about 41 B/clk per SM (bulk copies
 // reach 80); now, on one GPU, 32768 tokens, 16 heads, d = 64, (16,64) blocks, 15 % active in runs: 3.58 -> 2.77 ms; the
-// same with 32-key entries 4.01 -> 2.94 ms, (32,32) blocks at d = 128 52 -> 40 ms.  (Fragments loaded straight from
+// same with 32-key entries 4.01 -> 2.94 ms, (32,32) blocks at d = 128 52 -> 40 ms; maxima agreed on only where one has moved,
+// and items taken by free warps instead of a fixed share each: 2.82 -> 2.50, independent blocks at 15 % 2.48 -> 2.28, (16,16)
+// blocks at 10 %, 16384 tokens, 4 heads 222 -> 182 us.  (Fragments loaded straight from
 // global memory, no shared memory at all: 5.4 ms, the L1 miss path moves about 32 B/clk.  Fourteen warps: spills, 3.95.)
 // The register-level instruction peaks at about a third of the tcgen05 rate on this GPU, so the kernel pays off only
 // where Coarsening wastes more than that; the plan table decides per regime.
@@ -118,6 +120,7 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ __align__(8) uint64_t bars[kRbWarps][2 * NST];  // K slots, then V slots: the copy has landed
     __shared__ uint32_t abort_flag;
+    __shared__ int next_round;  // of the CTA's items: the next one no warp has taken
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int g = lane >> 2, t = lane & 3;
     const uint32_t sK = smem_u32(smem + warp * 2 * kRbStageBytes), sV = sK + kRbStageBytes;
@@ -126,7 +129,7 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
         if (threadIdx.x == 0) atomicExch(&p.counters->status, (int)BSA_ERR_CUDA);
         return;
     }
-    if (threadIdx.x == 0) abort_flag = 0;
+    if (threadIdx.x == 0) abort_flag = next_round = 0;
     if (lane == 0) {
         for (int i = 0; i < 2 * NST; ++i) mbar_init(bK + i * 8, 1);
         fence_mbar_init();
@@ -135,20 +138,25 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
     volatile uint32_t* abortp = &abort_flag;
 
     const int n_items = p.counters->nitems;
-    const int total_warps = (int)gridDim.x * kRbWarps;
-    const int gw = (int)blockIdx.x * kRbWarps + warp;
-    const int n_rounds = (n_items + total_warps - 1) / total_warps;
+    // The CTA's items (dealt in alternating directions per round of the list, longest first) go to whichever warp is free.
+    // A fixed share per warp left the SM to its last busy warps: with row lists of 14 to 431 entries (32768 tokens, 16
+    // heads, runs) the SMs' sums of fixed shares differ by 19 %, a warp's from the mean by 24 %.
+    auto take_item = [&]() -> int {
+        int k = 0;
+        if (lane == 0) k = atomicAdd(&next_round, 1);
+        k = __shfl_sync(kFullMask, k, 0);
+        return k * (int)gridDim.x + ((k & 1) ? ((int)gridDim.x - 1 - (int)blockIdx.x) : (int)blockIdx.x);
+    };
+    auto load_record = [&](int idx) { return __ldg(reinterpret_cast<const int4*>(p.items + (idx < n_items ? idx : 0))); };
     const float c2 = p.scale_log2;
     int slot = 0;          // ring slot of the current step (the same for K and V)
     uint32_t phase = 0;    // its barriers' phase
     bool ok = true;
 
-    for (int k = 0; k < n_rounds && ok; ++k) {
-        // items arrive longest first: rounds are dealt alternately forwards and backwards to even out the warps' sums
-        const int idx = k * total_warps + ((k & 1) ? (total_warps - 1 - gw) : gw);
-        if (idx >= n_items) continue;
-        const int4 ia = __ldg(reinterpret_cast<const int4*>(p.items + idx));
-        const int head = ia.x, q_tile = ia.y, tile_begin = ia.z, tile_end = ia.w;
+    int idx = take_item();
+    int4 record = load_record(idx);
+    while (idx < n_items) {
+        const int head = record.x, q_tile = record.y, tile_begin = record.z, tile_end = record.w;
         const int row0 = q_tile * 16;
         const int r_lo = row0 + g, r_hi = row0 + g + 8;
         __nv_bfloat16* o_lo = p.O + (long long)head * p.q_head + (long long)r_lo * p.q_row;
@@ -163,6 +171,8 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
                 if (r_lo < p.N) p.LSE[(long long)head * p.N + r_lo] = -INFINITY;
                 if (r_hi < p.N) p.LSE[(long long)head * p.N + r_hi] = -INFINITY;
             }
+            idx = take_item();
+            record = load_record(idx);
             continue;
         }
         const int n_steps = (tile_end - tile_begin) * SPE;
@@ -205,6 +215,10 @@ bsa_attention_rb_kernel(const __grid_constant__ CUtensorMap tmK, const __grid_co
 
         for (int st = 0; st < n_steps; ++st) {
             const bool more = st + NST < n_steps;
+            if (st == n_steps - NST || (st == 0 && n_steps < NST)) {  // nothing left to copy: the next item's record instead
+                idx = take_item();
+                record = load_record(idx);
+            }
             const int key_in = key_next;
             if (st + NST + 1 < n_steps) key_next = first_key(st + NST + 1);
             const uint32_t cK = sK + slot * SLOT, cV = sV + slot * SLOT;
@@ -354,8 +368,7 @@ cudaError_t launch_rb_t(const ForwardArgs& a, const RbParams& p, cudaStream_t st
         }
         attr_set_dev[dev].store(1, std::memory_order_relaxed);
     }
-    long long want = ((long long)a.max_items + kRbWarps - 1) / kRbWarps;
-    int grid = want < a.num_sms ? (int)want : a.num_sms;
+    int grid = a.max_items < a.num_sms ? a.max_items : a.num_sms;  // (few items: one warp each on as many SMs as there are)
     if (grid < 1) grid = 1;
     CUtensorMap tk, tv;
     if (!encode_kv_map(&tk, a.K, a.g.N_kv, a.g.H, D, kRbStep<D, CK>, F16, a.nhd) ||
