@@ -1343,6 +1343,18 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // (the V ring gives up one of its four), loaded by the K producer.  Forward at 32768 tokens, 8 heads, n tiles per item,
 // TMEM / shared memory in us: n = 1 46.8 / 41.4, 2 55.4 / 52.1, 3 68.3 / 66.0, 4 81.3 / 79.7, 6 107.6 / 106.1; at 16384
 // tokens 8 67.5 / 67.5, 12 93.4 / 93.9.  Hence shared memory below eight tiles per item on average (bsa_plan::short_lists).
+// Reference maximum at d = 128, bf16, long lists (kFirstRef): the maximum of the first tile that reaches a row serves the
+// whole item.  bf16 and fp32 keep their relative precision over 2^100, so it does not matter how far later scores lie above
+// it; from its second tile on a softmax warpgroup neither looks for maxima (64 instructions and about 300 clk per tile) nor
+// takes and publishes a word per row and tile, and nothing is rescaled.  Where it fails (a row sum beyond 2^100 or undefined,
+// or an accumulator that overflows) the epilogue marks the item, and a second pass over the marked items follows the running
+// maximum as before, moved by more than 2^8 at a time.  Per 128-key tile the softmax chain falls by a fifth.  Builds in turn,
+// back to back, before / after: 16384 tokens, 8 heads, (128,128) 153.5 / 144.4 us; 115200, 4 heads 1840 / 1725; 75600, 6
+// heads, (64,64) 3650 / 3510, 4 heads, (32,32) 4560 / 3700.  Half has no such range.  Short lists (Q in shared memory) and
+// d = 64 keep the running maximum: there the second copy of the loop costs more than it saves (32768 tokens, 8 heads, two
+// tiles per item 74 -> 82 us; 2048 tokens, 2 heads, d = 64 16.5 -> 18.5; (64,64) blocks at d = 64, 32768 tokens, 16 heads
+// 1310 -> 1430).  Both kernels take a row's reference from the same tile, so that an item whose scores do not outgrow it by
+// 2^8 has the same bits in either.
 // Two kernels and not a flag in one: what an item pays at its boundary is mostly instruction fetch, and the softmax code
 // has no register to spare (one kernel with both bodies was 1-2 % slower on long lists).
 //
@@ -1418,9 +1430,18 @@ struct RingPos {
 
 struct __align__(8) PpBarriers {
     uint64_t q_full[2], qt_full, q_free, q_drained, o_free, o_full, e_ready, e_taken;
+    uint64_t pass_done, tags_reset;
     uint64_t k_full[kMaxStages], k_empty[kMaxStages], v_full[kMaxStages], v_empty[kMaxStages];
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2];
 };
+
+constexpr int kRedoBits = 512;  // rounds of a CTA told apart when items are computed again
+template <int V>
+struct IntC {
+    static constexpr int value = V;
+};
+// A row sum (at least 1: the reference's own weight; 0: no active block) is trusted up to 2^100.
+__device__ __forceinline__ bool sum_is_doubtful(float l) { return !(l <= 1.2676506e30f); }
 
 // Tensor-memory columns of the ping-pong kernel (Q's are in use only where Q K^T reads it from there).
 template <int D>
@@ -1460,6 +1481,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int V_SUB = (G == 1) ? KV_SUB : GK * 128;  // a V tile holds its entries one after the other
     using Cols = PpCols<D>;
     constexpr bool kOwnO = Cols::kOwnO;
+    constexpr bool kFirstRef = !F16 && !kSmemQ;  // a row's first reference serves the whole item (see above)
     static_assert(!kOwnO || kSmemQ, "d = 64 has no tensor-memory columns left for Q");
     static_assert(kOwnO || NSUB * Q_SUB == KV_TILE, "at d = 128 the second Q tile takes the place of a V tile");
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
@@ -1474,10 +1496,13 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // the word's two low bits hold (publish index + 1) mod 4, so the reader of the next tile (always the same
     // row's thread of the other warpgroup, which consumes every publish in order) needs one shared-memory
     // read, with no barrier in front of it, to know whether the value it got is the one it waits for.
-    // (d = 64: each warpgroup's own reference at the end of an item, plain.)
+    // (d = 64: each warpgroup's own reference at the end of an item, plain.  First pass under kFirstRef: [item parity][row],
+    // the references as far as they are known, handed from tile to tile until every row of the warp has one; tags 0 or 1
+    // from the item's first tile, by its number's second bit, then 2 and 3 in turn.)
     __shared__ uint32_t mref[2][kTQ];
     __shared__ float lfin[2][kTQ];   // [warpgroup][row]: an item's partial row sums (d = 128: in its final reference)
     __shared__ float mfin[kTQ];      // d = 128: the item's final reference maximum (log2 domain) per row
+    __shared__ uint32_t redo_bits[kRedoBits / 32], redo_any;  // rounds of the CTA's items that pass 1 computes again
     __shared__ uint32_t tmem_base_s;
     __shared__ uint32_t abort_flag;
 
@@ -1501,6 +1526,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         mbar_init(smem_u32(&bars.o_full), 1);     // P V issuer: the item's last P V has completed
         mbar_init(smem_u32(&bars.e_ready), 256);  // softmax threads: row sums of the item are in shared memory
         mbar_init(smem_u32(&bars.e_taken), 128);  // epilogue threads: row sums read
+        mbar_init(smem_u32(&bars.pass_done), 384);  // epilogue and softmax threads: the first pass is over
+        mbar_init(smem_u32(&bars.tags_reset), 256);
         for (int s = 0; s < kMaxStages; ++s) {
             mbar_init(smem_u32(&bars.k_full[s]), 1);
             mbar_init(smem_u32(&bars.k_empty[s]), 1);
@@ -1515,7 +1542,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
         fence_mbar_init();
     }
-    if (tid < 2 * kTQ) (&mref[0][0])[tid] = 0u;  // tag 0: matches no first publish
+    if (tid < 2 * kTQ) (&mref[0][0])[tid] = kFirstRef ? 2u : 0u;  // a tag that matches no first publish
+    if (tid < kRedoBits / 32) redo_bits[tid] = 0u;
+    if (tid == kTQ) redo_any = 0u;
     if (warp == 9) {
         tmem_alloc(smem_u32(&tmem_base_s), kTmemCols);
         tmem_relinquish();
@@ -1536,6 +1565,18 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     grid_dependency_wait();
     const int n_items = p.counters->nitems;
     const int n_rounds = (n_items + (int)gridDim.x - 1) / (int)gridDim.x;
+    // Pass 0 goes through all of the CTA's items, pass 1 (bf16) through those that the epilogue has marked.
+    auto item_at = [&](auto pass_c, int kr) -> int {  // the list's index of round kr, past the end where the pass leaves it out
+        if constexpr (decltype(pass_c)::value == 1) {
+            const int bit = kr % kRedoBits;
+            if (!((redo_bits[bit >> 5] >> (bit & 31)) & 1u)) return n_items;
+        }
+        return cta_item_index(kr, blockIdx.x, gridDim.x);
+    };
+    // Every role between its two passes: whether there is a second one.
+    auto second_pass = [&]() -> bool {
+        return mbar_wait(smem_u32(&bars.pass_done), 0, abortp) && *reinterpret_cast<volatile uint32_t*>(&redo_any) != 0;
+    };
 
     if (warp >= 12) {
         // =========================== epilogue warpgroup ===========================
@@ -1550,11 +1591,12 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // them.  From TMEM: TMA into one buffer one item ahead, then to TMEM through this warpgroup's registers. ----
         int kq = 0;       // round of the next Q tile to load
         uint32_t nq = 0;  // Q tiles loaded so far
-        auto load_q = [&]() {  // lane 0 of the warpgroup's first warp issues; every thread follows the item list
+        bool arrived = false;  // at pass_done
+        auto load_q = [&](auto pass_c) {  // lane 0 of the warpgroup's first warp issues; every thread follows the item list
             WorkItem w;
             do {
                 if (kq >= n_rounds) return;
-                w = load_item(p.items, cta_item_index(kq++, blockIdx.x, gridDim.x), n_items);
+                w = load_item(p.items, item_at(pass_c, kq++), n_items);
             } while (w.ntiles <= 0);
             const uint32_t b = kOwnO ? (nq & 1u) : 0u;
             if (tw == 0) {
@@ -1564,21 +1606,21 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             ++nq;
         };
         uint32_t sq = 0;  // Q tiles moved to TMEM
-        auto stage_q = [&]() -> bool {
+        auto stage_q = [&](auto pass_c) -> bool {
             bool good = mbar_wait(smem_u32(&bars.q_full[0]), sq & 1, abortp);
             good = good && mbar_wait(smem_u32(&bars.q_free), (sq & 1) ^ 1, abortp);
             if (!__all_sync(0xffffffffu, good)) return false;
             tc_fence_after();
             const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + Cols::kQ;
 #pragma unroll 1
-            for (int s = 0; s < NSUB; ++s) {  // 64 head-dimension columns: eight swizzled 16-byte chunks of this row
-                uint32_t v[32];
+            for (int s = 0; s < 2 * NSUB; ++s) {  // 32 head-dimension columns: four swizzled 16-byte chunks of this row
+                uint32_t v[16];
 #pragma unroll
-                for (int c = 0; c < 8; ++c) {
-                    const uint4 w = *reinterpret_cast<const uint4*>(sQ + s * Q_SUB + tw * 128 + ((c ^ (tw & 7)) << 4));
+                for (int c = 0; c < 4; ++c) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(sQ + (s >> 1) * Q_SUB + tw * 128 + ((((s & 1) * 4 + c) ^ (tw & 7)) << 4));
                     v[4 * c] = w.x; v[4 * c + 1] = w.y; v[4 * c + 2] = w.z; v[4 * c + 3] = w.w;
                 }
-                tmem_st32(t_q + s * 32, v);
+                tmem_st16(t_q + s * 16, v);
             }
             mbar_arrive(smem_u32(&bars.q_drained));
             tc_wait_st();
@@ -1587,20 +1629,23 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if (tw == 0) good = mbar_wait(smem_u32(&bars.q_drained), sq & 1, abortp);  // then the next Q tile may land
             if (!__all_sync(0xffffffffu, good)) return false;
             ++sq;
-            load_q();
+            load_q(pass_c);
             return true;
         };
-        if constexpr (kOwnO || !kSmemQ) load_q();
-        if constexpr (kOwnO) load_q();
-        WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
+        const auto run = [&](auto pass_c) {
+        constexpr int pass = decltype(pass_c)::value;
+        kq = 0;
+        if constexpr (kOwnO || !kSmemQ) load_q(pass_c);
+        if constexpr (kOwnO) load_q(pass_c);
+        WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
         for (int kr = 0; kr < n_rounds && ok; ++kr) {
             const WorkItem it = it_next;
-            it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
+            it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
             const int row = it.q_tile * kTQ + tw;
             const bool row_ok = row < p.N;
             if (it.ntiles < 0) continue;  // past the end of the list
             if (it.ntiles == 0) {  // no active column: zero output, LSE = -inf
-                if (row_ok) {
+                if (row_ok && pass == 0) {
                     uint4* o = reinterpret_cast<uint4*>(p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row));
 #pragma unroll
                     for (int c = 0; c < D / 8; ++c) o[c] = make_uint4(0, 0, 0, 0);
@@ -1611,17 +1656,18 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); the one TMEM buffer is
             // free after this item's last Q K^T, which comes well before its last P V
             if constexpr (!kSmemQ) {
-                while (ok && nq > sq && sq <= itn + 1) ok = stage_q();
+                while (ok && nq > sq && sq <= itn + 1) ok = stage_q(pass_c);
                 if (!ok) break;
             }
             ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
             if (!ok) break;
-            if constexpr (kOwnO) load_q();  // this item's scores have all been read: its buffer is free for the item after next
+            if constexpr (kOwnO) load_q(pass_c);  // this item's scores have all been read: its buffer is free for the item after next
             // d = 64: weights of the accumulator of the item's first tile (a) and of the other one (b).  Which warpgroup took
             // the first tile follows from the tiles this CTA had before, so everything below goes by a and b and not by
             // warpgroup: an item's bits are the same wherever it stands in a CTA's list.
             const uint32_t first = g_start & 1u;
             float l_tot, m_final, wa = 1.f, wb = 1.f;
+            bool doubtful = false;
             if constexpr (kOwnO) {
                 const float ma = __uint_as_float(mref[first][tw]), mb = __uint_as_float(mref[first ^ 1u][tw]);
                 m_final = fmaxf(ma, mb);
@@ -1631,8 +1677,27 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             } else {
                 l_tot = lfin[0][tw] + lfin[1][tw];
                 m_final = mfin[tw];
+                if (kFirstRef && pass == 0) doubtful = row_ok && sum_is_doubtful(l_tot);
             }
             mbar_arrive(smem_u32(&bars.e_taken));
+            // An accumulator can overflow only where the weights are far above those of a reference that follows the maximum:
+            // then its values decide as well.  Otherwise the verdict is in before the item's stores, which an arrival behind
+            // them would wait for.
+            const bool big = kFirstRef && pass == 0 && __any_sync(0xffffffffu, l_tot > 33554432.f);
+            const auto mark = [&]() {
+                if (__any_sync(0xffffffffu, doubtful) && lane == 0) {
+                    const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
+                    atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
+                    redo_any = 1u;
+                }
+            };
+            if (kFirstRef && pass == 0 && !big) {
+                mark();
+                if (kr == n_rounds - 1) {
+                    mbar_arrive(smem_u32(&bars.pass_done));
+                    arrived = true;
+                }
+            }
             const float inv_l = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
             const float lse = (l_tot > 0.f) ? fmaf(m_final, 0.6931471805599453f, logf(l_tot)) : -INFINITY;
             if (lane == 0) BSA_TRACE_POINT(11, tn, 32);
@@ -1647,6 +1712,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             const int n_tiles = tiles_of<G>(it.ntiles);  // 1: the other accumulator is stale
             g_start += (uint32_t)n_tiles;
             const float sa = inv_l * wa, sb = inv_l * wb;
+            float nonfinite = 0.f;
 #pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
             for (int c = 0; c < D / CW; ++c) {
                 uint32_t o[CW];
@@ -1665,6 +1731,10 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     tc_wait_ld();
 #pragma unroll
                     for (int e = 0; e < CW; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * sa);
+                }
+                if (kFirstRef && pass == 0 && big) {  // zero as long as every output is finite
+#pragma unroll
+                    for (int e = 0; e < CW; ++e) nonfinite = fmaf(__uint_as_float(o[e]), 0.f, nonfinite);
                 }
                 if (c == D / CW - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
                     tc_fence_before();
@@ -1701,6 +1771,18 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 p.ws_LSE[(size_t)it.ws_slot * kTQ + tw] = lse;
             }
             if (lane == 0) BSA_TRACE_POINT(11, tn, 34);
+            if (kFirstRef && pass == 0 && big) {
+                doubtful = doubtful || (row_ok && !(nonfinite == 0.f));
+                mark();
+            }
+        }
+        };
+        run(IntC<0>());
+        if constexpr (kFirstRef) {
+            if (ok) {
+                if (!arrived) mbar_arrive(smem_u32(&bars.pass_done));
+                if (__all_sync(0xffffffffu, second_pass())) run(IntC<1>());
+            }
         }
         if (!ok && tw == 0) {  // a Q tile in flight lands before the CTA's shared memory goes away
             const uint64_t t0 = globaltimer_ns();
@@ -1718,10 +1800,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             RingPos ring;  // K ring position of tile g
             bool ok = true;
             BSA_TRACE_DECL(tn);
-            WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
+            const auto run = [&](auto pass_c) {
+            WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const WorkItem it = it_next;
-                it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
+                it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
                 if (it.ntiles <= 0) continue;
                 TileKeys<G, GK> next;
                 next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
@@ -1753,6 +1836,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     BSA_TRACE_POINT(0, tn, 21);
                 }
             }
+            };
+            run(IntC<0>());
+            if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
             if (!ok) {
                 const uint64_t t0 = globaltimer_ns();
                 while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
@@ -1763,10 +1849,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             RingPos ring;  // V ring position of tile g
             bool ok = true;
             const bool withhold = *reinterpret_cast<volatile int*>(&g_withhold_arrival) != 0;  // test hook, see above
-            WorkItem it_next = load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
+            const auto run = [&](auto pass_c) {
+            WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const WorkItem it = it_next;
-                it_next = load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items);
+                it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
                 if (it.ntiles <= 0) continue;
                 TileKeys<G, GK> next;
                 next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
@@ -1785,6 +1872,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                                     cur.key0[e], 0, it.head);
                 }
             }
+            };
+            run(IntC<0>());
+            if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
             if (!ok) {
                 const uint64_t t0 = globaltimer_ns();
                 while (globaltimer_ns() - t0 < 200000ull) __nanosleep(1000);
@@ -1799,10 +1889,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             bool ok = true;
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
-            int n_next = tiles_of<G>(load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles);
+            const auto run = [&](auto pass_c) {
+            int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const int n = n_next;
-                n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
+                n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
                 if (n <= 0) continue;
                 const uint32_t qb = kSmemQ ? (itq & 1u) : 0u;  // this item's Q buffer
                 ok = kSmemQ ? mbar_wait(smem_u32(&bars.q_full[qb]), (itq >> 1) & 1, abortp)
@@ -1845,6 +1936,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 g += n;
                 ++itq;
             }
+            };
+            run(IntC<0>());
+            if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
 #ifdef BSA_PHASES
             if (blockIdx.x == 1) { g_trace[0][0] = ph_acc[0]; g_trace[0][1] = ph_acc[1]; g_trace[0][8] = ph_n; }
 #endif
@@ -1857,10 +1951,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             bool ok = true;
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
-            int n_next = tiles_of<G>(load_item(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items).ntiles);
+            const auto run = [&](auto pass_c) {
+            int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
             for (int kr = 0; kr < n_rounds && ok; ++kr) {
                 const int n = n_next;
-                n_next = tiles_of<G>(load_item(p.items, cta_item_index(kr + 1, blockIdx.x, gridDim.x), n_items).ntiles);
+                n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
                 if (n <= 0) continue;
                 for (int j = 0; j < n; ++j, ring.advance(NSV)) {
                     const uint32_t gp = g + j;
@@ -1898,6 +1993,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 g += n;
                 ++itq;
             }
+            };
+            run(IntC<0>());
+            if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
 #ifdef BSA_PHASES
             if (blockIdx.x == 1) { g_trace[1][0] = ph_acc[0]; g_trace[1][1] = ph_acc[1]; g_trace[1][8] = ph_n; }
 #endif
@@ -1913,6 +2011,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const uint32_t t_o = tmem + lane_base + (x ? Cols::kO1 : Cols::kO0);
         uint32_t g = 0;          // running tile index at the start of the current item (all warpgroups agree)
         uint32_t itn = 0;        // non-empty items finished
+        uint32_t g0 = 0;         // running tile index at the start of this pass
         bool ok = true;
         BSA_TRACE_DECL(tn);
         const float c2 = p.scale_log2;
@@ -1935,7 +2034,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         // The reference after global tile t (taken by the other warpgroup), given a word read earlier from its slot:
         // if that word already carries the publish's tag it is used, else the slot is polled (bounded).
         auto take_reference = [&](uint32_t t, uint32_t word, float& m_out) -> bool {
-            const uint32_t tag = ((t >> 1) + 1) & 3u;
+            const uint32_t tag = ((t >> 1) - (g0 >> 1) + 1) & 3u;
             if ((word & 3u) != tag) {
                 volatile uint32_t* slot = &mref[x ^ 1][tw];
                 long long t0 = 0;
@@ -1957,10 +2056,31 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             m_out = __uint_as_float(word & ~3u);
             return true;
         };
+        // polls a reference's word until it carries the tag (bounded)
+        auto take_word = [&](volatile uint32_t* slot, uint32_t tag, float& m_out) -> bool {
+            uint32_t word = *slot;
+            long long t0 = 0;
+            for (uint32_t spins = 1; (word & 3u) != tag; ++spins) {
+                if ((spins & 63u) == 0) {
+                    if (*abortp) return false;
+                    const long long now = clock64();
+                    if (t0 == 0) t0 = now;
+                    if (now - t0 > *reinterpret_cast<volatile long long*>(&g_wait_limit_cycles)) {
+                        *abortp = 1;
+                        return false;
+                    }
+                }
+                word = *slot;
+            }
+            m_out = __uint_as_float(word & ~3u);
+            return true;
+        };
+        bool again = true;
+        if constexpr (kFirstRef) {
         // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
         // item nor the metadata that depends on it is waited for at an item boundary
-        ItemSpan it_next = load_item_span(p.items, cta_item_index(0, blockIdx.x, gridDim.x), n_items);
-        ItemSpan it_next2 = load_item_span(p.items, cta_item_index(1, blockIdx.x, gridDim.x), n_items);
+        ItemSpan it_next = load_item_span(p.items, item_at(IntC<0>(), 0), n_items);
+        ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<0>(), 1), n_items);
         int last_col = 0;
         uint32_t first_word = 0;
         {
@@ -1971,7 +2091,186 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         for (int kr = 0; kr < n_rounds && ok; ++kr) {
             const ItemSpan it = it_next;
             it_next = it_next2;
-            it_next2 = load_item_span(p.items, cta_item_index(kr + 2, blockIdx.x, gridDim.x), n_items);
+            it_next2 = load_item_span(p.items, item_at(IntC<0>(), kr + 2), n_items);
+            const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
+            uint32_t word_next = first_word;
+            // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
+            const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
+            {   // the next item's first tile of this warpgroup: its parity follows from g + n
+                const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
+                first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+                if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
+            }
+            if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
+            float m_ref = -INFINITY, l = 0.f;
+            bool settled = false;  // every row of the warp has its reference
+            // first local tile index of this warpgroup inside the item
+            const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
+            for (int j = j0; j < n; j += 2) {
+                const uint32_t gs = g + j;
+                uint32_t ballot = full_ballot;
+                if (G > 1 || has_bits) {
+                    ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
+                    if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
+                }
+                const bool need_mask = ballot != full_ballot;
+                const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
+                const bool ragged = (j == n - 1) && n_valid < TK;
+                if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
+                BSA_PH(7);
+                ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
+                if (!ok) break;
+                BSA_PH(0);
+                if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
+                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 10);
+                tc_fence_after();
+                uint32_t r[TK];
+#pragma unroll
+                for (int c = 0; c < TK / 32; ++c) tmem_ld32(t_s + c * 32, &r[c * 32]);
+                tc_wait_ld();
+                BSA_PH(1);
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bars.s_free[x]));  // S[x] is in registers: the next Q K^T into it may start
+                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
+                if (need_mask) {
+                    // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
+                    // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
+#pragma unroll
+                    for (int gq = 0; gq < TK / 16; ++gq) {
+                        const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
+#pragma unroll
+                        for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
+                    }
+                }
+                if (ragged) {
+#pragma unroll
+                    for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
+                }
+                if (!settled) {  // the item's first tile, and where some row has not been reached yet
+                    float m_prev = -INFINITY;
+                    if (j > 0) {  // (published, since this warp is not settled; its slot is not written again before this tile's P V)
+                        ok = __all_sync(0xffffffffu, take_word(&mref[itn & 1][tw], (j == 1) ? (itn >> 1) & 1u : 2u + (j & 1u), m_prev));
+                        if (!ok) break;
+                    }
+                    if (!__all_sync(0xffffffffu, m_prev != -INFINITY)) {
+                        float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+                        for (int i = 0; i < TK; i += 8) {
+                            m0 = max3(m0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+                            m1 = max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+                            m2 = max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
+                            m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
+                        }
+                        const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
+                        if (m_prev == -INFINITY) m_prev = __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
+                        *reinterpret_cast<volatile uint32_t*>(&mref[itn & 1][tw]) =
+                            __float_as_uint(m_prev) | ((j == 0) ? (itn >> 1) & 1u : 3u - (j & 1u));
+                    }
+                    m_ref = m_prev;
+                    settled = __all_sync(0xffffffffu, m_ref != -INFINITY);
+                }
+                const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
+                const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
+                uint64_t sum01 = pack_f32x2(0.f, 0.f), sum23 = sum01;
+                // P[x] was last read by the P V of tile gs-2 (normally long complete).  With d = 64 it is waited for
+                // here and the P tile stored 32 columns at a time while the next columns are still being exponentiated
+                // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
+                constexpr bool kStoreInLoop = (D == 64);
+                if (kStoreInLoop && gs >= 2) {
+                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
+                    if (!ok) break;
+                    tc_fence_after();
+                }
+#pragma unroll
+                for (int i = 0; i < TK; i += 4) {
+                    float x0, x1, x2, x3;
+                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), c22, nm2), x0, x1);
+                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), c22, nm2), x2, x3);
+                    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
+                    sum01 = add_f32x2(sum01, pack_f32x2(p0, p1));
+                    sum23 = add_f32x2(sum23, pack_f32x2(p2, p3));
+                    r[i / 2] = pack_16x2<F16>(p0, p1);
+                    r[i / 2 + 1] = pack_16x2<F16>(p2, p3);
+                    if (kStoreInLoop && (i & 31) == 28) tmem_st16(t_p + (i >> 5) * 16, &r[(i >> 5) * 16]);
+                }
+                float s0, s1, s2, s3;
+                unpack_f32x2(sum01, s0, s1);
+                unpack_f32x2(sum23, s2, s3);
+                l += (s0 + s1) + (s2 + s3);
+#ifdef BSA_PHASES
+                {
+                    float f0_ = l;
+                    uint32_t u0_ = r[TK / 2 - 1];
+                    asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+r"(u0_));
+                }
+#endif
+                BSA_PH(4);
+                if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
+                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
+                if (!kStoreInLoop) {
+                    if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+                    BSA_PH(5);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
+#pragma unroll
+                    for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
+                }
+                tc_wait_st();
+                tc_fence_before();
+                mbar_arrive(smem_u32(&bars.p_ready[x]));
+                BSA_PH(6);
+                if (lane == 0) BSA_STAMP(2 + warp, gs, 3);
+#ifdef BSA_PHASES
+                ++ph_n;
+#endif
+                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 16);
+            }
+            if (!ok) break;
+            // ---- hand this warpgroup's row sums to the epilogue warpgroup ----
+            {
+                // the previous item's sums must have been read
+                ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
+                if (!ok) break;
+                lfin[x][tw] = l;
+                if (((g + n - 1) & 1) == (uint32_t)x) mfin[tw] = m_ref;  // whoever took the last tile knows the reference of every row
+                mbar_arrive(smem_u32(&bars.e_ready));
+                ++itn;
+                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
+            }
+            g += n;
+            BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
+        }
+        // ---- pass 1: the items whose first reference did not serve, with a reference that follows the running maximum ----
+        if (ok) {
+            mbar_arrive(smem_u32(&bars.pass_done));
+            again = __all_sync(0xffffffffu, second_pass());
+            if (!kOwnO && again) {  // everything has been read: the tags start over
+                mref[x][tw] = 0u;
+                mbar_arrive(smem_u32(&bars.tags_reset));
+                again = ok = mbar_wait_warp(smem_u32(&bars.tags_reset), 0, abortp);
+            }
+        }
+        }
+        g0 = g;
+        if (ok && again) {
+        // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
+        // item nor the metadata that depends on it is waited for at an item boundary
+        ItemSpan it_next = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 0), n_items);
+        ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 1), n_items);
+        int last_col = 0;
+        uint32_t first_word = 0;
+        {
+            const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
+            first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+            if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
+        }
+        for (int kr = 0; kr < n_rounds && ok; ++kr) {
+            const ItemSpan it = it_next;
+            it_next = it_next2;
+            it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), kr + 2), n_items);
             const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
             uint32_t word_next = first_word;
             // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
@@ -2045,9 +2344,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 if constexpr (!kOwnO) {
                     // ---- reference maximum handed over from the previous tile (other warpgroup) ----
                     float m_prev = -INFINITY;
-                    if (gs > 0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
+                    if (gs > g0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
                         float m_taken;
-                        if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) + 1) & 3u))) {
+                        if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) - (g0 >> 1) + 1) & 3u))) {
                             m_taken = __uint_as_float(ref_word & ~3u);
                         } else {
                             ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
@@ -2082,7 +2381,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 if constexpr (!kOwnO) {
                     // publish: the next tile's warpgroup may take its decision
-                    *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) + 1) & 3u);
+                    *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) - (g0 >> 1) + 1) & 3u);
                 }
                 BSA_PH(3);
                 const float neg_m = (m_know == -INFINITY) ? 0.f : -m_know;
@@ -2136,7 +2435,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 // ---- the reference moved at this tile: rescale the running output (its last P V has been waited for above) ----
                 if (j > 0 && __any_sync(0xffffffffu, rescale)) {
-                    if constexpr (!kOwnO && !kSmemQ) {  // (returns at once; without it ptxas spills in the gathered kernels)
+                    if constexpr (!kOwnO && (!kSmemQ || kFirstRef)) {  // (returns at once; without it ptxas spills in the gathered kernels)
                         ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
                         if (!ok) break;
                         tc_fence_after();
@@ -2185,6 +2484,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             }
             g += n;
             BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
+        }
         }
 #ifdef BSA_PHASES
         if (blockIdx.x == 1 && lane == 0) {
