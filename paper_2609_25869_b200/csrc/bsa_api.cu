@@ -87,6 +87,7 @@ struct bsa_plan {
     // measured there).  Exact where no dimension is Coarsened; a Coarsened list is taken to be that of independent blocks, at
     // most the true length's multiple by the blocks per tile, on a line where the two forms are within 2 % of each other.
     int32_t short_lists;
+    int32_t long_lists;  // 32 tiles and more, on the same estimate: the form of the ping-pong kernel at d = 64 follows from it
     // Split-K workspace
     float* ws_O;
     float* ws_LSE;
@@ -457,6 +458,7 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
         const double entries = (double)g.nKt * (1.0 - pow(1.0 - density, (double)(g.sQ * g.sK)));
         const double parts = pmax > 1 ? fmin((double)pmax, fmax(1.0, entries / p->desc.split_tau)) : 1.0;
         p->short_lists = entries * p->desc.T_KV < 8.0 * 128.0 * parts;
+        p->long_lists = entries * p->desc.T_KV >= 32.0 * 128.0 * parts;
     }
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
@@ -650,6 +652,7 @@ static void fill_forward_args(const bsa_plan_t* p, const void* Q, const void* K,
     a.kernel = p->desc.kernel;
     a.has_split = p->desc.split_pmax > 1;
     a.short_lists = p->short_lists;
+    a.long_lists = p->long_lists;
     a.max_items = (int32_t)(p->max_items < (1 << 30) ? p->max_items : (1 << 30));
     a.max_split_rows = p->g.H * p->g.nQt * p->g.slots;
     a.num_sms = p->num_sms;

@@ -1343,18 +1343,20 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // (the V ring gives up one of its four), loaded by the K producer.  Forward at 32768 tokens, 8 heads, n tiles per item,
 // TMEM / shared memory in us: n = 1 46.8 / 41.4, 2 55.4 / 52.1, 3 68.3 / 66.0, 4 81.3 / 79.7, 6 107.6 / 106.1; at 16384
 // tokens 8 67.5 / 67.5, 12 93.4 / 93.9.  Hence shared memory below eight tiles per item on average (bsa_plan::short_lists).
-// Reference maximum at d = 128, bf16, long lists (kFirstRef): the maximum of the first tile that reaches a row serves the
+// Reference maximum in bf16 on long lists (kFirstRef): the maximum of the first tile that reaches a row serves the
 // whole item.  bf16 and fp32 keep their relative precision over 2^100, so it does not matter how far later scores lie above
 // it; from its second tile on a softmax warpgroup neither looks for maxima (64 instructions and about 300 clk per tile) nor
 // takes and publishes a word per row and tile, and nothing is rescaled.  Where it fails (a row sum beyond 2^100 or undefined,
 // or an accumulator that overflows) the epilogue marks the item, and a second pass over the marked items follows the running
 // maximum as before, moved by more than 2^8 at a time.  Per 128-key tile the softmax chain falls by a fifth.  Builds in turn,
 // back to back, before / after: 16384 tokens, 8 heads, (128,128) 153.5 / 144.4 us; 115200, 4 heads 1840 / 1725; 75600, 6
-// heads, (64,64) 3650 / 3510, 4 heads, (32,32) 4560 / 3700.  Half has no such range.  Short lists (Q in shared memory) and
-// d = 64 keep the running maximum: there the second copy of the loop costs more than it saves (32768 tokens, 8 heads, two
-// tiles per item 74 -> 82 us; 2048 tokens, 2 heads, d = 64 16.5 -> 18.5; (64,64) blocks at d = 64, 32768 tokens, 16 heads
-// 1310 -> 1430).  Both kernels take a row's reference from the same tile, so that an item whose scores do not outgrow it by
-// 2^8 has the same bits in either.
+// heads, (64,64) 3650 / 3510, 4 heads, (32,32) 4560 / 3700.  At d = 64 (each warpgroup has its own) on lists of 32
+// tiles and more: 32768 tokens, 16 heads, (256,256) 1230 / 1190; 8 heads, (32,32) 1218 / 1089; 23296 tokens, 2 heads, (256,256)
+// at 44 % 276 / 215.  The running maximum stays for half, which has no such range, and for short lists, where the second copy
+// of the loop costs more than it saves (d = 128, 32768 tokens, 8 heads, two tiles per item 74 -> 82 us; d = 64, 2048 tokens, 2
+// heads 16.5 -> 18.5, 10240 tokens, 8 heads, 9 tiles of runs 55 -> 63; 16384 tokens, 16 heads, (32,32), 15 tiles 244 -> 250);
+// at d = 64 also for tiles of two entries ((64,64) at 48 tiles 1360 -> 1440).  Both forms take a row's reference from the same
+// tile, so that an item whose scores do not outgrow it by 2^8 has the same bits in either.
 // Two kernels and not a flag in one: what an item pays at its boundary is mostly instruction fetch, and the softmax code
 // has no register to spare (one kernel with both bodies was 1-2 % slower on long lists).
 //
@@ -1467,7 +1469,7 @@ struct TileKeys {
     }
 };
 
-template <int D, bool F16, int G, bool kSmemQ>
+template <int D, bool F16, int G, bool kShort>
 __global__ void __launch_bounds__(kPpThreads, 1)
 bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -1480,9 +1482,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     constexpr int GV_TILE = KV_TILE / G;
     constexpr int V_SUB = (G == 1) ? KV_SUB : GK * 128;  // a V tile holds its entries one after the other
     using Cols = PpCols<D>;
+    constexpr bool kSmemQ = kShort || D == 64;  // (at d = 64 no tensor-memory columns are left for Q)
     constexpr bool kOwnO = Cols::kOwnO;
-    constexpr bool kFirstRef = !F16 && !kSmemQ;  // a row's first reference serves the whole item (see above)
-    static_assert(!kOwnO || kSmemQ, "d = 64 has no tensor-memory columns left for Q");
+    constexpr bool kFirstRef = !F16 && !kShort;  // a row's first reference serves the whole item (see above)
     static_assert(kOwnO || NSUB * Q_SUB == KV_TILE, "at d = 128 the second Q tile takes the place of a V tile");
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -1674,6 +1676,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 wa = (ma == -INFINITY) ? 0.f : ex2_approx(ma - m_final);
                 wb = (mb == -INFINITY) ? 0.f : ex2_approx(mb - m_final);
                 l_tot = fmaf(lfin[first ^ 1u][tw], wb, lfin[first][tw] * wa);
+                if (kFirstRef && pass == 0) doubtful = row_ok && (sum_is_doubtful(lfin[0][tw]) || sum_is_doubtful(lfin[1][tw]));
             } else {
                 l_tot = lfin[0][tw] + lfin[1][tw];
                 m_final = mfin[tw];
@@ -2148,7 +2151,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 }
                 if (!settled) {  // the item's first tile, and where some row has not been reached yet
                     float m_prev = -INFINITY;
-                    if (j > 0) {  // (published, since this warp is not settled; its slot is not written again before this tile's P V)
+                    if (kOwnO) m_prev = m_ref;
+                    else if (j > 0) {  // (published, since this warp is not settled; its slot is not written again before this tile's P V)
                         ok = __all_sync(0xffffffffu, take_word(&mref[itn & 1][tw], (j == 1) ? (itn >> 1) & 1u : 2u + (j & 1u), m_prev));
                         if (!ok) break;
                     }
@@ -2162,8 +2166,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
                         }
                         const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
-                        if (m_prev == -INFINITY) m_prev = __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
-                        *reinterpret_cast<volatile uint32_t*>(&mref[itn & 1][tw]) =
+                        if (m_prev == -INFINITY) m_prev = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
+                        if (!kOwnO) *reinterpret_cast<volatile uint32_t*>(&mref[itn & 1][tw]) =
                             __float_as_uint(m_prev) | ((j == 0) ? (itn >> 1) & 1u : 3u - (j & 1u));
                     }
                     m_ref = m_prev;
@@ -2235,7 +2239,8 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
                 if (!ok) break;
                 lfin[x][tw] = l;
-                if (((g + n - 1) & 1) == (uint32_t)x) mfin[tw] = m_ref;  // whoever took the last tile knows the reference of every row
+                if (kOwnO) mref[x][tw] = __float_as_uint(m_ref);
+                else if (((g + n - 1) & 1) == (uint32_t)x) mfin[tw] = m_ref;  // whoever took the last tile knows the reference of every row
                 mbar_arrive(smem_u32(&bars.e_ready));
                 ++itn;
                 if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
@@ -2662,8 +2667,10 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
             const auto allow = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
             e = allow(bsa_attention_pp_kernel<D, false, G, true>);
             if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, true>);
-            if constexpr (D != 64) {
+            if constexpr (D != 64 || G != 2) {
                 if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, false, G, false>);
+            }
+            if constexpr (D != 64) {
                 if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, false>);
             }
         }
@@ -2700,11 +2707,15 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         const auto launch = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, tq, tk, tv, p); };
-        cudaError_t le;
-        if (D == 64 || (a.short_lists && p.stages == 2 && p.stages_v > 2)) {  // (the K producer relies on the two K tiles)
+        cudaError_t le = cudaErrorInvalidValue;
+        // (at d = 128 the K producer of the short form relies on the two K tiles)
+        const bool short_form = D == 64 ? (G == 2 || a.f16 || !a.long_lists) : (a.short_lists && p.stages == 2 && p.stages_v > 2);
+        if (short_form) {
             le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, true>) : launch(bsa_attention_pp_kernel<D, false, G, true>);
         } else if constexpr (D != 64) {
             le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, false>) : launch(bsa_attention_pp_kernel<D, false, G, false>);
+        } else if constexpr (G != 2) {
+            le = launch(bsa_attention_pp_kernel<D, false, G, false>);
         }
         count_launch();
         return le;

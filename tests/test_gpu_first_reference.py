@@ -11,22 +11,22 @@ from tests import helpers as Hh
 pytestmark = pytest.mark.gpu
 
 
-def _request(B, N_kv, late_rows, seed=5):
-    """Three heads of 300 query rows, about 20 tiles per item: Q goes through tensor memory."""
+def _request(B, N_kv, late_rows, seed=5, d=128):
+    """Three heads of 300 query rows, lists long enough for the form that keeps a row's first reference."""
     N = 300
     nq, nk = I.cdiv(N, B), I.cdiv(N_kv, B)
     M = I.random_mask(seed + B, 3, nq, nk, 0.8, empty_rows=0.1)
     if late_rows:  # every other row block is reached by the last blocks only, its neighbours from the first on
         M[:, ::2, : nk - 3] = 0
         M[:, 1::2] = 1
-    return I.Request("first", 3, N, 128, B, B, M, qkv_seed=seed, N_kv=N_kv)
+    return I.Request("first", 3, N, d, B, B, M, qkv_seed=seed, N_kv=N_kv)
 
 
-@pytest.mark.parametrize("B,plan_id", [(128, 22), (64, 23), (32, 39)])
+@pytest.mark.parametrize("B,plan_id,d", [(128, 22, 128), (64, 23, 128), (32, 39, 128), (128, 22, 64), (32, 39, 64)])
 @pytest.mark.parametrize("late_rows", [False, True])
 @pytest.mark.parametrize("top", [1.0, 8.0, 60.0])  # scores up to about 5, 40 and 300 (in units of e)
-def test_scores_that_outgrow_the_first_tile(B, plan_id, late_rows, top):
-    req = _request(B, 25 * 128 - 7, late_rows)
+def test_scores_that_outgrow_the_first_tile(B, plan_id, d, late_rows, top):
+    req = _request(B, (25 if d == 128 else 45) * 128 - 7, late_rows, d=d)
     q, k, v = req.qkv()
     scale = torch.ones(req.n_kv)
     scale[-200:] = top
