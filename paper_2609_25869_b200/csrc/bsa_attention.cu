@@ -1635,150 +1635,150 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             return true;
         };
         const auto run = [&](auto pass_c) {
-        constexpr int pass = decltype(pass_c)::value;
-        kq = 0;
-        if constexpr (kOwnO || !kSmemQ) load_q(pass_c);
-        if constexpr (kOwnO) load_q(pass_c);
-        WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
-        for (int kr = 0; kr < n_rounds && ok; ++kr) {
-            const WorkItem it = it_next;
-            it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
-            const int row = it.q_tile * kTQ + tw;
-            const bool row_ok = row < p.N;
-            if (it.ntiles < 0) continue;  // past the end of the list
-            if (it.ntiles == 0) {  // no active column: zero output, LSE = -inf
-                if (row_ok && pass == 0) {
-                    uint4* o = reinterpret_cast<uint4*>(p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row));
+            constexpr int pass = decltype(pass_c)::value;
+            kq = 0;
+            if constexpr (kOwnO || !kSmemQ) load_q(pass_c);
+            if constexpr (kOwnO) load_q(pass_c);
+            WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
+            for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                const WorkItem it = it_next;
+                it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
+                const int row = it.q_tile * kTQ + tw;
+                const bool row_ok = row < p.N;
+                if (it.ntiles < 0) continue;  // past the end of the list
+                if (it.ntiles == 0) {  // no active column: zero output, LSE = -inf
+                    if (row_ok && pass == 0) {
+                        uint4* o = reinterpret_cast<uint4*>(p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row));
 #pragma unroll
-                    for (int c = 0; c < D / 8; ++c) o[c] = make_uint4(0, 0, 0, 0);
-                    p.LSE[(size_t)it.head * p.N + row] = -INFINITY;
-                }
-                continue;
-            }
-            // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); the one TMEM buffer is
-            // free after this item's last Q K^T, which comes well before its last P V
-            if constexpr (!kSmemQ) {
-                while (ok && nq > sq && sq <= itn + 1) ok = stage_q(pass_c);
-                if (!ok) break;
-            }
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
-            if (!ok) break;
-            if constexpr (kOwnO) load_q(pass_c);  // this item's scores have all been read: its buffer is free for the item after next
-            // d = 64: weights of the accumulator of the item's first tile (a) and of the other one (b).  Which warpgroup took
-            // the first tile follows from the tiles this CTA had before, so everything below goes by a and b and not by
-            // warpgroup: an item's bits are the same wherever it stands in a CTA's list.
-            const uint32_t first = g_start & 1u;
-            float l_tot, m_final, wa = 1.f, wb = 1.f;
-            bool doubtful = false;
-            if constexpr (kOwnO) {
-                const float ma = __uint_as_float(mref[first][tw]), mb = __uint_as_float(mref[first ^ 1u][tw]);
-                m_final = fmaxf(ma, mb);
-                wa = (ma == -INFINITY) ? 0.f : ex2_approx(ma - m_final);
-                wb = (mb == -INFINITY) ? 0.f : ex2_approx(mb - m_final);
-                l_tot = fmaf(lfin[first ^ 1u][tw], wb, lfin[first][tw] * wa);
-                if (kFirstRef && pass == 0) doubtful = row_ok && (sum_is_doubtful(lfin[0][tw]) || sum_is_doubtful(lfin[1][tw]));
-            } else {
-                l_tot = lfin[0][tw] + lfin[1][tw];
-                m_final = mfin[tw];
-                if (kFirstRef && pass == 0) doubtful = row_ok && sum_is_doubtful(l_tot);
-            }
-            mbar_arrive(smem_u32(&bars.e_taken));
-            // An accumulator can overflow only where the weights are far above those of a reference that follows the maximum:
-            // then its values decide as well.  Otherwise the verdict is in before the item's stores, which an arrival behind
-            // them would wait for.
-            const bool big = kFirstRef && pass == 0 && __any_sync(0xffffffffu, l_tot > 33554432.f);
-            const auto mark = [&]() {
-                if (__any_sync(0xffffffffu, doubtful) && lane == 0) {
-                    const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
-                    atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
-                    redo_any = 1u;
-                }
-            };
-            if (kFirstRef && pass == 0 && !big) {
-                mark();
-                if (kr == n_rounds - 1) {
-                    mbar_arrive(smem_u32(&bars.pass_done));
-                    arrived = true;
-                }
-            }
-            const float inv_l = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
-            const float lse = (l_tot > 0.f) ? fmaf(m_final, 0.6931471805599453f, logf(l_tot)) : -INFINITY;
-            if (lane == 0) BSA_TRACE_POINT(11, tn, 32);
-            ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_full), itn & 1, abortp));
-            if (!ok) break;
-            tc_fence_after();
-            if (lane == 0) BSA_TRACE_POINT(11, tn, 31);
-            ++itn;
-            __nv_bfloat16* orow = p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row);
-            float* wrow = p.ws_O + ((size_t)it.ws_slot * kTQ + tw) * D;
-            constexpr int CW = kOwnO ? 16 : 32;  // columns at a time
-            const int n_tiles = tiles_of<G>(it.ntiles);  // 1: the other accumulator is stale
-            g_start += (uint32_t)n_tiles;
-            const float sa = inv_l * wa, sb = inv_l * wb;
-            float nonfinite = 0.f;
-#pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
-            for (int c = 0; c < D / CW; ++c) {
-                uint32_t o[CW];
-                if constexpr (kOwnO) {
-                    uint32_t ob[CW];
-                    tmem_ld16(t_lane + (first ? Cols::kO1 : Cols::kO0) + c * CW, o);
-                    tmem_ld16(t_lane + (first ? Cols::kO0 : Cols::kO1) + c * CW, ob);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < CW; ++e) {
-                        const float a = __uint_as_float(o[e]) * sa;
-                        o[e] = __float_as_uint(n_tiles > 1 ? fmaf(__uint_as_float(ob[e]), sb, a) : a);
+                        for (int c = 0; c < D / 8; ++c) o[c] = make_uint4(0, 0, 0, 0);
+                        p.LSE[(size_t)it.head * p.N + row] = -INFINITY;
                     }
+                    continue;
+                }
+                // the next item's Q tile first (its Q K^T runs ahead of this item's softmax); the one TMEM buffer is
+                // free after this item's last Q K^T, which comes well before its last P V
+                if constexpr (!kSmemQ) {
+                    while (ok && nq > sq && sq <= itn + 1) ok = stage_q(pass_c);
+                    if (!ok) break;
+                }
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.e_ready), itn & 1, abortp));
+                if (!ok) break;
+                if constexpr (kOwnO) load_q(pass_c);  // this item's scores have all been read: its buffer is free for the item after next
+                // d = 64: weights of the accumulator of the item's first tile (a) and of the other one (b).  Which warpgroup took
+                // the first tile follows from the tiles this CTA had before, so everything below goes by a and b and not by
+                // warpgroup: an item's bits are the same wherever it stands in a CTA's list.
+                const uint32_t first = g_start & 1u;
+                float l_tot, m_final, wa = 1.f, wb = 1.f;
+                bool doubtful = false;
+                if constexpr (kOwnO) {
+                    const float ma = __uint_as_float(mref[first][tw]), mb = __uint_as_float(mref[first ^ 1u][tw]);
+                    m_final = fmaxf(ma, mb);
+                    wa = (ma == -INFINITY) ? 0.f : ex2_approx(ma - m_final);
+                    wb = (mb == -INFINITY) ? 0.f : ex2_approx(mb - m_final);
+                    l_tot = fmaf(lfin[first ^ 1u][tw], wb, lfin[first][tw] * wa);
+                    if (kFirstRef && pass == 0) doubtful = row_ok && (sum_is_doubtful(lfin[0][tw]) || sum_is_doubtful(lfin[1][tw]));
                 } else {
-                    tmem_ld32(t_lane + kColO + c * CW, o);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int e = 0; e < CW; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * sa);
+                    l_tot = lfin[0][tw] + lfin[1][tw];
+                    m_final = mfin[tw];
+                    if (kFirstRef && pass == 0) doubtful = row_ok && sum_is_doubtful(l_tot);
                 }
-                if (kFirstRef && pass == 0 && big) {  // zero as long as every output is finite
-#pragma unroll
-                    for (int e = 0; e < CW; ++e) nonfinite = fmaf(__uint_as_float(o[e]), 0.f, nonfinite);
+                mbar_arrive(smem_u32(&bars.e_taken));
+                // An accumulator can overflow only where the weights are far above those of a reference that follows the maximum:
+                // then its values decide as well.  Otherwise the verdict is in before the item's stores, which an arrival behind
+                // them would wait for.
+                const bool big = kFirstRef && pass == 0 && __any_sync(0xffffffffu, l_tot > 33554432.f);
+                const auto mark = [&]() {
+                    if (__any_sync(0xffffffffu, doubtful) && lane == 0) {
+                        const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
+                        atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
+                        redo_any = 1u;
+                    }
+                };
+                if (kFirstRef && pass == 0 && !big) {
+                    mark();
+                    if (kr == n_rounds - 1) {
+                        mbar_arrive(smem_u32(&bars.pass_done));
+                        arrived = true;
+                    }
                 }
-                if (c == D / CW - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
-                    tc_fence_before();
-                    mbar_arrive(smem_u32(&bars.o_free));
-                    if (lane == 0) BSA_TRACE_POINT(11, tn, 33);
-                }
-                if (it.nparts == 1) {
-                    if (row_ok) {  // 32-byte stores: every thread fills whole 32-byte sectors of its own row
+                const float inv_l = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
+                const float lse = (l_tot > 0.f) ? fmaf(m_final, 0.6931471805599453f, logf(l_tot)) : -INFINITY;
+                if (lane == 0) BSA_TRACE_POINT(11, tn, 32);
+                ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&bars.o_full), itn & 1, abortp));
+                if (!ok) break;
+                tc_fence_after();
+                if (lane == 0) BSA_TRACE_POINT(11, tn, 31);
+                ++itn;
+                __nv_bfloat16* orow = p.O + ((size_t)it.head * p.o_head + (size_t)row * p.o_row);
+                float* wrow = p.ws_O + ((size_t)it.ws_slot * kTQ + tw) * D;
+                constexpr int CW = kOwnO ? 16 : 32;  // columns at a time
+                const int n_tiles = tiles_of<G>(it.ntiles);  // 1: the other accumulator is stale
+                g_start += (uint32_t)n_tiles;
+                const float sa = inv_l * wa, sb = inv_l * wb;
+                float nonfinite = 0.f;
+#pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
+                for (int c = 0; c < D / CW; ++c) {
+                    uint32_t o[CW];
+                    if constexpr (kOwnO) {
+                        uint32_t ob[CW];
+                        tmem_ld16(t_lane + (first ? Cols::kO1 : Cols::kO0) + c * CW, o);
+                        tmem_ld16(t_lane + (first ? Cols::kO0 : Cols::kO1) + c * CW, ob);
+                        tc_wait_ld();
 #pragma unroll
-                        for (int q = 0; q < CW / 16; ++q) {
-                            uint32_t v[8];
+                        for (int e = 0; e < CW; ++e) {
+                            const float a = __uint_as_float(o[e]) * sa;
+                            o[e] = __float_as_uint(n_tiles > 1 ? fmaf(__uint_as_float(ob[e]), sb, a) : a);
+                        }
+                    } else {
+                        tmem_ld32(t_lane + kColO + c * CW, o);
+                        tc_wait_ld();
 #pragma unroll
-                            for (int e = 0; e < 8; ++e)
-                                v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]), __uint_as_float(o[q * 16 + 2 * e + 1]));
-                            if constexpr (kSmemQ) {  // (long lists: the branch is the cheaper form)
-                                st_global_v8_or_2v4(orow + c * CW + q * 16, v, p.o_wide);
-                            } else if (p.o_wide) {
-                                st_global_v8(orow + c * CW + q * 16, v);
-                            } else {
-                                uint4* dst = reinterpret_cast<uint4*>(orow + c * CW + q * 16);
-                                dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
-                                dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                        for (int e = 0; e < CW; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * sa);
+                    }
+                    if (kFirstRef && pass == 0 && big) {  // zero as long as every output is finite
+#pragma unroll
+                        for (int e = 0; e < CW; ++e) nonfinite = fmaf(__uint_as_float(o[e]), 0.f, nonfinite);
+                    }
+                    if (c == D / CW - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
+                        tc_fence_before();
+                        mbar_arrive(smem_u32(&bars.o_free));
+                        if (lane == 0) BSA_TRACE_POINT(11, tn, 33);
+                    }
+                    if (it.nparts == 1) {
+                        if (row_ok) {  // 32-byte stores: every thread fills whole 32-byte sectors of its own row
+#pragma unroll
+                            for (int q = 0; q < CW / 16; ++q) {
+                                uint32_t v[8];
+#pragma unroll
+                                for (int e = 0; e < 8; ++e)
+                                    v[e] = pack_16x2<F16>(__uint_as_float(o[q * 16 + 2 * e]), __uint_as_float(o[q * 16 + 2 * e + 1]));
+                                if constexpr (kSmemQ) {  // (long lists: the branch is the cheaper form)
+                                    st_global_v8_or_2v4(orow + c * CW + q * 16, v, p.o_wide);
+                                } else if (p.o_wide) {
+                                    st_global_v8(orow + c * CW + q * 16, v);
+                                } else {
+                                    uint4* dst = reinterpret_cast<uint4*>(orow + c * CW + q * 16);
+                                    dst[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                                    dst[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                                }
                             }
                         }
-                    }
-                } else {  // Split-K partial: normalised fp32 rows in the workspace
+                    } else {  // Split-K partial: normalised fp32 rows in the workspace
 #pragma unroll
-                    for (int q = 0; q < CW / 8; ++q) st_global_v8(wrow + c * CW + q * 8, o + q * 8);
+                        for (int q = 0; q < CW / 8; ++q) st_global_v8(wrow + c * CW + q * 8, o + q * 8);
+                    }
+                }
+                if (it.nparts == 1) {
+                    if (row_ok) p.LSE[(size_t)it.head * p.N + row] = lse;
+                } else {
+                    p.ws_LSE[(size_t)it.ws_slot * kTQ + tw] = lse;
+                }
+                if (lane == 0) BSA_TRACE_POINT(11, tn, 34);
+                if (kFirstRef && pass == 0 && big) {
+                    doubtful = doubtful || (row_ok && !(nonfinite == 0.f));
+                    mark();
                 }
             }
-            if (it.nparts == 1) {
-                if (row_ok) p.LSE[(size_t)it.head * p.N + row] = lse;
-            } else {
-                p.ws_LSE[(size_t)it.ws_slot * kTQ + tw] = lse;
-            }
-            if (lane == 0) BSA_TRACE_POINT(11, tn, 34);
-            if (kFirstRef && pass == 0 && big) {
-                doubtful = doubtful || (row_ok && !(nonfinite == 0.f));
-                mark();
-            }
-        }
         };
         run(IntC<0>());
         if constexpr (kFirstRef) {
@@ -1804,41 +1804,41 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             bool ok = true;
             BSA_TRACE_DECL(tn);
             const auto run = [&](auto pass_c) {
-            WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
-            for (int kr = 0; kr < n_rounds && ok; ++kr) {
-                const WorkItem it = it_next;
-                it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
-                if (it.ntiles <= 0) continue;
-                TileKeys<G, GK> next;
-                next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
-                for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSK)) {
-                    const TileKeys<G, GK> cur = next;
-                    if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
-                    const int stage = ring.stage;
-                    const uint32_t ph = ring.phase;
-                    BSA_TRACE_POINT(0, tn, 19);
-                    ok = mbar_wait(smem_u32(&bars.k_empty[stage]), ph ^ 1, abortp);
-                    if (!ok) break;
-                    BSA_TRACE_POINT(0, tn, 20);
-                    if (!kOwnO && kSmemQ && j == it.tile_begin) {
-                        const uint32_t b = itq++ & 1u;
-                        mbar_arrive_expect_tx(smem_u32(&bars.q_full[b]), NSUB * Q_SUB);
-                        tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, smem_u32(&bars.q_full[b]), 0, it.q_tile * kTQ, 0, it.head);
-                    }
-                    mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), KV_TILE);
-                    if constexpr (G == 1) {
-                        tma_load_4d(smem_u32(sK + stage * KV_TILE), &tmK, smem_u32(&bars.k_full[stage]), 0, cur.key0[0], 0, it.head);
-                    } else {
+                WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
+                for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                    const WorkItem it = it_next;
+                    it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
+                    if (it.ntiles <= 0) continue;
+                    TileKeys<G, GK> next;
+                    next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
+                    for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSK)) {
+                        const TileKeys<G, GK> cur = next;
+                        if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
+                        const int stage = ring.stage;
+                        const uint32_t ph = ring.phase;
+                        BSA_TRACE_POINT(0, tn, 19);
+                        ok = mbar_wait(smem_u32(&bars.k_empty[stage]), ph ^ 1, abortp);
+                        if (!ok) break;
+                        BSA_TRACE_POINT(0, tn, 20);
+                        if (!kOwnO && kSmemQ && j == it.tile_begin) {
+                            const uint32_t b = itq++ & 1u;
+                            mbar_arrive_expect_tx(smem_u32(&bars.q_full[b]), NSUB * Q_SUB);
+                            tma_load_4d(smem_u32(sQ + b * NSUB * Q_SUB), &tmQ, smem_u32(&bars.q_full[b]), 0, it.q_tile * kTQ, 0, it.head);
+                        }
+                        mbar_arrive_expect_tx(smem_u32(&bars.k_full[stage]), KV_TILE);
+                        if constexpr (G == 1) {
+                            tma_load_4d(smem_u32(sK + stage * KV_TILE), &tmK, smem_u32(&bars.k_full[stage]), 0, cur.key0[0], 0, it.head);
+                        } else {
 #pragma unroll
-                        for (int e = 0; e < G; ++e)
+                            for (int e = 0; e < G; ++e)
 #pragma unroll
-                            for (int s = 0; s < NSUB; ++s)
-                                tma_load_4d(smem_u32(sK + stage * KV_TILE + s * KV_SUB + e * GK * 128), &tmK,
-                                            smem_u32(&bars.k_full[stage]), 0, cur.key0[e], s, it.head);
+                                for (int s = 0; s < NSUB; ++s)
+                                    tma_load_4d(smem_u32(sK + stage * KV_TILE + s * KV_SUB + e * GK * 128), &tmK,
+                                                smem_u32(&bars.k_full[stage]), 0, cur.key0[e], s, it.head);
+                        }
+                        BSA_TRACE_POINT(0, tn, 21);
                     }
-                    BSA_TRACE_POINT(0, tn, 21);
                 }
-            }
             };
             run(IntC<0>());
             if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
@@ -1853,28 +1853,28 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             bool ok = true;
             const bool withhold = *reinterpret_cast<volatile int*>(&g_withhold_arrival) != 0;  // test hook, see above
             const auto run = [&](auto pass_c) {
-            WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
-            for (int kr = 0; kr < n_rounds && ok; ++kr) {
-                const WorkItem it = it_next;
-                it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
-                if (it.ntiles <= 0) continue;
-                TileKeys<G, GK> next;
-                next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
-                for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSV)) {
-                    const TileKeys<G, GK> cur = next;
-                    if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
-                    const int stage = ring.stage;
-                    const uint32_t ph = ring.phase;
-                    if (withhold && g == 0) continue;  // this tile never arrives
-                    ok = mbar_wait(smem_u32(&bars.v_empty[stage]), ph ^ 1, abortp);
-                    if (!ok) break;
-                    mbar_arrive_expect_tx(smem_u32(&bars.v_full[stage]), KV_TILE);
+                WorkItem it_next = load_item(p.items, item_at(pass_c, 0), n_items);
+                for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                    const WorkItem it = it_next;
+                    it_next = load_item(p.items, item_at(pass_c, kr + 1), n_items);
+                    if (it.ntiles <= 0) continue;
+                    TileKeys<G, GK> next;
+                    next.load(p.tile_col, it.tile_begin, it.tile_end, p.Nkv);
+                    for (int j = it.tile_begin; j < it.tile_end; j += G, ++g, ring.advance(NSV)) {
+                        const TileKeys<G, GK> cur = next;
+                        if (j + G < it.tile_end) next.load(p.tile_col, j + G, it.tile_end, p.Nkv);
+                        const int stage = ring.stage;
+                        const uint32_t ph = ring.phase;
+                        if (withhold && g == 0) continue;  // this tile never arrives
+                        ok = mbar_wait(smem_u32(&bars.v_empty[stage]), ph ^ 1, abortp);
+                        if (!ok) break;
+                        mbar_arrive_expect_tx(smem_u32(&bars.v_full[stage]), KV_TILE);
 #pragma unroll
-                    for (int e = 0; e < G; ++e)
-                        tma_load_4d(smem_u32(sV + stage * KV_TILE + e * GV_TILE), &tmV, smem_u32(&bars.v_full[stage]), 0,
-                                    cur.key0[e], 0, it.head);
+                        for (int e = 0; e < G; ++e)
+                            tma_load_4d(smem_u32(sV + stage * KV_TILE + e * GV_TILE), &tmV, smem_u32(&bars.v_full[stage]), 0,
+                                        cur.key0[e], 0, it.head);
+                    }
                 }
-            }
             };
             run(IntC<0>());
             if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
@@ -1893,52 +1893,52 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
             const auto run = [&](auto pass_c) {
-            int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
-            for (int kr = 0; kr < n_rounds && ok; ++kr) {
-                const int n = n_next;
-                n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
-                if (n <= 0) continue;
-                const uint32_t qb = kSmemQ ? (itq & 1u) : 0u;  // this item's Q buffer
-                ok = kSmemQ ? mbar_wait(smem_u32(&bars.q_full[qb]), (itq >> 1) & 1, abortp)
-                            : mbar_wait(smem_u32(&bars.qt_full), itq & 1, abortp);
-                if (!ok) break;
-                const uint64_t descQ = descQ0 + (uint64_t)((qb * NSUB * Q_SUB) >> 4);
-                for (int j = 0; j < n; ++j, ring.advance(NSK)) {
-                    const uint32_t gs = g + j;
-                    const int stage = ring.stage;
-                    const uint32_t ph = ring.phase, sb = gs & 1;
-                    // K tile present, and S[sb] read into registers by the softmax of tile gs-2
-                    if (gs >= 2)
-                        ok = mbar_wait2(smem_u32(&bars.s_free[sb]), ((gs >> 1) - 1) & 1, smem_u32(&bars.k_full[stage]), ph, abortp);
-                    else
-                        ok = mbar_wait(smem_u32(&bars.k_full[stage]), ph, abortp);
+                int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
+                for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                    const int n = n_next;
+                    n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
+                    if (n <= 0) continue;
+                    const uint32_t qb = kSmemQ ? (itq & 1u) : 0u;  // this item's Q buffer
+                    ok = kSmemQ ? mbar_wait(smem_u32(&bars.q_full[qb]), (itq >> 1) & 1, abortp)
+                                : mbar_wait(smem_u32(&bars.qt_full), itq & 1, abortp);
                     if (!ok) break;
-                    BSA_PH(0);
-                    BSA_STAMP(0, gs, 0);
-                    BSA_TRACE_POINT(1, tn, 6);
-                    tc_fence_after();
-                    const uint32_t d_s = tmem + (sb ? kColS1 : kColS0);
-#pragma unroll(kSmemQ ? 4 : 8)  // (all eight with both operands' descriptors do not fit this thread's registers)
-                    for (int k = 0; k < D / 16; ++k) {
-                        const uint64_t b = descK + (uint64_t)((stage * KV_TILE + (k / 4) * KV_SUB + (k % 4) * 32) >> 4);
-                        if constexpr (kSmemQ)
-                            mma_ss(d_s, descQ + (uint64_t)(((k / 4) * Q_SUB + (k % 4) * 32) >> 4), b, idesc_qk, k > 0);
+                    const uint64_t descQ = descQ0 + (uint64_t)((qb * NSUB * Q_SUB) >> 4);
+                    for (int j = 0; j < n; ++j, ring.advance(NSK)) {
+                        const uint32_t gs = g + j;
+                        const int stage = ring.stage;
+                        const uint32_t ph = ring.phase, sb = gs & 1;
+                        // K tile present, and S[sb] read into registers by the softmax of tile gs-2
+                        if (gs >= 2)
+                            ok = mbar_wait2(smem_u32(&bars.s_free[sb]), ((gs >> 1) - 1) & 1, smem_u32(&bars.k_full[stage]), ph, abortp);
                         else
-                            mma_ts(d_s, tmem + Cols::kQ + k * 8, b, idesc_qk, k > 0);
-                    }
-                    mma_commit(smem_u32(&bars.k_empty[stage]));
-                    mma_commit(smem_u32(&bars.s_full[sb]));
-                    BSA_PH(1);
-                    BSA_STAMP(0, gs, 1);
+                            ok = mbar_wait(smem_u32(&bars.k_full[stage]), ph, abortp);
+                        if (!ok) break;
+                        BSA_PH(0);
+                        BSA_STAMP(0, gs, 0);
+                        BSA_TRACE_POINT(1, tn, 6);
+                        tc_fence_after();
+                        const uint32_t d_s = tmem + (sb ? kColS1 : kColS0);
+#pragma unroll(kSmemQ ? 4 : 8)  // (all eight with both operands' descriptors do not fit this thread's registers)
+                        for (int k = 0; k < D / 16; ++k) {
+                            const uint64_t b = descK + (uint64_t)((stage * KV_TILE + (k / 4) * KV_SUB + (k % 4) * 32) >> 4);
+                            if constexpr (kSmemQ)
+                                mma_ss(d_s, descQ + (uint64_t)(((k / 4) * Q_SUB + (k % 4) * 32) >> 4), b, idesc_qk, k > 0);
+                            else
+                                mma_ts(d_s, tmem + Cols::kQ + k * 8, b, idesc_qk, k > 0);
+                        }
+                        mma_commit(smem_u32(&bars.k_empty[stage]));
+                        mma_commit(smem_u32(&bars.s_full[sb]));
+                        BSA_PH(1);
+                        BSA_STAMP(0, gs, 1);
 #ifdef BSA_PHASES
-                    ++ph_n;
+                        ++ph_n;
 #endif
-                    BSA_TRACE_POINT(1, tn, 2);
-                    if (!kSmemQ && j == n - 1) mma_commit(smem_u32(&bars.q_free));
+                        BSA_TRACE_POINT(1, tn, 2);
+                        if (!kSmemQ && j == n - 1) mma_commit(smem_u32(&bars.q_free));
+                    }
+                    g += n;
+                    ++itq;
                 }
-                g += n;
-                ++itq;
-            }
             };
             run(IntC<0>());
             if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
@@ -1955,47 +1955,47 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             BSA_TRACE_DECL(tn);
             BSA_PH_DECL;
             const auto run = [&](auto pass_c) {
-            int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
-            for (int kr = 0; kr < n_rounds && ok; ++kr) {
-                const int n = n_next;
-                n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
-                if (n <= 0) continue;
-                for (int j = 0; j < n; ++j, ring.advance(NSV)) {
-                    const uint32_t gp = g + j;
-                    const int stage = ring.stage;
-                    const uint32_t ph = ring.phase, sb = gp & 1;
-                    // V tile present (normally long before), accumulator drained by the epilogue (first tile of an
-                    // item), and last the P tile, which is the one this thread normally waits for
-                    if (j == 0) {
-                        ok = mbar_wait(smem_u32(&bars.o_free), (itq & 1) ^ 1, abortp);
+                int n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, 0), n_items).ntiles);
+                for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                    const int n = n_next;
+                    n_next = tiles_of<G>(load_item(p.items, item_at(pass_c, kr + 1), n_items).ntiles);
+                    if (n <= 0) continue;
+                    for (int j = 0; j < n; ++j, ring.advance(NSV)) {
+                        const uint32_t gp = g + j;
+                        const int stage = ring.stage;
+                        const uint32_t ph = ring.phase, sb = gp & 1;
+                        // V tile present (normally long before), accumulator drained by the epilogue (first tile of an
+                        // item), and last the P tile, which is the one this thread normally waits for
+                        if (j == 0) {
+                            ok = mbar_wait(smem_u32(&bars.o_free), (itq & 1) ^ 1, abortp);
+                            if (!ok) break;
+                        }
+                        ok = mbar_wait2(smem_u32(&bars.v_full[stage]), ph, smem_u32(&bars.p_ready[sb]), (gp >> 1) & 1, abortp);
                         if (!ok) break;
-                    }
-                    ok = mbar_wait2(smem_u32(&bars.v_full[stage]), ph, smem_u32(&bars.p_ready[sb]), (gp >> 1) & 1, abortp);
-                    if (!ok) break;
-                    BSA_PH(0);
-                    BSA_STAMP(1, gp, 0);
-                    BSA_TRACE_POINT(10, tn, 3);
+                        BSA_PH(0);
+                        BSA_STAMP(1, gp, 0);
+                        BSA_TRACE_POINT(10, tn, 3);
 
-                    tc_fence_after();
-                    const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0), d_o = tmem + (sb ? Cols::kO1 : Cols::kO0);
+                        tc_fence_after();
+                        const uint32_t a_p = tmem + (sb ? Cols::kP1 : Cols::kP0), d_o = tmem + (sb ? Cols::kO1 : Cols::kO0);
 #pragma unroll
-                    for (int k = 0; k < TK / 16; ++k) {
-                        const uint64_t b = descV + (uint64_t)((stage * KV_TILE + (k / (GK / 16)) * GV_TILE + (k % (GK / 16)) * 2048) >> 4);
-                        mma_ts(d_o, a_p + k * 8, b, idesc_pv, (j > (kOwnO ? 1 : 0) || k > 0) ? 1u : 0u);
-                    }
-                    mma_commit(smem_u32(&bars.v_empty[stage]));
-                    mma_commit(smem_u32(&bars.pv_done[sb]));
-                    if (j == n - 1) mma_commit(smem_u32(&bars.o_full));
-                    BSA_PH(1);
-                    BSA_STAMP(1, gp, 1);
+                        for (int k = 0; k < TK / 16; ++k) {
+                            const uint64_t b = descV + (uint64_t)((stage * KV_TILE + (k / (GK / 16)) * GV_TILE + (k % (GK / 16)) * 2048) >> 4);
+                            mma_ts(d_o, a_p + k * 8, b, idesc_pv, (j > (kOwnO ? 1 : 0) || k > 0) ? 1u : 0u);
+                        }
+                        mma_commit(smem_u32(&bars.v_empty[stage]));
+                        mma_commit(smem_u32(&bars.pv_done[sb]));
+                        if (j == n - 1) mma_commit(smem_u32(&bars.o_full));
+                        BSA_PH(1);
+                        BSA_STAMP(1, gp, 1);
 #ifdef BSA_PHASES
-                    ++ph_n;
+                        ++ph_n;
 #endif
-                    BSA_TRACE_POINT(10, tn, 5);
+                        BSA_TRACE_POINT(10, tn, 5);
+                    }
+                    g += n;
+                    ++itq;
                 }
-                g += n;
-                ++itq;
-            }
             };
             run(IntC<0>());
             if constexpr (kFirstRef) if (ok && second_pass()) run(IntC<1>());
@@ -2080,416 +2080,416 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         };
         bool again = true;
         if constexpr (kFirstRef) {
-        // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
-        // item nor the metadata that depends on it is waited for at an item boundary
-        ItemSpan it_next = load_item_span(p.items, item_at(IntC<0>(), 0), n_items);
-        ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<0>(), 1), n_items);
-        int last_col = 0;
-        uint32_t first_word = 0;
-        {
-            const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
-            first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
-            if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
-        }
-        for (int kr = 0; kr < n_rounds && ok; ++kr) {
-            const ItemSpan it = it_next;
-            it_next = it_next2;
-            it_next2 = load_item_span(p.items, item_at(IntC<0>(), kr + 2), n_items);
-            const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
-            uint32_t word_next = first_word;
-            // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
-            const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
-            {   // the next item's first tile of this warpgroup: its parity follows from g + n
-                const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
+            // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
+            // item nor the metadata that depends on it is waited for at an item boundary
+            ItemSpan it_next = load_item_span(p.items, item_at(IntC<0>(), 0), n_items);
+            ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<0>(), 1), n_items);
+            int last_col = 0;
+            uint32_t first_word = 0;
+            {
+                const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
                 first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
                 if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
             }
-            if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
-            float m_ref = -INFINITY, l = 0.f;
-            bool settled = false;  // every row of the warp has its reference
-            // first local tile index of this warpgroup inside the item
-            const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
-            for (int j = j0; j < n; j += 2) {
-                const uint32_t gs = g + j;
-                uint32_t ballot = full_ballot;
-                if (G > 1 || has_bits) {
-                    ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
-                    if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
+            for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                const ItemSpan it = it_next;
+                it_next = it_next2;
+                it_next2 = load_item_span(p.items, item_at(IntC<0>(), kr + 2), n_items);
+                const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
+                uint32_t word_next = first_word;
+                // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
+                const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
+                {   // the next item's first tile of this warpgroup: its parity follows from g + n
+                    const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
+                    first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+                    if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
                 }
-                const bool need_mask = ballot != full_ballot;
-                const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
-                const bool ragged = (j == n - 1) && n_valid < TK;
-                if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
-                BSA_PH(7);
-                ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
-                if (!ok) break;
-                BSA_PH(0);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 10);
-                tc_fence_after();
-                uint32_t r[TK];
-#pragma unroll
-                for (int c = 0; c < TK / 32; ++c) tmem_ld32(t_s + c * 32, &r[c * 32]);
-                tc_wait_ld();
-                BSA_PH(1);
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars.s_free[x]));  // S[x] is in registers: the next Q K^T into it may start
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
-                if (need_mask) {
-                    // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
-                    // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
-#pragma unroll
-                    for (int gq = 0; gq < TK / 16; ++gq) {
-                        const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
-#pragma unroll
-                        for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
+                if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
+                float m_ref = -INFINITY, l = 0.f;
+                bool settled = false;  // every row of the warp has its reference
+                // first local tile index of this warpgroup inside the item
+                const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
+                for (int j = j0; j < n; j += 2) {
+                    const uint32_t gs = g + j;
+                    uint32_t ballot = full_ballot;
+                    if (G > 1 || has_bits) {
+                        ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
+                        if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
                     }
-                }
-                if (ragged) {
-#pragma unroll
-                    for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
-                }
-                if (!settled) {  // the item's first tile, and where some row has not been reached yet
-                    float m_prev = -INFINITY;
-                    if (kOwnO) m_prev = m_ref;
-                    else if (j > 0) {  // (published, since this warp is not settled; its slot is not written again before this tile's P V)
-                        ok = __all_sync(0xffffffffu, take_word(&mref[itn & 1][tw], (j == 1) ? (itn >> 1) & 1u : 2u + (j & 1u), m_prev));
-                        if (!ok) break;
-                    }
-                    if (!__all_sync(0xffffffffu, m_prev != -INFINITY)) {
-                        float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
-#pragma unroll
-                        for (int i = 0; i < TK; i += 8) {
-                            m0 = max3(m0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
-                            m1 = max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
-                            m2 = max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
-                            m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
-                        }
-                        const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
-                        if (m_prev == -INFINITY) m_prev = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
-                        if (!kOwnO) *reinterpret_cast<volatile uint32_t*>(&mref[itn & 1][tw]) =
-                            __float_as_uint(m_prev) | ((j == 0) ? (itn >> 1) & 1u : 3u - (j & 1u));
-                    }
-                    m_ref = m_prev;
-                    settled = __all_sync(0xffffffffu, m_ref != -INFINITY);
-                }
-                const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
-                const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
-                uint64_t sum01 = pack_f32x2(0.f, 0.f), sum23 = sum01;
-                // P[x] was last read by the P V of tile gs-2 (normally long complete).  With d = 64 it is waited for
-                // here and the P tile stored 32 columns at a time while the next columns are still being exponentiated
-                // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
-                constexpr bool kStoreInLoop = (D == 64);
-                if (kStoreInLoop && gs >= 2) {
-                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
+                    const bool need_mask = ballot != full_ballot;
+                    const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
+                    const bool ragged = (j == n - 1) && n_valid < TK;
+                    if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
+                    BSA_PH(7);
+                    ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
                     if (!ok) break;
+                    BSA_PH(0);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 10);
                     tc_fence_after();
-                }
+                    uint32_t r[TK];
 #pragma unroll
-                for (int i = 0; i < TK; i += 4) {
-                    float x0, x1, x2, x3;
-                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), c22, nm2), x0, x1);
-                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), c22, nm2), x2, x3);
-                    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
-                    sum01 = add_f32x2(sum01, pack_f32x2(p0, p1));
-                    sum23 = add_f32x2(sum23, pack_f32x2(p2, p3));
-                    r[i / 2] = pack_16x2<F16>(p0, p1);
-                    r[i / 2 + 1] = pack_16x2<F16>(p2, p3);
-                    if (kStoreInLoop && (i & 31) == 28) tmem_st16(t_p + (i >> 5) * 16, &r[(i >> 5) * 16]);
-                }
-                float s0, s1, s2, s3;
-                unpack_f32x2(sum01, s0, s1);
-                unpack_f32x2(sum23, s2, s3);
-                l += (s0 + s1) + (s2 + s3);
-#ifdef BSA_PHASES
-                {
-                    float f0_ = l;
-                    uint32_t u0_ = r[TK / 2 - 1];
-                    asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+r"(u0_));
-                }
-#endif
-                BSA_PH(4);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
-                if (!kStoreInLoop) {
-                    if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
-                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                    for (int c = 0; c < TK / 32; ++c) tmem_ld32(t_s + c * 32, &r[c * 32]);
+                    tc_wait_ld();
+                    BSA_PH(1);
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&bars.s_free[x]));  // S[x] is in registers: the next Q K^T into it may start
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
+                    if (need_mask) {
+                        // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
+                        // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
+#pragma unroll
+                        for (int gq = 0; gq < TK / 16; ++gq) {
+                            const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
+#pragma unroll
+                            for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
+                        }
+                    }
+                    if (ragged) {
+#pragma unroll
+                        for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
+                    }
+                    if (!settled) {  // the item's first tile, and where some row has not been reached yet
+                        float m_prev = -INFINITY;
+                        if (kOwnO) m_prev = m_ref;
+                        else if (j > 0) {  // (published, since this warp is not settled; its slot is not written again before this tile's P V)
+                            ok = __all_sync(0xffffffffu, take_word(&mref[itn & 1][tw], (j == 1) ? (itn >> 1) & 1u : 2u + (j & 1u), m_prev));
+                            if (!ok) break;
+                        }
+                        if (!__all_sync(0xffffffffu, m_prev != -INFINITY)) {
+                            float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+                            for (int i = 0; i < TK; i += 8) {
+                                m0 = max3(m0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+                                m1 = max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+                                m2 = max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
+                                m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
+                            }
+                            const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
+                            if (m_prev == -INFINITY) m_prev = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
+                            if (!kOwnO) *reinterpret_cast<volatile uint32_t*>(&mref[itn & 1][tw]) =
+                                __float_as_uint(m_prev) | ((j == 0) ? (itn >> 1) & 1u : 3u - (j & 1u));
+                        }
+                        m_ref = m_prev;
+                        settled = __all_sync(0xffffffffu, m_ref != -INFINITY);
+                    }
+                    const float neg_m = (m_ref == -INFINITY) ? 0.f : -m_ref;
+                    const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
+                    uint64_t sum01 = pack_f32x2(0.f, 0.f), sum23 = sum01;
+                    // P[x] was last read by the P V of tile gs-2 (normally long complete).  With d = 64 it is waited for
+                    // here and the P tile stored 32 columns at a time while the next columns are still being exponentiated
+                    // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
+                    constexpr bool kStoreInLoop = (D == 64);
+                    if (kStoreInLoop && gs >= 2) {
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
                         if (!ok) break;
                         tc_fence_after();
                     }
-                    BSA_PH(5);
-                    if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
 #pragma unroll
-                    for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
-                }
-                tc_wait_st();
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars.p_ready[x]));
-                BSA_PH(6);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 3);
+                    for (int i = 0; i < TK; i += 4) {
+                        float x0, x1, x2, x3;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), c22, nm2), x0, x1);
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), c22, nm2), x2, x3);
+                        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
+                        sum01 = add_f32x2(sum01, pack_f32x2(p0, p1));
+                        sum23 = add_f32x2(sum23, pack_f32x2(p2, p3));
+                        r[i / 2] = pack_16x2<F16>(p0, p1);
+                        r[i / 2 + 1] = pack_16x2<F16>(p2, p3);
+                        if (kStoreInLoop && (i & 31) == 28) tmem_st16(t_p + (i >> 5) * 16, &r[(i >> 5) * 16]);
+                    }
+                    float s0, s1, s2, s3;
+                    unpack_f32x2(sum01, s0, s1);
+                    unpack_f32x2(sum23, s2, s3);
+                    l += (s0 + s1) + (s2 + s3);
 #ifdef BSA_PHASES
-                ++ph_n;
+                    {
+                        float f0_ = l;
+                        uint32_t u0_ = r[TK / 2 - 1];
+                        asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+r"(u0_));
+                    }
 #endif
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 16);
-            }
-            if (!ok) break;
-            // ---- hand this warpgroup's row sums to the epilogue warpgroup ----
-            {
-                // the previous item's sums must have been read
-                ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
+                    BSA_PH(4);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
+                    if (!kStoreInLoop) {
+                        if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
+                            ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        BSA_PH(5);
+                        if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
+#pragma unroll
+                        for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
+                    }
+                    tc_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&bars.p_ready[x]));
+                    BSA_PH(6);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 3);
+#ifdef BSA_PHASES
+                    ++ph_n;
+#endif
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 16);
+                }
                 if (!ok) break;
-                lfin[x][tw] = l;
-                if (kOwnO) mref[x][tw] = __float_as_uint(m_ref);
-                else if (((g + n - 1) & 1) == (uint32_t)x) mfin[tw] = m_ref;  // whoever took the last tile knows the reference of every row
-                mbar_arrive(smem_u32(&bars.e_ready));
-                ++itn;
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
+                // ---- hand this warpgroup's row sums to the epilogue warpgroup ----
+                {
+                    // the previous item's sums must have been read
+                    ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
+                    if (!ok) break;
+                    lfin[x][tw] = l;
+                    if (kOwnO) mref[x][tw] = __float_as_uint(m_ref);
+                    else if (((g + n - 1) & 1) == (uint32_t)x) mfin[tw] = m_ref;  // whoever took the last tile knows the reference of every row
+                    mbar_arrive(smem_u32(&bars.e_ready));
+                    ++itn;
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
+                }
+                g += n;
+                BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
             }
-            g += n;
-            BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
-        }
-        // ---- pass 1: the items whose first reference did not serve, with a reference that follows the running maximum ----
-        if (ok) {
-            mbar_arrive(smem_u32(&bars.pass_done));
-            again = __all_sync(0xffffffffu, second_pass());
-            if (!kOwnO && again) {  // everything has been read: the tags start over
-                mref[x][tw] = 0u;
-                mbar_arrive(smem_u32(&bars.tags_reset));
-                again = ok = mbar_wait_warp(smem_u32(&bars.tags_reset), 0, abortp);
+            // ---- pass 1: the items whose first reference did not serve, with a reference that follows the running maximum ----
+            if (ok) {
+                mbar_arrive(smem_u32(&bars.pass_done));
+                again = __all_sync(0xffffffffu, second_pass());
+                if (!kOwnO && again) {  // everything has been read: the tags start over
+                    mref[x][tw] = 0u;
+                    mbar_arrive(smem_u32(&bars.tags_reset));
+                    again = ok = mbar_wait_warp(smem_u32(&bars.tags_reset), 0, abortp);
+                }
             }
-        }
         }
         g0 = g;
         if (ok && again) {
-        // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
-        // item nor the metadata that depends on it is waited for at an item boundary
-        ItemSpan it_next = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 0), n_items);
-        ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 1), n_items);
-        int last_col = 0;
-        uint32_t first_word = 0;
-        {
-            const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
-            first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
-            if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
-        }
-        for (int kr = 0; kr < n_rounds && ok; ++kr) {
-            const ItemSpan it = it_next;
-            it_next = it_next2;
-            it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), kr + 2), n_items);
-            const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
-            uint32_t word_next = first_word;
-            // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
-            const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
-            {   // the next item's first tile of this warpgroup: its parity follows from g + n
-                const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
+            // work items are fetched two items ahead and the first tile's metadata one item ahead, so that neither the
+            // item nor the metadata that depends on it is waited for at an item boundary
+            ItemSpan it_next = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 0), n_items);
+            ItemSpan it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), 1), n_items);
+            int last_col = 0;
+            uint32_t first_word = 0;
+            {
+                const int j0n = ((g & 1) == (uint32_t)x) ? 0 : 1;
                 first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
                 if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
             }
-            if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
-            float m_know = -INFINITY;  // reference maximum this thread's partial sum l is expressed in
-            float l = 0.f;
-            // first local tile index of this warpgroup inside the item
-            const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
-            for (int j = j0; j < n; j += 2) {
-                const uint32_t gs = g + j;
-                uint32_t ballot = full_ballot;
-                if (G > 1 || has_bits) {
-                    ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
-                    if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
+            for (int kr = 0; kr < n_rounds && ok; ++kr) {
+                const ItemSpan it = it_next;
+                it_next = it_next2;
+                it_next2 = load_item_span(p.items, item_at(IntC<kFirstRef ? 1 : 0>(), kr + 2), n_items);
+                const int n = tiles_of<G>(it.ntiles), end = it.tile_begin + it.ntiles;
+                uint32_t word_next = first_word;
+                // keys of the last tile that exist (columns are ascending, so only its last entry can be ragged)
+                const int n_valid = ((it.ntiles - 1) & (G - 1)) * GK + (p.Nkv - last_col * GK);
+                {   // the next item's first tile of this warpgroup: its parity follows from g + n
+                    const int j0n = (((g + n) & 1) == (uint32_t)x) ? 0 : 1;
+                    first_word = load_bit(it_next.tile_begin + j0n * G, it_next.tile_begin + it_next.ntiles);
+                    if (it_next.ntiles > 0) last_col = ldg_pinned_s32(p.tile_col + it_next.tile_begin + it_next.ntiles - 1);
                 }
-                const bool need_mask = ballot != full_ballot;
-                const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
-                const bool ragged = (j == n - 1) && n_valid < TK;
-                if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
-                BSA_PH(7);
-                ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
-                if (!ok) break;
-                BSA_PH(0);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 10);
-                tc_fence_after();
-                uint32_t r[TK];
-#pragma unroll
-                for (int c = 0; c < TK / 32; ++c) tmem_ld32(t_s + c * 32, &r[c * 32]);
-                tc_wait_ld();
-                BSA_PH(1);
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars.s_free[x]));  // S[x] is in registers: the next Q K^T into it may start
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
-                // The previous tile's reference has normally been published by now: its slot is read here and the
-                // word checked after the max phase, so that the shared-memory round trip overlaps that phase.
-                uint32_t ref_word = 0;
-                if constexpr (!kOwnO) ref_word = *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]);
-                if (need_mask) {
-                    // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
-                    // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
-#pragma unroll
-                    for (int gq = 0; gq < TK / 16; ++gq) {
-                        const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
-#pragma unroll
-                        for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
+                if (n <= 0) continue;  // the epilogue warpgroup writes the empty rows
+                float m_know = -INFINITY;  // reference maximum this thread's partial sum l is expressed in
+                float l = 0.f;
+                // first local tile index of this warpgroup inside the item
+                const int j0 = ((g & 1) == (uint32_t)x) ? 0 : 1;
+                for (int j = j0; j < n; j += 2) {
+                    const uint32_t gs = g + j;
+                    uint32_t ballot = full_ballot;
+                    if (G > 1 || has_bits) {
+                        ballot = __ballot_sync(0xffffffffu, (word_next >> (mbit & 31)) & 1u);
+                        if (j + 2 < n) word_next = load_bit(it.tile_begin + (j + 2) * G, end);
                     }
-                }
-                if (ragged) {
+                    const bool need_mask = ballot != full_ballot;
+                    const uint32_t row_bits = (ballot >> (lane & 16)) & full_bits;
+                    const bool ragged = (j == n - 1) && n_valid < TK;
+                    if (lane == 0 && j == j0) BSA_TRACE_POINT(2 + warp, tn, 35);
+                    BSA_PH(7);
+                    ok = mbar_wait_warp(smem_u32(&bars.s_full[x]), (gs >> 1) & 1, abortp);
+                    if (!ok) break;
+                    BSA_PH(0);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 0);
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 10);
+                    tc_fence_after();
+                    uint32_t r[TK];
 #pragma unroll
-                    for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
-                }
-                float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+                    for (int c = 0; c < TK / 32; ++c) tmem_ld32(t_s + c * 32, &r[c * 32]);
+                    tc_wait_ld();
+                    BSA_PH(1);
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&bars.s_free[x]));  // S[x] is in registers: the next Q K^T into it may start
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 11);
+                    // The previous tile's reference has normally been published by now: its slot is read here and the
+                    // word checked after the max phase, so that the shared-memory round trip overlaps that phase.
+                    uint32_t ref_word = 0;
+                    if constexpr (!kOwnO) ref_word = *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]);
+                    if (need_mask) {
+                        // a sub-block has at least 16 key columns: one activity bit per 16, one instruction per element
+                        // (skipping the exponentials of 32 columns that no row of the warp needs brought nothing)
 #pragma unroll
-                for (int i = 0; i < TK; i += 8) {
-                    m0 = max3(m0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
-                    m1 = max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
-                    m2 = max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
-                    m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
-                }
-                const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
-#ifdef BSA_TRACE
-                if (lane == 0 && mx2 != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 17);
-#endif
-                if constexpr (!kOwnO) {
-                    // ---- reference maximum handed over from the previous tile (other warpgroup) ----
-                    float m_prev = -INFINITY;
-                    if (gs > g0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
-                        float m_taken;
-                        if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) - (g0 >> 1) + 1) & 3u))) {
-                            m_taken = __uint_as_float(ref_word & ~3u);
-                        } else {
-                            ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
-                            if (!ok) break;
+                        for (int gq = 0; gq < TK / 16; ++gq) {
+                            const bool grp = (row_bits >> ((gq * 16) >> p.lgBKV)) & 1u;
+#pragma unroll
+                            for (int i = gq * 16; i < gq * 16 + 16; ++i) r[i] = grp ? r[i] : 0xff800000u;
                         }
-                        if (j > 0) m_prev = m_taken;  // the previous tile belongs to this item
                     }
+                    if (ragged) {
+#pragma unroll
+                        for (int i = 0; i < TK; ++i) r[i] = (i < n_valid) ? r[i] : 0xff800000u;
+                    }
+                    float m0 = -INFINITY, m1 = -INFINITY, m2 = -INFINITY, m3 = -INFINITY;
+#pragma unroll
+                    for (int i = 0; i < TK; i += 8) {
+                        m0 = max3(m0, __uint_as_float(r[i]), __uint_as_float(r[i + 1]));
+                        m1 = max3(m1, __uint_as_float(r[i + 2]), __uint_as_float(r[i + 3]));
+                        m2 = max3(m2, __uint_as_float(r[i + 4]), __uint_as_float(r[i + 5]));
+                        m3 = max3(m3, __uint_as_float(r[i + 6]), __uint_as_float(r[i + 7]));
+                    }
+                    const float mx2 = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3)) * c2;
+#ifdef BSA_TRACE
+                    if (lane == 0 && mx2 != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 17);
+#endif
+                    if constexpr (!kOwnO) {
+                        // ---- reference maximum handed over from the previous tile (other warpgroup) ----
+                        float m_prev = -INFINITY;
+                        if (gs > g0) {  // every publish is consumed, in order, also across item boundaries (the tags rely on it)
+                            float m_taken;
+                            if (__all_sync(0xffffffffu, (ref_word & 3u) == ((((gs - 1) >> 1) - (g0 >> 1) + 1) & 3u))) {
+                                m_taken = __uint_as_float(ref_word & ~3u);
+                            } else {
+                                ok = __all_sync(0xffffffffu, take_reference(gs - 1, ref_word, m_taken));
+                                if (!ok) break;
+                            }
+                            if (j > 0) m_prev = m_taken;  // the previous tile belongs to this item
+                        }
+#ifdef BSA_PHASES
+                        {
+                            float f0_ = mx2, f1_ = m_prev;  // real instructions that read the values: the clock is read after them
+                            asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+f"(f1_));
+                        }
+#endif
+                        BSA_PH(2);
+#ifdef BSA_TRACE
+                        if (lane == 0 && m_prev != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 18);
+#endif
+                        if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 12);
+                        if (m_prev != m_know) {  // the other warpgroup moved the reference since this thread last looked
+                            l *= ex2_approx(m_know - m_prev);  // m_know = -inf only while l = 0
+                            m_know = m_prev;
+                        }
+                    }
+                    float alpha = 1.f;
+                    bool rescale = false;
+                    if (mx2 > m_know + kRescaleThreshold) {
+                        const float m_new = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
+                        alpha = ex2_approx(m_know - m_new);
+                        rescale = (j > (kOwnO ? 1 : 0)) && (m_know != -INFINITY);
+                        l *= alpha;
+                        m_know = m_new;
+                    }
+                    if constexpr (!kOwnO) {
+                        // publish: the next tile's warpgroup may take its decision
+                        *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) - (g0 >> 1) + 1) & 3u);
+                    }
+                    BSA_PH(3);
+                    const float neg_m = (m_know == -INFINITY) ? 0.f : -m_know;
+                    const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
+                    uint64_t sum01 = pack_f32x2(0.f, 0.f), sum23 = sum01;
+                    // P[x] was last read by the P V of tile gs-2 (normally long complete).  With d = 64 it is waited for
+                    // here and the P tile stored 32 columns at a time while the next columns are still being exponentiated
+                    // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
+                    constexpr bool kStoreInLoop = (D == 64);
+                    if (kStoreInLoop && gs >= 2) {
+                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
+                        if (!ok) break;
+                        tc_fence_after();
+                    }
+#pragma unroll
+                    for (int i = 0; i < TK; i += 4) {
+                        float x0, x1, x2, x3;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), c22, nm2), x0, x1);
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), c22, nm2), x2, x3);
+                        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
+                        sum01 = add_f32x2(sum01, pack_f32x2(p0, p1));
+                        sum23 = add_f32x2(sum23, pack_f32x2(p2, p3));
+                        r[i / 2] = pack_16x2<F16>(p0, p1);
+                        r[i / 2 + 1] = pack_16x2<F16>(p2, p3);
+                        if (kStoreInLoop && (i & 31) == 28) tmem_st16(t_p + (i >> 5) * 16, &r[(i >> 5) * 16]);
+                    }
+                    float s0, s1, s2, s3;
+                    unpack_f32x2(sum01, s0, s1);
+                    unpack_f32x2(sum23, s2, s3);
+                    l += (s0 + s1) + (s2 + s3);
 #ifdef BSA_PHASES
                     {
-                        float f0_ = mx2, f1_ = m_prev;  // real instructions that read the values: the clock is read after them
-                        asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+f"(f1_));
+                        float f0_ = l;
+                        uint32_t u0_ = r[TK / 2 - 1];
+                        asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+r"(u0_));
                     }
 #endif
-                    BSA_PH(2);
-#ifdef BSA_TRACE
-                    if (lane == 0 && m_prev != 12345.f) BSA_TRACE_POINT(2 + warp, tn, 18);
-#endif
-                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 12);
-                    if (m_prev != m_know) {  // the other warpgroup moved the reference since this thread last looked
-                        l *= ex2_approx(m_know - m_prev);  // m_know = -inf only while l = 0
-                        m_know = m_prev;
-                    }
-                }
-                float alpha = 1.f;
-                bool rescale = false;
-                if (mx2 > m_know + kRescaleThreshold) {
-                    const float m_new = kOwnO ? mx2 : __uint_as_float(__float_as_uint(mx2) & ~3u);  // two low bits clear (see mref)
-                    alpha = ex2_approx(m_know - m_new);
-                    rescale = (j > (kOwnO ? 1 : 0)) && (m_know != -INFINITY);
-                    l *= alpha;
-                    m_know = m_new;
-                }
-                if constexpr (!kOwnO) {
-                    // publish: the next tile's warpgroup may take its decision
-                    *reinterpret_cast<volatile uint32_t*>(&mref[x][tw]) = __float_as_uint(m_know) | (((gs >> 1) - (g0 >> 1) + 1) & 3u);
-                }
-                BSA_PH(3);
-                const float neg_m = (m_know == -INFINITY) ? 0.f : -m_know;
-                const uint64_t c22 = pack_f32x2(c2, c2), nm2 = pack_f32x2(neg_m, neg_m);
-                uint64_t sum01 = pack_f32x2(0.f, 0.f), sum23 = sum01;
-                // P[x] was last read by the P V of tile gs-2 (normally long complete).  With d = 64 it is waited for
-                // here and the P tile stored 32 columns at a time while the next columns are still being exponentiated
-                // (+4 % on Stress-B); with d = 128 the stores follow the loop (the split loop was 1-2 % slower there).
-                constexpr bool kStoreInLoop = (D == 64);
-                if (kStoreInLoop && gs >= 2) {
-                    ok = mbar_wait_warp(smem_u32(&bars.pv_done[x]), ((gs >> 1) - 1) & 1, abortp);
-                    if (!ok) break;
-                    tc_fence_after();
-                }
+                    BSA_PH(4);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
+                    if (!kStoreInLoop) {
+                        if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
+                            ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
+                        BSA_PH(5);
+                        if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
 #pragma unroll
-                for (int i = 0; i < TK; i += 4) {
-                    float x0, x1, x2, x3;
-                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i]), __uint_as_float(r[i + 1])), c22, nm2), x0, x1);
-                    unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(r[i + 2]), __uint_as_float(r[i + 3])), c22, nm2), x2, x3);
-                    const float p0 = ex2_approx(x0), p1 = ex2_approx(x1), p2 = ex2_approx(x2), p3 = ex2_approx(x3);
-                    sum01 = add_f32x2(sum01, pack_f32x2(p0, p1));
-                    sum23 = add_f32x2(sum23, pack_f32x2(p2, p3));
-                    r[i / 2] = pack_16x2<F16>(p0, p1);
-                    r[i / 2 + 1] = pack_16x2<F16>(p2, p3);
-                    if (kStoreInLoop && (i & 31) == 28) tmem_st16(t_p + (i >> 5) * 16, &r[(i >> 5) * 16]);
-                }
-                float s0, s1, s2, s3;
-                unpack_f32x2(sum01, s0, s1);
-                unpack_f32x2(sum23, s2, s3);
-                l += (s0 + s1) + (s2 + s3);
-#ifdef BSA_PHASES
-                {
-                    float f0_ = l;
-                    uint32_t u0_ = r[TK / 2 - 1];
-                    asm volatile("mov.b32 %0, %0;\n\tmov.b32 %1, %1;" : "+f"(f0_), "+r"(u0_));
-                }
-#endif
-                BSA_PH(4);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 1);
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 14);
-                if (!kStoreInLoop) {
-                    if (gs >= 1) {  // the P tile before this one (other warpgroup's) must have been consumed
-                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
-                        if (!ok) break;
-                        tc_fence_after();
+                        for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
                     }
-                    BSA_PH(5);
-                    if (lane == 0) BSA_STAMP(2 + warp, gs, 2);
-#pragma unroll
-                    for (int c = 0; c < TK / 32; ++c) tmem_st16(t_p + c * 16, &r[c * 16]);
-                }
-                // ---- the reference moved at this tile: rescale the running output (its last P V has been waited for above) ----
-                if (j > 0 && __any_sync(0xffffffffu, rescale)) {
-                    if constexpr (!kOwnO && (!kSmemQ || kFirstRef)) {  // (returns at once; without it ptxas spills in the gathered kernels)
-                        ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
-                        if (!ok) break;
-                        tc_fence_after();
-                    }
+                    // ---- the reference moved at this tile: rescale the running output (its last P V has been waited for above) ----
+                    if (j > 0 && __any_sync(0xffffffffu, rescale)) {
+                        if constexpr (!kOwnO && (!kSmemQ || kFirstRef)) {  // (returns at once; without it ptxas spills in the gathered kernels)
+                            ok = mbar_wait_warp(smem_u32(&bars.pv_done[x ^ 1]), ((gs - 1) >> 1) & 1, abortp);
+                            if (!ok) break;
+                            tc_fence_after();
+                        }
 #pragma unroll 1  // rare path: kept small
-                    for (int c = 0; c < D / 32; ++c) {
-                        uint32_t o[32];
-                        tmem_ld32(t_o + c * 32, o);
-                        tc_wait_ld();
+                        for (int c = 0; c < D / 32; ++c) {
+                            uint32_t o[32];
+                            tmem_ld32(t_o + c * 32, o);
+                            tc_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
-                        tmem_st32(t_o + c * 32, o);
+                            for (int i = 0; i < 32; ++i) o[i] = __float_as_uint(__uint_as_float(o[i]) * alpha);
+                            tmem_st32(t_o + c * 32, o);
+                        }
                     }
-                }
-                tc_wait_st();
-                tc_fence_before();
-                mbar_arrive(smem_u32(&bars.p_ready[x]));
-                BSA_PH(6);
-                if (lane == 0) BSA_STAMP(2 + warp, gs, 3);
+                    tc_wait_st();
+                    tc_fence_before();
+                    mbar_arrive(smem_u32(&bars.p_ready[x]));
+                    BSA_PH(6);
+                    if (lane == 0) BSA_STAMP(2 + warp, gs, 3);
 #ifdef BSA_PHASES
-                ++ph_n;
+                    ++ph_n;
 #endif
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 16);
-            }
-            if (!ok) break;
-            // ---- hand this warpgroup's row sums, expressed in the item's final reference, to the epilogue warpgroup ----
-            {
-                const uint32_t gl = g + n - 1;  // last tile of the item
-                const bool owner = (gl & 1) == (uint32_t)x;
-                float m_final = m_know;
-                if (!kOwnO && !owner) {  // the other warpgroup took the last tile: its publish holds the final reference
-                    ok = __all_sync(0xffffffffu,
-                                    take_reference(gl, *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]), m_final));
-                    if (!ok) break;
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 16);
                 }
-                if (m_final != m_know) l *= ex2_approx(m_know - m_final);  // l = 0 whenever m_know = -inf
-                // the previous item's sums must have been read
-                ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
                 if (!ok) break;
-                lfin[x][tw] = l;
-                if (kOwnO) mref[x][tw] = __float_as_uint(m_know);
-                else if (owner) mfin[tw] = m_final;
-                mbar_arrive(smem_u32(&bars.e_ready));
-                ++itn;
-                if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
+                // ---- hand this warpgroup's row sums, expressed in the item's final reference, to the epilogue warpgroup ----
+                {
+                    const uint32_t gl = g + n - 1;  // last tile of the item
+                    const bool owner = (gl & 1) == (uint32_t)x;
+                    float m_final = m_know;
+                    if (!kOwnO && !owner) {  // the other warpgroup took the last tile: its publish holds the final reference
+                        ok = __all_sync(0xffffffffu,
+                                        take_reference(gl, *reinterpret_cast<volatile uint32_t*>(&mref[x ^ 1][tw]), m_final));
+                        if (!ok) break;
+                    }
+                    if (m_final != m_know) l *= ex2_approx(m_know - m_final);  // l = 0 whenever m_know = -inf
+                    // the previous item's sums must have been read
+                    ok = mbar_wait_warp(smem_u32(&bars.e_taken), (itn & 1) ^ 1, abortp);
+                    if (!ok) break;
+                    lfin[x][tw] = l;
+                    if (kOwnO) mref[x][tw] = __float_as_uint(m_know);
+                    else if (owner) mfin[tw] = m_final;
+                    mbar_arrive(smem_u32(&bars.e_ready));
+                    ++itn;
+                    if (lane == 0) BSA_TRACE_POINT(2 + warp, tn, 30);
+                }
+                g += n;
+                BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
             }
-            g += n;
-            BSA_PH(7);  // item boundary: sums handed over, next item's first tile not yet waited for
-        }
         }
 #ifdef BSA_PHASES
         if (blockIdx.x == 1 && lane == 0) {
