@@ -1454,10 +1454,11 @@ struct PpCols {
     static constexpr uint32_t kQ = 448;
 };
 
-// Tiles of a list of n entries, G entries to a tile (n <= 0: no tiles, or past the end of the list).
+// Tiles of a list of n entries, G entries to a tile.  An item past the end of the list or left out of a pass (n = -1) has
+// none: the softmax warpgroups add this number up over all items, left out or not, to know which of them takes a tile.
 template <int G>
 __device__ __forceinline__ int tiles_of(int n) {
-    return n > 0 ? (n + G - 1) / G : n;
+    return n > 0 ? (n + G - 1) / G : 0;
 }
 // First keys of the entries of one tile; entries beyond the list start at N_kv, where the copy reads zeros.
 template <int G, int GK>
