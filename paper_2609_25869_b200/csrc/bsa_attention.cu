@@ -1347,7 +1347,7 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // whole item.  bf16 and fp32 keep their relative precision over 2^100, so it does not matter how far later scores lie above
 // it; from its second tile on a softmax warpgroup neither looks for maxima (64 instructions and about 300 clk per tile) nor
 // takes and publishes a word per row and tile, and nothing is rescaled.  Where it fails (a row sum beyond 2^100 or undefined,
-// or an accumulator that overflows) the epilogue marks the item, and a second pass over the marked items follows the running
+// or an output that is not finite) the epilogue marks the item, and a second pass over the marked items follows the running
 // maximum as before, moved by more than 2^8 at a time.  Per 128-key tile the softmax chain falls by a fifth.  Builds in turn,
 // back to back, before / after: 16384 tokens, 8 heads, (128,128) 153.5 / 144.4 us; 115200, 4 heads 1840 / 1725; 75600, 6
 // heads, (64,64) 3650 / 3510, 4 heads, (32,32) 4560 / 3700.  At d = 64 (each warpgroup has its own) on lists of 32
@@ -1684,24 +1684,6 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     if (kFirstRef && pass == 0) doubtful = row_ok && sum_is_doubtful(l_tot);
                 }
                 mbar_arrive(smem_u32(&bars.e_taken));
-                // An accumulator can overflow only where the weights are far above those of a reference that follows the maximum:
-                // then its values decide as well.  Otherwise the verdict is in before the item's stores, which an arrival behind
-                // them would wait for.
-                const bool big = kFirstRef && pass == 0 && __any_sync(0xffffffffu, l_tot > 33554432.f);
-                const auto mark = [&]() {
-                    if (__any_sync(0xffffffffu, doubtful) && lane == 0) {
-                        const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
-                        atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
-                        redo_any = 1u;
-                    }
-                };
-                if (kFirstRef && pass == 0 && !big) {
-                    mark();
-                    if (kr == n_rounds - 1) {
-                        mbar_arrive(smem_u32(&bars.pass_done));
-                        arrived = true;
-                    }
-                }
                 const float inv_l = (l_tot > 0.f) ? 1.f / l_tot : 0.f;
                 const float lse = (l_tot > 0.f) ? fmaf(m_final, 0.6931471805599453f, logf(l_tot)) : -INFINITY;
                 if (lane == 0) BSA_TRACE_POINT(11, tn, 32);
@@ -1716,7 +1698,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const int n_tiles = tiles_of<G>(it.ntiles);  // 1: the other accumulator is stale
                 g_start += (uint32_t)n_tiles;
                 const float sa = inv_l * wa, sb = inv_l * wb;
-                float nonfinite = 0.f;
+                // An accumulator can overflow where the running maximum's weights of at most 2^8 would not: however small the row's
+                // sum is, its outputs decide as well (d = 64: those of either accumulator, weighted by zero or not).
+                uint64_t nf0 = pack_f32x2(0.f, 0.f), nf1 = nf0;  // zero as long as every output is finite
 #pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
                 for (int c = 0; c < D / CW; ++c) {
                     uint32_t o[CW];
@@ -1736,14 +1720,31 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 #pragma unroll
                         for (int e = 0; e < CW; ++e) o[e] = __float_as_uint(__uint_as_float(o[e]) * sa);
                     }
-                    if (kFirstRef && pass == 0 && big) {  // zero as long as every output is finite
-#pragma unroll
-                        for (int e = 0; e < CW; ++e) nonfinite = fmaf(__uint_as_float(o[e]), 0.f, nonfinite);
-                    }
                     if (c == D / CW - 1) {  // the accumulator is in registers: the next item's first P V may overwrite it
                         tc_fence_before();
                         mbar_arrive(smem_u32(&bars.o_free));
                         if (lane == 0) BSA_TRACE_POINT(11, tn, 33);
+                    }
+                    if (kFirstRef && pass == 0) {
+                        const uint64_t zero2 = pack_f32x2(0.f, 0.f);
+#pragma unroll
+                        for (int e = 0; e < CW; e += 4) {
+                            nf0 = fma_f32x2(pack_f32x2(__uint_as_float(o[e]), __uint_as_float(o[e + 1])), zero2, nf0);
+                            nf1 = fma_f32x2(pack_f32x2(__uint_as_float(o[e + 2]), __uint_as_float(o[e + 3])), zero2, nf1);
+                        }
+                        if (c == D / CW - 1) {
+                            float f0, f1;
+                            unpack_f32x2(add_f32x2(nf0, nf1), f0, f1);
+                            if (__any_sync(0xffffffffu, doubtful || (row_ok && !(f0 + f1 == 0.f))) && lane == 0) {
+                                const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
+                                atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
+                                redo_any = 1u;
+                            }
+                            if (kr == n_rounds - 1) {  // the verdict on the CTA's last item is in
+                                mbar_arrive(smem_u32(&bars.pass_done));
+                                arrived = true;
+                            }
+                        }
                     }
                     if (it.nparts == 1) {
                         if (row_ok) {  // 32-byte stores: every thread fills whole 32-byte sectors of its own row
@@ -1775,10 +1776,6 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     p.ws_LSE[(size_t)it.ws_slot * kTQ + tw] = lse;
                 }
                 if (lane == 0) BSA_TRACE_POINT(11, tn, 34);
-                if (kFirstRef && pass == 0 && big) {
-                    doubtful = doubtful || (row_ok && !(nonfinite == 0.f));
-                    mark();
-                }
             }
         };
         run(IntC<0>());

@@ -60,3 +60,42 @@ def test_undefined_rows_stay_alone(B, d, plan_id):
     for h, t in MARKED:
         Ob[h, t * 128 + 7], Lb[h, t * 128 + 7] = O[h, t * 128 + 7], L[h, t * 128 + 7]
     Hh.compare_with_oracle(req, Ob, Lb, cpu)
+
+
+def _against_64_bits(scores_of_keys, values, d, N_kv):
+    """One head of 300 rows, dense, every row with (about) the given score per key; outputs against 64 bits."""
+    gen = torch.Generator().manual_seed(d)
+    q, k, v = (torch.randn(1, n, d, generator=gen) for n in (300, N_kv, N_kv))
+    q[..., 0] = 8.0
+    k[..., 0] = scores_of_keys * (d ** 0.5 / 8.0)
+    q, k, v = (t.bfloat16().cuda() for t in (q, k * torch.tensor([1.0] + [0.1] * (d - 1)), v * values[None, :, None]))
+    mask = torch.ones(1, 3, I.cdiv(N_kv, 128), dtype=torch.uint8, device="cuda")
+    with bsa.plan_create(mask, 128, 128, 300, 1, d, plan_id=22, N_kv=N_kv) as plan:
+        O, L = plan.forward(q, k, v)
+        assert plan.info()["device_status"] == 0
+    S = q[0].double() @ k[0].double().t() / d ** 0.5
+    ref = torch.softmax(S, dim=1) @ v[0].double()
+    assert torch.isfinite(O.float()).all()
+    assert (L[0].double() - torch.logsumexp(S, dim=1)).abs().max() <= 1e-4
+    # P and O are rounded to bf16 (2^-9 each, P's share of the normalisation another 2^-9), relative to the largest |v|
+    assert (O[0].double() - ref).abs().max() <= 4 * 2.0 ** -9 * v.double().abs().max()
+
+
+@pytest.mark.parametrize("d", [64, 128])
+@pytest.mark.parametrize("low", [0, 1])  # the tiles of this parity start low and catch up
+def test_one_half_of_the_tiles_outgrows_its_first(d, low):
+    """At d = 64 each half of an item's tiles has its own reference and accumulator.  One half starts 2^87 below the other and
+    reaches it at its second tile: its sum stays below 2^100 and the item's total is small, its accumulator overflows."""
+    N_kv = 40 * 128
+    s = torch.zeros(40)
+    s[1 - low], s[low + 2] = 60.0, 60.0
+    _against_64_bits(s.repeat_interleave(128), torch.full((N_kv,), 2.0 ** 60), d, N_kv)
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_one_large_value_behind_a_moderate_weight(d):
+    """A weight of 2^20 against the first tile on a value of about 2^110: their product overflows, the row's sum is small."""
+    N_kv = 40 * 128
+    s, x = torch.zeros(N_kv), torch.ones(N_kv)
+    s[700], x[700] = 14.0, 2.0 ** 110
+    _against_64_bits(s, x, d, N_kv)
