@@ -1700,7 +1700,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                 const float sa = inv_l * wa, sb = inv_l * wb;
                 // An accumulator can overflow where the running maximum's weights of at most 2^8 would not: however small the row's
                 // sum is, its outputs decide as well (d = 64: those of either accumulator, weighted by zero or not).
-                uint64_t nf0 = pack_f32x2(0.f, 0.f), nf1 = nf0;  // zero as long as every output is finite
+                uint64_t nf = pack_f32x2(0.f, 0.f);  // zero as long as every output is finite
 #pragma unroll 1  // once per item: a rolled loop keeps the kernel's code small
                 for (int c = 0; c < D / CW; ++c) {
                     uint32_t o[CW];
@@ -1728,13 +1728,11 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                     if (kFirstRef && pass == 0) {
                         const uint64_t zero2 = pack_f32x2(0.f, 0.f);
 #pragma unroll
-                        for (int e = 0; e < CW; e += 4) {
-                            nf0 = fma_f32x2(pack_f32x2(__uint_as_float(o[e]), __uint_as_float(o[e + 1])), zero2, nf0);
-                            nf1 = fma_f32x2(pack_f32x2(__uint_as_float(o[e + 2]), __uint_as_float(o[e + 3])), zero2, nf1);
-                        }
+                        for (int e = 0; e < CW; e += 2)
+                            nf = fma_f32x2(pack_f32x2(__uint_as_float(o[e]), __uint_as_float(o[e + 1])), zero2, nf);
                         if (c == D / CW - 1) {
                             float f0, f1;
-                            unpack_f32x2(add_f32x2(nf0, nf1), f0, f1);
+                            unpack_f32x2(add_f32x2(nf, zero2), f0, f1);  // (without this sum ptxas' d = 64 loops are 1.5 % slower)
                             if (__any_sync(0xffffffffu, doubtful || (row_ok && !(f0 + f1 == 0.f))) && lane == 0) {
                                 const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
                                 atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
