@@ -1437,7 +1437,10 @@ struct __align__(8) PpBarriers {
     uint64_t s_full[2], s_free[2], p_ready[2], pv_done[2];
 };
 
-constexpr int kRedoBits = 512;  // rounds of a CTA told apart when items are computed again
+// Rounds of a CTA at most where items can be computed again: each has its own mark (an item that shared one would be computed
+// again with the other, in another form).  1024 marks are what the kernel's static shared memory has left; a list of more than
+// 1024 items per SM is shared out among twice as many CTAs, or more (see the launch).
+constexpr int kRedoBits = 1024;
 template <int V>
 struct IntC {
     static constexpr int value = V;
@@ -1571,7 +1574,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // Pass 0 goes through all of the CTA's items, pass 1 (bf16) through those that the epilogue has marked.
     auto item_at = [&](auto pass_c, int kr) -> int {  // the list's index of round kr, past the end where the pass leaves it out
         if constexpr (decltype(pass_c)::value == 1) {
-            const int bit = kr % kRedoBits;
+            const int bit = kr % kRedoBits;  // (kr runs up to two rounds past the end)
             if (!((redo_bits[bit >> 5] >> (bit & 31)) & 1u)) return n_items;
         }
         return cta_item_index(kr, blockIdx.x, gridDim.x);
@@ -1734,8 +1737,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
                             float f0, f1;
                             unpack_f32x2(add_f32x2(nf, zero2), f0, f1);  // (without this sum ptxas' d = 64 loops are 1.5 % slower)
                             if (__any_sync(0xffffffffu, doubtful || (row_ok && !(f0 + f1 == 0.f))) && lane == 0) {
-                                const int bit = kr % kRedoBits;  // (of more rounds than bits several share one)
-                                atomicOr(&redo_bits[bit >> 5], 1u << (bit & 31));
+                                atomicOr(&redo_bits[kr >> 5], 1u << (kr & 31));
                                 redo_any = 1u;
                             }
                             if (kr == n_rounds - 1) {  // the verdict on the CTA's last item is in
@@ -2706,6 +2708,8 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         cudaError_t le = cudaErrorInvalidValue;
         // (at d = 128 the K producer of the short form relies on the two K tiles)
         const bool short_form = D == 64 ? (G == 2 || a.f16 || !a.long_lists) : (a.short_lists && p.stages == 2 && p.stages_v > 2);
+        if (!short_form && !a.f16)  // whole waves of CTAs, of at most kRedoBits rounds each (max_items bounds the list's length)
+            cfg.gridDim.x = (unsigned)(((int64_t)a.max_items + (int64_t)kRedoBits * grid - 1) / ((int64_t)kRedoBits * grid) * grid);
         if (short_form) {
             le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, true>) : launch(bsa_attention_pp_kernel<D, false, G, true>);
         } else if constexpr (D != 64) {

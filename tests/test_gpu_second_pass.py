@@ -99,3 +99,29 @@ def test_one_large_value_behind_a_moderate_weight(d):
     s, x = torch.zeros(N_kv), torch.ones(N_kv)
     s[700], x[700] = 14.0, 2.0 ** 110
     _against_64_bits(s, x, d, N_kv)
+
+
+def test_marks_are_not_shared_in_long_lists():
+    """More than 1024 items per SM: items computed again change no bit of any other, whose scores outgrow their first tile too."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    H, d, nk = 64, 128, 12
+    nq = 1024 * sms // H + 5
+    N, N_kv = nq * 128, nk * 128
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    q = torch.randn(H, N, d, device="cuda", generator=gen, dtype=torch.bfloat16)
+    k, v = (torch.randn(H, N_kv, d, device="cuda", generator=gen, dtype=torch.bfloat16) for _ in range(2))
+    k[:, -200:] *= 8
+    mask = torch.ones(H, nq, nk, dtype=torch.uint8, device="cuda")
+    marked = [(0, 1), (17, nq // 2), (40, 3), (63, nq - 1)]
+    with bsa.plan_create(mask, 128, 128, N, H, d, plan_id=22, N_kv=N_kv) as plan:
+        O, L = plan.forward(q, k, v)
+        for h, t in marked:
+            q[h, t * 128:(t + 1) * 128] *= 60
+        Ob, Lb = plan.forward(q, k, v)
+        assert plan.info()["device_status"] == 0 and plan.info()["nitems"] > 1024 * sms
+    same = torch.ones(H, nq, dtype=torch.bool, device="cuda")
+    for h, t in marked:
+        same[h, t] = False
+        assert not torch.equal(Lb[h, t * 128:(t + 1) * 128], L[h, t * 128:(t + 1) * 128])
+    assert ((O.view(H, nq, -1) == Ob.view(H, nq, -1)).all(dim=2) | ~same).all()
+    assert ((L.view(H, nq, -1) == Lb.view(H, nq, -1)).all(dim=2) | ~same).all()
