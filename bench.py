@@ -40,7 +40,7 @@ NCU_TRAFFIC_BYTES = {
     "stress_a": (266.9e6, "one ncu capture of one launch of this workload (row-block kernel)"),
 }
 KERNEL_NAMES = {0: "bsa_attention_kernel<D,TK,false>", 1: "bsa_attention_pair_kernel<D,TK>", 2: "bsa_attention_cs_kernel<D,TK>",
-                3: "bsa_attention_kernel<D,TK,true>", 4: "bsa_attention_pp_kernel<D,F16,G,SMEM_Q>", 5: "bsa_attention_rb_kernel<D,CK>"}
+                3: "bsa_attention_kernel<D,TK,true>", 4: "bsa_attention_pp_kernel<D,F16,G,SHORT,FIRST_REF>", 5: "bsa_attention_rb_kernel<D,CK>"}
 TENSOR_FLOP_PER_CLK_PER_SM = 8192  # dense bf16, fp32 accumulate
 
 

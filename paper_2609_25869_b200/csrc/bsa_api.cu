@@ -87,7 +87,7 @@ struct bsa_plan {
     // measured there).  Exact where no dimension is Coarsened; a Coarsened list is taken to be that of independent blocks, at
     // most the true length's multiple by the blocks per tile, on a line where the two forms are within 2 % of each other.
     int32_t short_lists;
-    int32_t long_lists;  // 32 tiles and more, on the same estimate: the form of the ping-pong kernel at d = 64 follows from it
+    int32_t first_refs;  // lists on which a row's first reference maximum serves the whole item (bf16, see choose_list_form)
     // Split-K workspace
     float* ws_O;
     float* ws_LSE;
@@ -179,6 +179,41 @@ static bool release_plan(bsa_plan* p) {
     if (p->refs.fetch_sub(1, std::memory_order_acq_rel) > 1) return false;
     free_plan(p);
     return true;
+}
+
+// The form of the ping-pong kernel that suits the plan's lists, from the mean number of 128-key tiles per work item (see
+// bsa_plan::short_lists).  In bf16 a row's first reference maximum is kept on lists that are long enough for it, and long next
+// to the time until all rows have been reached: until then some of the softmax warps look for maxima and some do not, they no
+// longer share their instructions' fetches, and a tile takes longer than where all follow the running maximum.  For independent
+// blocks a row block is active in a listed tile with probability q, and the last of b row blocks is reached after about
+// (1 + 1/2 + .. + 1/b) / -ln(1 - q) tiles.  First references against the running maximum, 4 heads of 9472 tokens,
+// tiles per item / ratio of times (rows reached after):
+//   d = 128, (16,64) blocks 9 1.07, 16 1.09, 30 1.04, 60 0.96 (10); (32,64) 9 1.01, 16 1.00, 30 0.97 (4); (64,64) 9 0.97,
+//   16 0.98, 30 0.97 (1); (16,128) 9 1.10, 16 1.09, 30 1.06, 60 0.97 (20); (32,128) 9 1.06, 16 1.02, 30 0.98, 60 0.91 (7);
+//   (64,128) 9 1.03, 16 0.99, 30 0.95 (2); one block per row 8 0.95; tiles of four entries always gain ((16,32) 11 0.92)
+//   d = 64, (16,128) 34 1.10, 64 1.08, 100 1.06 (20); (32,128) 34 1.05, 64 1.02, 100 0.99 (7); (16,32) 34 1.03, 44 1.02, 64 0.98 (5);
+//   (32,32) 34 0.98 (2); (128,128) 34 0.97; four entries to a tile and nothing masked, (128,32), 34 1.01, 44 1.01, 64 1.00, 100 0.98
+//   (the line of these tiles lies at 48: neighbouring rows share columns in real masks and the estimate is too high for them,
+//   19392 tokens, 3 heads, (32,16), 39 tiles by the estimate and 18 in truth, first call 122.5 us against 120.0)
+static void choose_list_form(bsa_plan* p, double density, int pmax) {
+    const MapGeom& g = p->g;
+    const double listed = 1.0 - pow(1.0 - density, (double)(g.sQ * g.sK));
+    const double entries = (double)g.nKt * listed;
+    const double parts = pmax > 1 ? fmin((double)pmax, fmax(1.0, entries / p->desc.split_tau)) : 1.0;
+    const double tiles = entries * p->desc.T_KV / (128.0 * parts);
+    const int per_tile = 128 / p->desc.T_KV;  // entries
+    double reached = 0.0;
+    if (g.sQ > 1 && listed > 0.0 && density < 1.0) {
+        const double own = fmin(1.0, (1.0 - pow(1.0 - density, (double)g.sK)) / listed);
+        const double missed = pow(1.0 - own, (double)per_tile);  // 1 - q
+        for (int b = 1; b <= g.sQ; ++b) reached += 1.0 / b;
+        reached = missed > 0.0 ? reached / -log(missed) : 0.0;
+    }
+    p->short_lists = tiles < 8.0;
+    double line;
+    if (p->d == 64) line = fmax(per_tile == 4 ? 48.0 : 32.0, 12.0 * reached);
+    else line = per_tile == 4 ? 8.0 : 8.0 + 2.0 * per_tile * reached;
+    p->first_refs = p->dtype == BSA_DTYPE_BF16 && tiles >= line;
 }
 
 // `packed_stride` = 0: one byte per logical block; > 0: bit-packed rows of that many bytes (bsa_plan_create_packed).
@@ -454,12 +489,7 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
     const int pmax = p->desc.split_pmax < 1 ? 1 : p->desc.split_pmax;
     const int64_t trows = (int64_t)heads * g.nQt;
     p->max_items = trows * pmax;
-    {
-        const double entries = (double)g.nKt * (1.0 - pow(1.0 - density, (double)(g.sQ * g.sK)));
-        const double parts = pmax > 1 ? fmin((double)pmax, fmax(1.0, entries / p->desc.split_tau)) : 1.0;
-        p->short_lists = entries * p->desc.T_KV < 8.0 * 128.0 * parts;
-        p->long_lists = entries * p->desc.T_KV >= 32.0 * 128.0 * parts;
-    }
+    choose_list_form(p, density, pmax);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
     const size_t o_col = early_fill ? 0 : take(sizeof(int32_t) * (size_t)(nnz_i + 1));
@@ -652,7 +682,7 @@ static void fill_forward_args(const bsa_plan_t* p, const void* Q, const void* K,
     a.kernel = p->desc.kernel;
     a.has_split = p->desc.split_pmax > 1;
     a.short_lists = p->short_lists;
-    a.long_lists = p->long_lists;
+    a.first_refs = p->first_refs;
     a.max_items = (int32_t)(p->max_items < (1 << 30) ? p->max_items : (1 << 30));
     a.max_split_rows = p->g.H * p->g.nQt * p->g.slots;
     a.num_sms = p->num_sms;

@@ -1355,10 +1355,14 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // at 44 % 276 / 215.  The running maximum stays for half, which has no such range, and for short lists, where the second copy
 // of the loop costs more than it saves (d = 128, 32768 tokens, 8 heads, two tiles per item 74 -> 82 us; d = 64, 2048 tokens, 2
 // heads 16.5 -> 18.5, 10240 tokens, 8 heads, 9 tiles of runs 55 -> 63; 16384 tokens, 16 heads, (32,32), 15 tiles 244 -> 250);
-// at d = 64 also for tiles of two entries ((64,64) at 48 tiles 1360 -> 1440).  Both forms take a row's reference from the same
-// tile, so that an item whose scores do not outgrow it by 2^8 has the same bits in either.
-// Two kernels and not a flag in one: what an item pays at its boundary is mostly instruction fetch, and the softmax code
-// has no register to spare (one kernel with both bodies was 1-2 % slower on long lists).
+// at d = 64 also for tiles of two entries ((64,64) at 48 tiles 1360 -> 1440); and for lists that are short next to the time until
+// all rows of a tile have been reached (choose_list_form in bsa_api.cu has the lines).  Both forms take a row's reference from
+// the same tile, so that an item whose scores do not outgrow it by 2^8 has the same bits in either.
+// What the second pass costs: an item with one marked row is computed twice by its CTA.  32768 tokens, 8 heads, no item marked /
+// one in a hundred / all, the running maximum in brackets: (128,128) 24 tiles 304 / 353 / 664 (329) us, (128,64) 333 / 382 / 774
+// (350), (128,32) 329 / 364 / 862 (380); d = 64, 40 tiles, (128,128) 484 / 562 / 1000 (490), (128,32) 480 / 517 / 935 (475).
+// Kernels and not flags in one: what an item pays at its boundary is mostly instruction fetch, and the softmax code
+// has no register to spare (one kernel with both places of Q was 1-2 % slower on long lists).
 //
 // G: a 128-key tile is made up of G entries of the plan's tile list (T_KV = 128 / G keys each), whichever they are: the
 // producers copy them one by one, and a 128-row, 128-column MMA works on a tile without gaps.  G = 1 where the logical
@@ -1473,7 +1477,7 @@ struct TileKeys {
     }
 };
 
-template <int D, bool F16, int G, bool kShort>
+template <int D, bool F16, int G, bool kShort, bool kFirstRef>
 __global__ void __launch_bounds__(kPpThreads, 1)
 bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmK,
                         const __grid_constant__ CUtensorMap tmV, const AttnParams p) {
@@ -1488,7 +1492,7 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     using Cols = PpCols<D>;
     constexpr bool kSmemQ = kShort || D == 64;  // (at d = 64 no tensor-memory columns are left for Q)
     constexpr bool kOwnO = Cols::kOwnO;
-    constexpr bool kFirstRef = !F16 && !kShort;  // a row's first reference serves the whole item (see above)
+    static_assert(!(kFirstRef && (F16 || kShort)), "a row's first reference serves the whole item: long lists in bf16 only");
     static_assert(kOwnO || NSUB * Q_SUB == KV_TILE, "at d = 128 the second Q tile takes the place of a V tile");
     // dynamic shared memory starts on a 1024-byte boundary (the swizzled tiles need it); checked below
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -2663,13 +2667,15 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
             e = cudaFuncSetAttribute(bsa_attention_cs_kernel<D, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         else {
             const auto allow = [&](auto kernel) { return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem); };
-            e = allow(bsa_attention_pp_kernel<D, false, G, true>);
-            if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, true>);
+            e = allow(bsa_attention_pp_kernel<D, false, G, true, false>);
+            if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, true, false>);
             if constexpr (D != 64 || G != 2) {
-                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, false, G, false>);
+                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, false, G, false, true>);
             }
             if constexpr (D != 64) {
-                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, false>);
+                if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, true, G, false, false>);
+                if constexpr (G != 4)
+                    if (e == cudaSuccess) e = allow(bsa_attention_pp_kernel<D, false, G, false, false>);
             }
         }
         if (e != cudaSuccess) {
@@ -2706,16 +2712,19 @@ cudaError_t launch_attn(const ForwardArgs& a, const AttnParams& p, cudaStream_t 
         cfg.numAttrs = 1;
         const auto launch = [&](auto kernel) { return cudaLaunchKernelEx(&cfg, kernel, tq, tk, tv, p); };
         cudaError_t le = cudaErrorInvalidValue;
-        // (at d = 128 the K producer of the short form relies on the two K tiles)
-        const bool short_form = D == 64 ? (G == 2 || a.f16 || !a.long_lists) : (a.short_lists && p.stages == 2 && p.stages_v > 2);
-        if (!short_form && !a.f16)  // whole waves of CTAs, of at most kRedoBits rounds each (max_items bounds the list's length)
+        // (at d = 128 the K producer of the short form relies on the two K tiles; tiles of two entries at d = 64 and of four at
+        // d = 128 have one long form each, which serves them all: see choose_list_form)
+        const bool short_form = D == 64 ? (G == 2 || !a.first_refs) : (a.short_lists && p.stages == 2 && p.stages_v > 2);
+        const bool first_refs = !short_form && !a.f16 && (a.first_refs || G == 4);
+        if (first_refs)  // whole waves of CTAs, of at most kRedoBits rounds each (max_items bounds the list's length)
             cfg.gridDim.x = (unsigned)(((int64_t)a.max_items + (int64_t)kRedoBits * grid - 1) / ((int64_t)kRedoBits * grid) * grid);
         if (short_form) {
-            le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, true>) : launch(bsa_attention_pp_kernel<D, false, G, true>);
+            le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, true, false>) : launch(bsa_attention_pp_kernel<D, false, G, true, false>);
+        } else if (first_refs) {
+            if constexpr (D != 64 || G != 2) le = launch(bsa_attention_pp_kernel<D, false, G, false, true>);
         } else if constexpr (D != 64) {
-            le = a.f16 ? launch(bsa_attention_pp_kernel<D, true, G, false>) : launch(bsa_attention_pp_kernel<D, false, G, false>);
-        } else if constexpr (G != 2) {
-            le = launch(bsa_attention_pp_kernel<D, false, G, false>);
+            if (a.f16) le = launch(bsa_attention_pp_kernel<D, true, G, false, false>);
+            else if constexpr (G != 4) le = launch(bsa_attention_pp_kernel<D, false, G, false, false>);
         }
         count_launch();
         return le;

@@ -115,7 +115,7 @@ struct ForwardArgs {
     int32_t kernel;
     int32_t has_split;
     int32_t short_lists;     // the plan's work items have few tiles (see bsa_plan::short_lists)
-    int32_t long_lists;      // or many
+    int32_t first_refs;      // or suit a row's first reference (see choose_list_form)
     int32_t max_items;       // host-side upper bound of the item count
     int32_t max_split_rows;  // host-side upper bound
     int32_t num_sms;

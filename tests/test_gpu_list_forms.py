@@ -1,0 +1,22 @@
+"""Lists whose rows are reached late, or by no tile at all, on both sides of the lines where the ping-pong kernel changes its
+form: a few active blocks per row block, in lists of many tiles that its neighbours need."""
+import numpy as np
+import pytest
+
+from paper_2609_25869_b200 import inputs as I
+from tests import helpers as Hh
+
+pytestmark = pytest.mark.gpu
+
+
+# (d, blocks, plan, 128-key tiles in all, density): about 9, 25 and 70 tiles per item at d = 128, 34 and 180 at d = 64
+@pytest.mark.parametrize("d,B,plan_id,n_kt,density", [
+    (128, (16, 64), 23, 75, 0.016), (128, (16, 64), 23, 180, 0.02), (128, (16, 64), 23, 180, 0.06),
+    (128, (32, 64), 23, 75, 0.032), (128, (32, 64), 23, 75, 0.1), (128, (16, 128), 22, 75, 0.016), (128, (16, 128), 22, 180, 0.06),
+    (128, (16, 32), 39, 75, 0.02), (64, (16, 128), 22, 75, 0.08), (64, (16, 128), 22, 400, 0.09), (64, (32, 128), 22, 180, 0.15),
+    (64, (16, 32), 39, 75, 0.08), (64, (128, 32), 39, 100, 0.4), (64, (128, 32), 39, 100, 0.6)])
+def test_rows_reached_late(d, B, plan_id, n_kt, density):
+    H, N, N_kv = 2, 5 * 128 - 7, n_kt * 128 - 11
+    M = I.random_mask(d + B[0] + n_kt, H, I.cdiv(N, B[0]), I.cdiv(N_kv, B[1]), density, empty_rows=0.05)
+    M[1, ::3, : -M.shape[2] // 8] = 0  # every third row block of one head: the last eighth of the keys only
+    Hh.run_request(I.Request("late", H, N, d, B[0], B[1], M, qkv_seed=n_kt, N_kv=N_kv), plan_id=plan_id)
