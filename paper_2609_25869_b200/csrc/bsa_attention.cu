@@ -1622,15 +1622,21 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if (!__all_sync(0xffffffffu, good)) return false;
             tc_fence_after();
             const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + Cols::kQ;
+            // swizzled 16-byte chunks of this row at a time: more of them spill beside the verdict on first references, and half's
+            // other tiles are slower with them (58594 tokens, 15 heads, (64,128) 2910 / 3015 us; four entries to a tile, 55376 tokens, 3 heads
+            // 2517 / 2486)
+            constexpr int PC = F16 && G == 4 ? 8 : 4;
 #pragma unroll 1
-            for (int s = 0; s < 2 * NSUB; ++s) {  // 32 head-dimension columns: four swizzled 16-byte chunks of this row
-                uint32_t v[16];
+            for (int s = 0; s < 8 * NSUB / PC; ++s) {
+                uint32_t v[4 * PC];
+                const uint8_t* row = sQ + (s * PC >> 3) * Q_SUB + tw * 128;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    const uint4 w = *reinterpret_cast<const uint4*>(sQ + (s >> 1) * Q_SUB + tw * 128 + ((((s & 1) * 4 + c) ^ (tw & 7)) << 4));
+                for (int c = 0; c < PC; ++c) {
+                    const uint4 w = *reinterpret_cast<const uint4*>(row + (((s * PC & 7) + c) ^ (tw & 7)) * 16);
                     v[4 * c] = w.x; v[4 * c + 1] = w.y; v[4 * c + 2] = w.z; v[4 * c + 3] = w.w;
                 }
-                tmem_st16(t_q + s * 16, v);
+                if constexpr (PC == 8) tmem_st32(t_q + s * 32, v);
+                else tmem_st16(t_q + s * 16, v);
             }
             mbar_arrive(smem_u32(&bars.q_drained));
             tc_wait_st();
