@@ -1622,9 +1622,9 @@ bsa_attention_pp_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
             if (!__all_sync(0xffffffffu, good)) return false;
             tc_fence_after();
             const uint32_t t_q = tmem + ((uint32_t)((warp & 3) * 32) << 16) + Cols::kQ;
-            // swizzled 16-byte chunks of this row at a time: more of them spill beside the verdict on first references, and half's
-            // other tiles are slower with them (58594 tokens, 15 heads, (64,128) 2910 / 3015 us; four entries to a tile, 55376 tokens, 3 heads
-            // 2517 / 2486)
+            // Swizzled 16-byte chunks of this row at a time.  Eight of them spill beside the verdict on first references; in half
+            // tiles of four entries are faster with eight (16384 tokens, 4 heads, (32,32) 143.0 -> 141.1 us, 2 heads, (16,16) 172.1 -> 170.4), the
+            // others are not (58594 tokens, 15 heads, (64,128) 2910 -> 3015).
             constexpr int PC = F16 && G == 4 ? 8 : 4;
 #pragma unroll 1
             for (int s = 0; s < 8 * NSUB / PC; ++s) {

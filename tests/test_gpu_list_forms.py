@@ -1,8 +1,9 @@
 """Lists whose rows are reached late, or by no tile at all, on both sides of the lines where the ping-pong kernel changes its
 form: a few active blocks per row block, in lists of many tiles that its neighbours need."""
-import numpy as np
 import pytest
+import torch
 
+from paper_2609_25869_b200 import bsa
 from paper_2609_25869_b200 import inputs as I
 from tests import helpers as Hh
 
@@ -20,3 +21,25 @@ def test_rows_reached_late(d, B, plan_id, n_kt, density):
     M = I.random_mask(d + B[0] + n_kt, H, I.cdiv(N, B[0]), I.cdiv(N_kv, B[1]), density, empty_rows=0.05)
     M[1, ::3, : -M.shape[2] // 8] = 0  # every third row block of one head: the last eighth of the keys only
     Hh.run_request(I.Request("late", H, N, d, B[0], B[1], M, qkv_seed=n_kt, N_kv=N_kv), plan_id=plan_id)
+
+
+@pytest.mark.parametrize("d,B,plan_id", [(64, 128, 22), (64, 32, 39), (128, 64, 23), (128, 128, 22)])
+def test_heads_of_a_whole_request_equal_the_heads_alone(d, B, plan_id):
+    """Long lists that keep first references, some of their items computed again: 720 items against 45, bit for bit."""
+    H, N, N_kv = 16, 45 * 128 - 9, 63 * 128 - 5
+    M = I.random_mask(d + B, H, I.cdiv(N, B), I.cdiv(N_kv, B), 0.85, empty_rows=0.05)
+    req = I.Request("position", H, N, d, B, B, M, qkv_seed=B, N_kv=N_kv)
+    mask, q, k, v, _ = Hh.to_dev(req)
+    for h in range(H):
+        for t in {(7 * h + 2) % 45, (11 * h) % 45, 44}:
+            q[h, t * 128 + 9:t * 128 + 30] *= 200
+    kw = {"N_kv": N_kv, "plan_id": plan_id}
+    with bsa.plan_create(mask, B, B, N, H, d, **kw) as plan:
+        O, L = plan.forward(q, k, v)
+        assert plan.info()["nitems"] > 4 * torch.cuda.get_device_properties(0).multi_processor_count
+    for h in range(H):
+        one = slice(h, h + 1)
+        with bsa.plan_create(mask[one].contiguous(), B, B, N, 1, d, **kw) as plan:
+            Oh, Lh = plan.forward(q[one].contiguous(), k[one].contiguous(), v[one].contiguous())
+            assert plan.info()["device_status"] == 0
+        assert torch.equal(Lh, L[one]) and torch.equal(Oh, O[one]), h
