@@ -195,7 +195,14 @@ static bool release_plan(bsa_plan* p) {
 //   (32,32) 34 0.98 (2); (128,128) 34 0.97; four entries to a tile and nothing masked, (128,32), 34 1.01, 44 1.01, 64 1.00, 100 0.98
 //   (the line of these tiles lies at 48: neighbouring rows share columns in real masks and the estimate is too high for them,
 //   19392 tokens, 3 heads, (32,16), 39 tiles by the estimate and 18 in truth, first call 122.5 us against 120.0)
-static void choose_list_form(bsa_plan* p, double density, int pmax) {
+// Where many more blocks lie in runs than of independent ones would (1 - (1 - density)^2 of them), the estimate of when rows are
+// reached says nothing.  Neighbourhoods with stripes / runs that differ from row to row, 4 to 6 heads, ratios as above:
+//   d = 128, (16,64) 1.00-1.13 / 1.01-1.15 (5280 to 16384 tokens), (32,64) 0.94-1.11 / 0.98-1.06, (32,128) 0.93-1.05 / 0.93-1.01,
+//   (64,64) 0.92-1.03 / 0.93-1.03, (64,128) 0.91-0.97 / 0.92-0.98, (16,16) 0.84-0.91 / 0.81-0.87;
+//   d = 64, (32,32) 0.98-1.04 / 1.04-1.08, (16,16) 0.96-1.05 / 1.05-1.11, (64,32) 0.99-1.02 / 0.99-1.04, (64,128) 0.98-1.02 / 0.97-1.02.
+// There the running maximum stays for four and more row blocks to a tile (but in the d = 128 tiles of one entry with 32-row blocks and
+// of four), and for all masked tiles of four entries at d = 64.
+static void choose_list_form(bsa_plan* p, double density, double run_cov, int pmax) {
     const MapGeom& g = p->g;
     const double listed = 1.0 - pow(1.0 - density, (double)(g.sQ * g.sK));
     const double entries = (double)g.nKt * listed;
@@ -210,10 +217,17 @@ static void choose_list_form(bsa_plan* p, double density, int pmax) {
         reached = missed > 0.0 ? reached / -log(missed) : 0.0;
     }
     p->short_lists = tiles < 8.0;
+    const bool clustered = run_cov > 1.3 * (1.0 - (1.0 - density) * (1.0 - density));
     double line;
-    if (p->d == 64) line = fmax(per_tile == 4 ? 48.0 : 32.0, 12.0 * reached);
-    else line = per_tile == 4 ? 8.0 : 8.0 + 2.0 * per_tile * reached;
-    p->first_refs = p->dtype == BSA_DTYPE_BF16 && tiles >= line;
+    bool late;
+    if (p->d == 64) {
+        line = fmax(per_tile == 4 ? 48.0 : 32.0, 12.0 * reached);
+        late = clustered && g.sQ >= (per_tile == 4 ? 2 : 4);
+    } else {
+        line = per_tile == 4 ? 8.0 : 8.0 + 2.0 * per_tile * reached;
+        late = clustered && (per_tile == 4 ? false : per_tile == 2 ? g.sQ >= 4 : g.sQ >= 8);
+    }
+    p->first_refs = p->dtype == BSA_DTYPE_BF16 && tiles >= line && !late;
 }
 
 // `packed_stride` = 0: one byte per logical block; > 0: bit-packed rows of that many bytes (bsa_plan_create_packed).
@@ -489,7 +503,7 @@ static bsa_status_t create_impl(const uint8_t* mask_dev, int64_t packed_stride, 
     const int pmax = p->desc.split_pmax < 1 ? 1 : p->desc.split_pmax;
     const int64_t trows = (int64_t)heads * g.nQt;
     p->max_items = trows * pmax;
-    choose_list_form(p, density, pmax);
+    choose_list_form(p, density, run_cov, pmax);
     size_t o = 0;
     auto take = [&](size_t bytes) { size_t r = o; o = align_up(o + bytes); return r; };
     const size_t o_col = early_fill ? 0 : take(sizeof(int32_t) * (size_t)(nnz_i + 1));

@@ -13,14 +13,15 @@
 //   * S = Q K^T, online softmax with the running row maximum in the exp2 domain, P rounded to bf16 in registers
 //     (the accumulator layout of two 8-key tiles is the A-operand layout of one 16-key step), O += P V;
 //   * no block-level synchronisation: twelve independent warps per SM, each takes the next of the CTA's items when it is free.
-// A block of 16 rows and 64 keys (d = 64) is 262 kflop on 16 KB of K and V, each byte used once: shared memory sees it
-// twice (copy in, ldmatrix), 256 clk per SM at 128 B/clk against 133 clk of MMA, which makes 2.2 ms of the workload
-// below.  With per-thread cp.async copies of whole entries the load path stopped at about 41 B/clk per SM (bulk copies
-// reach 80); now, on one GPU, 32768 tokens, 16 heads, d = 64, (16,64) blocks, 15 % active in runs: 3.58 -> 2.77 ms; the
-// same with 32-key entries 4.01 -> 2.94 ms, (32,32) blocks at d = 128 52 -> 40 ms; maxima agreed on only where one has moved,
-// and items taken by free warps instead of a fixed share each: 2.82 -> 2.50, independent blocks at 15 % 2.48 -> 2.28, (16,16)
-// blocks at 10 %, 16384 tokens, 4 heads 222 -> 182 us.  (Fragments loaded straight from
-// global memory, no shared memory at all: 5.4 ms, the L1 miss path moves about 32 B/clk.  Fourteen warps: spills, 3.95.)
+// A block of 16 rows and 64 keys (d = 64) is 262 kflop on 16 KB of K and V, each byte used once: 133 clk of MMA per SM, and
+// shared memory sees the bytes twice (copy in, ldmatrix).  The kernel takes 242 clk a block: tensor pipe 53 % busy, issue 44 %,
+// its three warps per sub-partition mostly wait for the latency of their own instructions.  With per-thread cp.async copies
+// of whole entries the load path stopped at about 41 B/clk per SM (bulk copies reach 80); now, on one GPU, 32768 tokens, 16
+// heads, d = 64, (16,64) blocks, 15 % active in runs: 3.58 -> 2.77 ms; the same with 32-key entries 4.01 -> 2.94 ms, (32,32)
+// blocks at d = 128 52 -> 40 ms; maxima agreed on only where one has moved, and items taken by free warps instead of a fixed
+// share each: 2.82 -> 2.50, independent blocks at 15 % 2.48 -> 2.28, (16,16) blocks at 10 %, 16384 tokens, 4 heads
+// 214 -> 170 us.  (Fragments loaded straight from global memory, no shared memory at all: 5.4 ms, the L1 miss path moves
+// about 32 B/clk.  Fourteen warps: spills, 3.95.)
 // The register-level instruction peaks at about a third of the tcgen05 rate on this GPU, so the kernel pays off only
 // where Coarsening wastes more than that; the plan table decides per regime.
 #include <cuda.h>

@@ -1,5 +1,6 @@
 """Lists whose rows are reached late, or by no tile at all, on both sides of the lines where the ping-pong kernel changes its
 form: a few active blocks per row block, in lists of many tiles that its neighbours need."""
+import numpy as np
 import pytest
 import torch
 
@@ -43,3 +44,25 @@ def test_heads_of_a_whole_request_equal_the_heads_alone(d, B, plan_id):
             Oh, Lh = plan.forward(q[one].contiguous(), k[one].contiguous(), v[one].contiguous())
             assert plan.info()["device_status"] == 0
         assert torch.equal(Lh, L[one]) and torch.equal(Oh, O[one]), h
+
+
+@pytest.mark.parametrize("d,B,plan_id", [(128, (16, 64), 23), (128, (32, 64), 23), (128, (32, 128), 22), (128, (64, 64), 23),
+                                         (64, (32, 32), 39), (64, (64, 128), 22)])
+@pytest.mark.parametrize("layout", ["hnd", "nhd"])
+def test_runs_that_differ_from_row_to_row(d, B, plan_id, layout):
+    """Two runs of keys per row block, wherever they begin: many more blocks in runs than independent ones would have."""
+    H, N, N_kv = 2, 4 * 128 - 3, 130 * 128 - 21
+    nq, nk = I.cdiv(N, B[0]), I.cdiv(N_kv, B[1])
+    rng = np.random.RandomState(d + B[0])
+    M = np.zeros((H, nq, nk), np.uint8)
+    for h in range(H):
+        for i in range(nq):
+            for a in rng.randint(0, nk - nk // 6, 2):
+                M[h, i, a:a + nk // 6] = 1
+    req = I.Request("runs", H, N, d, B[0], B[1], M, qkv_seed=d, N_kv=N_kv)
+    mask, q, k, v, cpu = Hh.to_dev(req)
+    nhd = layout == "nhd"
+    with bsa.plan_create(mask, *B, N, H, d, plan_id=plan_id, N_kv=N_kv, layout=layout) as plan:
+        O, L = plan.forward(*(t.transpose(0, 1).contiguous() if nhd else t for t in (q, k, v)))
+        assert plan.info()["device_status"] == 0
+    Hh.compare_with_oracle(req, O.transpose(0, 1).contiguous() if nhd else O, L, cpu)
