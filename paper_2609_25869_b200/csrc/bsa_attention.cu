@@ -1351,8 +1351,8 @@ bsa_attention_cs_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 // maximum as before, moved by more than 2^8 at a time.  Per 128-key tile the softmax chain falls by a fifth.  Builds in turn,
 // back to back, before / after: 16384 tokens, 8 heads, (128,128) 153.5 / 144.4 us; 115200, 4 heads 1840 / 1725; 75600, 6
 // heads, (64,64) 3650 / 3510, 4 heads, (32,32) 4560 / 3700.  At d = 64 (each warpgroup has its own) on lists of 32
-// tiles and more: 32768 tokens, 16 heads, (256,256) 1230 / 1190; 8 heads, (32,32) 1218 / 1089; 23296 tokens, 2 heads, (256,256)
-// at 44 % 276 / 215.  The running maximum stays for half, which has no such range, and for short lists, where the second copy
+// tiles and more: 32768 tokens, 16 heads, (256,256) 1250 / 1203; 8 heads, (32,32), 12 % independent blocks 1343 / 1284; 23296 tokens,
+// 2 heads, (256,256) at 44 % 190 / 185.  The running maximum stays for half, which has no such range, and for short lists, where the second copy
 // of the loop costs more than it saves (d = 128, 32768 tokens, 8 heads, two tiles per item 74 -> 82 us; d = 64, 2048 tokens, 2
 // heads 16.5 -> 18.5, 10240 tokens, 8 heads, 9 tiles of runs 55 -> 63; 16384 tokens, 16 heads, (32,32), 15 tiles 244 -> 250);
 // at d = 64 also for tiles of two entries ((64,64) at 48 tiles 1360 -> 1440); and for lists that are short next to the time until
